@@ -24,6 +24,9 @@ SOURCES = ["capi.cpp", "setup.cpp", "passes_f32.cu", "passes_f64.cu", "passes_df
            "passes_f64_a.cu", "passes_f64_b.cu", "passes_f64_c.cu",
            "passes_df_1.cu", "passes_df_2.cu", "passes_df_3.cu", "passes_df_4.cu", "passes_df_5.cu",
            "passes_df_6.cu", "passes_df_7.cu", "passes_df_8.cu", "passes_df_9.cu",
+           "passes_any_f32_x.cu", "passes_any_f32_y.cu", "passes_any_f32_z.cu",
+           "passes_any_f64_x.cu", "passes_any_f64_y.cu", "passes_any_f64_z.cu",
+           "passes_any_df_x.cu", "passes_any_df_y.cu", "passes_any_df_z.cu",
            "noalloc.cu", "reduce.cu", "sample.cu", "selector.cu", "selftest.cu", "setup_device.cu", "debug.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

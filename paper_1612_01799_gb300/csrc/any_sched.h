@@ -1,0 +1,182 @@
+// Radix schedules and index arithmetic of the runtime-length forms (passes_any.cuh), shared by
+// host and device.
+#pragma once
+#include <algorithm>
+
+#ifdef __CUDACC__
+#define GSP_HD __host__ __device__
+#else
+#define GSP_HD
+#endif
+
+namespace gsp {
+
+// Radix schedule of a runtime-length transform (the runtime-length pass forms): length L in
+// nst stages of radices r[0..nst), r[0] even.  M[st] is the product of the later radices, P[st]
+// of the earlier ones.  Digit st of a value's slot has stride S[st] (S[nst - 1] = 1), which is
+// M[st], or with padding the next odd number from r[st + 1] S[st + 1] on; slots = r[0] S[0].
+// mulM and mulR are the reciprocals floor(2^32 / d) + 1 of M[st] and r[st], so that
+// e / d = umulhi(e, mul) exactly for e < 2^20.
+constexpr int kAnyMaxStages = 8;
+struct AnySched {
+    int L;
+    int nst;
+    int slots;
+    int r[kAnyMaxStages], M[kAnyMaxStages], P[kAnyMaxStages], S[kAnyMaxStages];
+    unsigned mulM[kAnyMaxStages], mulR[kAnyMaxStages];
+};
+// The schedule of the even 5-smooth length L >= 4 with radices 2, 3, 4, 5, 6, 8, 9, 10 and 12
+// up to max_radix: at least two and otherwise the fewest stages, among those the smallest sum
+// of the radices; the largest even radix first (its stage skips the padding's zeros), the
+// smallest one, at most max_last, last.  nst = 0 if there is none.
+inline AnySched any_sched(int L, int max_radix, int max_last, bool pad) {
+    static const int kRadix[] = {12, 10, 9, 8, 6, 5, 4, 3, 2};
+    // Depth-first over non-increasing radices.
+    int cur[kAnyMaxStages], best[kAnyMaxStages], nbest = 0, sbest = 0;
+    auto search = [&](auto &&self, int m, int n, int from) -> void {
+        if (m == 1) {
+            if (n < 2 || (nbest && n > nbest)) return;
+            int even = -1, sum = 0;  // the largest even radix goes first
+            for (int i = 0; i < n; ++i) {
+                if (even < 0 && cur[i] % 2 == 0) even = i;
+                sum += cur[i];
+            }
+            if (even >= 0 && cur[even == n - 1 ? n - 2 : n - 1] <= max_last && (n < nbest || !nbest || sum < sbest)) {
+                nbest = n;
+                sbest = sum;
+                std::copy(cur, cur + n, best);
+            }
+            return;
+        }
+        if (n == kAnyMaxStages) return;
+        for (int i = from; i < 9; ++i)
+            if (kRadix[i] <= max_radix && m % kRadix[i] == 0) {
+                cur[n] = kRadix[i];
+                self(self, m / kRadix[i], n + 1, i);
+            }
+    };
+    search(search, L, 0, 0);
+    AnySched s{};
+    s.L = L;
+    s.nst = nbest;
+    for (int i = 0; i < nbest; ++i)
+        if (best[i] % 2 == 0) {
+            std::rotate(best, best + i, best + i + 1);
+            break;
+        }
+    for (int st = nbest - 1; st >= 0; --st) {
+        const bool last = st == nbest - 1;
+        s.r[st] = best[st];
+        s.M[st] = last ? 1 : s.M[st + 1] * s.r[st + 1];
+        s.S[st] = last ? 1 : s.r[st + 1] * s.S[st + 1];
+        if (pad && !last) s.S[st] |= 1;
+        s.mulM[st] = s.M[st] == 1 ? 0u : (unsigned)((1ull << 32) / (unsigned)s.M[st] + 1);
+        s.mulR[st] = (unsigned)((1ull << 32) / (unsigned)s.r[st] + 1);
+    }
+    for (int st = 0; st < nbest; ++st) s.P[st] = st == 0 ? 1 : s.P[st - 1] * s.r[st - 1];
+    s.slots = nbest ? s.r[0] * s.S[0] : 0;
+    return s;
+}
+
+// Largest radix, per arithmetic.  Double-float stops at 10: its butterflies are ten times longer
+// in instructions, and the stages of a kernel should stay within the instruction cache.
+constexpr int any_max_radix(bool df) { return df ? 10 : 12; }
+// Warps of an SM that their registers admit (80 in FP32, 128 otherwise).
+constexpr int any_max_warps(bool f32) { return f32 ? 24 : 16; }
+// Largest last radix of the x passes, whose last stage holds two butterflies.
+constexpr int kAnyRowsLast = 8;
+
+// Tile of a runtime-length pass: its schedule, 2^lg 16-byte groups, slots pitch groups apart,
+// threads, bytes of shared memory.
+struct AnyTile {
+    AnySched s;
+    int lg, pitch, threads, smem;
+};
+constexpr int kAnyThreads = 256;  // threads the kernels are compiled for
+
+// rows: an x pass (one more group of pitch, odd slot strides: conflict-free for neighbouring
+// groups and for neighbouring samples alike); else a column pass (eight groups fill a 128-byte
+// row, which a quarter-warp reads whole; four groups take odd strides instead).  Eight groups
+// while three CTAs fit an SM, else four (FP32, solves: N = 240 590 us with eight, 605 us with
+// four; N = 162 243 and 275 us; N = 400, where only two CTAs of eight fit, 2.86 and 2.83 ms).
+// Threads: the multiple of 32 with the most threads of
+// an SM at work, counting the share of thread slots that the rounds over the butterflies of
+// each stage fill and the CTAs that shared memory and max_warps (by registers) admit.
+inline AnyTile any_tile(int L, int max_radix, int max_warps, bool rows) {
+    AnyTile t{};
+    const int max_last = rows ? kAnyRowsLast : max_radix;
+    const AnySched wide = any_sched(L, max_radix, max_last, rows);
+    t.lg = wide.slots * (rows ? 9 : 8) * 16 <= 70 * 1024 ? 3 : 2;
+    t.s = t.lg == 3 ? wide : any_sched(L, max_radix, max_last, true);
+    t.pitch = (1 << t.lg) + (rows ? 1 : 0);
+    t.smem = t.s.slots * t.pitch * 16;
+    double best = 0.0;
+    for (int n = kAnyThreads; n >= 64; n -= 32) {
+        double slots = 0.0, used = 0.0;
+        for (int st = 0; st < t.s.nst; ++st) {
+            const int items = (L / t.s.r[st]) << t.lg;
+            slots += (double)((items + n - 1) / n) * n * t.s.r[st];
+            used += (double)items * t.s.r[st];
+        }
+        const int ctas = std::min(232448 / (t.smem + L * 16 + 1024), max_warps * 32 / n);
+        const double score = used / slots * ctas * n;
+        if (score > best * 1.02 || n == kAnyThreads) {
+            best = score;
+            t.threads = n;
+        }
+    }
+    return t;
+}
+
+// e / d by its reciprocal mul.
+GSP_HD inline int rdiv(int e, unsigned mul) { return (int)(((unsigned long long)(unsigned)e * mul) >> 32); }
+
+// Butterfly b < L / R of stage st: its first slot, the time index lo of its later digits and
+// the frequency of its earlier digits.
+struct AnyBfly {
+    int slot, lo, freq;
+};
+GSP_HD inline int any_lo_slot(const AnySched &s, int st, int lo) {
+    int a = 0;
+    for (int u = st + 1; u < s.nst - 1; ++u) {
+        const int q = rdiv(lo, s.mulM[u]);
+        a += q * s.S[u];
+        lo -= q * s.M[u];
+    }
+    return a + lo;
+}
+GSP_HD inline AnyBfly any_bfly(const AnySched &s, int st, int b) {
+    AnyBfly f;
+    int hi = b;
+    f.lo = 0;
+    f.slot = 0;
+    f.freq = 0;
+    if (st < s.nst - 1) {
+        hi = rdiv(b, s.mulM[st]);
+        f.lo = b - hi * s.M[st];
+        f.slot = any_lo_slot(s, st, f.lo);
+    }
+    if (st > 0) {
+        for (int u = st - 1; u >= 1; --u) {
+            const int q = rdiv(hi, s.mulR[u]), d = hi - q * s.r[u];
+            f.slot += d * s.S[u];
+            f.freq += d * s.P[u];
+            hi = q;
+        }
+        f.slot += hi * s.S[0];
+        f.freq += hi;
+    }
+    return f;
+}
+// Slot of frequency k.
+GSP_HD inline int any_freq_slot(const AnySched &s, int k) {
+    int a = 0;
+    for (int u = 0; u < s.nst - 1; ++u) {
+        const int q = rdiv(k, s.mulR[u]);
+        a += (k - q * s.r[u]) * s.S[u];
+        k = q;
+    }
+    return a + k;
+}
+
+}  // namespace gsp

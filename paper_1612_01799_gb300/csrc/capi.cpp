@@ -66,30 +66,10 @@ bool n_any(int N) {
     return N == 1;
 }
 
-AnySched any_sched(int L) {
-    AnySched s{};
-    s.L = L;
-    int m = L, n = 0;
-    for (int f : {5, 3})
-        while (m % f == 0 && n < kAnyMaxStages) {
-            s.r[n++] = f;
-            m /= f;
-        }
-    while (m % 4 == 0 && n < kAnyMaxStages) {
-        s.r[n++] = 4;
-        m /= 4;
-    }
-    if (m == 2 && n < kAnyMaxStages) {
-        s.r[n++] = 2;
-        m = 1;
-    }
-    s.nst = m == 1 ? n : 0;
-    unsigned long long ns = 1;
-    for (int st = 0; st < s.nst; ++st) {
-        s.mul[st] = ns == 1 ? 0u : (unsigned)((1ull << 32) / ns + 1);
-        ns *= (unsigned long long)s.r[st];
-    }
-    return s;
+void any_plan_tiles(DevicePlan &p) {
+    for (int df = 0; df < 2; ++df)
+        for (int q = 0; q < 3; ++q)
+            p.any_tile[df][q] = any_tile(q == 0 ? p.n3[0] : 2 * p.n3[q], any_max_radix(df != 0), any_max_warps(p.dtype == POISSON_F32), q == 0);
 }
 
 cudaError_t launch_solve(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int count,
@@ -543,6 +523,7 @@ static int plan_create_impl(poisson_plan *out, const int *n3, double L, const do
     p->dp.dtype = dtype;
     p->dp.any = any ? 1 : 0;
     for (int q = 0; q < 3; ++q) p->dp.n3[q] = n3[q];
+    gsp::any_plan_tiles(p->dp);
     p->dp.Px = gsp::pitch_for(nx);
     p->dp.Ps = gsp::sym_pitch_for(nx);
     const size_t cx = 2 * p->elem;

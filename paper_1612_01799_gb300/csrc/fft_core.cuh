@@ -156,6 +156,33 @@ __device__ __forceinline__ CDF cscale(CDF a, DF s) { return {a.re * s, a.im * s}
 // Lane-wise real scale (CV: one factor per column).
 __device__ __forceinline__ CV cscale2(CV a, float2 s) { return {f2mul(a.re, s), f2mul(a.im, s)}; }
 
+// a + x s and x sx + y sy (real s): fused multiply-adds where the arithmetic has them, in
+// double-float the one-pass sum of two products.
+__device__ __forceinline__ CF cfma(CF a, CF x, float s) { return {fmaf(x.re, s, a.re), fmaf(x.im, s, a.im)}; }
+__device__ __forceinline__ CD cfma(CD a, CD x, double s) { return {fma(x.re, s, a.re), fma(x.im, s, a.im)}; }
+__device__ __forceinline__ CV cfma(CV a, CV x, float s) {
+    return {f2fma(x.re, f2(s, s), a.re), f2fma(x.im, f2(s, s), a.im)};
+}
+__device__ __forceinline__ CDF cfma(CDF a, CDF x, DF s) { return {a.re + x.re * s, a.im + x.im * s}; }
+template <typename C, typename R> __device__ __forceinline__ C cdot2(C x, R sx, C y, R sy) {
+    return cfma(cscale(x, sx), y, sy);
+}
+__device__ __forceinline__ CDF cdot2(CDF x, DF sx, CDF y, DF sy) {
+    return {df_sum_prod(x.re, sx, y.re, sy), df_sum_prod(x.im, sx, y.im, sy)};
+}
+// a + x sx + y sy
+template <typename C, typename R> __device__ __forceinline__ C cacc2(C a, C x, R sx, C y, R sy) {
+    return cfma(cfma(a, y, sy), x, sx);
+}
+__device__ __forceinline__ CDF cacc2(CDF a, CDF x, DF sx, CDF y, DF sy) { return cadd(a, cdot2(x, sx, y, sy)); }
+// a - x / 2 (in double-float the halves are exact, no product)
+template <typename C> __device__ __forceinline__ C csub_half(C a, C x) {
+    return cfma(a, x, (typename CxReal<C>::T)-0.5);
+}
+__device__ __forceinline__ CDF csub_half(CDF a, CDF x) {
+    return {a.re + DF(-0.5f * x.re.hi, -0.5f * x.re.lo), a.im + DF(-0.5f * x.im.hi, -0.5f * x.im.lo)};
+}
+
 // a + i D b (D = +1 or -1): the product with +-i never materialises.
 template <int D> __device__ __forceinline__ CF add_rot(CF a, CF b) {
     return D > 0 ? CF{a.re - b.im, a.im + b.re} : CF{a.re + b.im, a.im - b.re};
@@ -171,6 +198,19 @@ template <int D> __device__ __forceinline__ CDF add_rot(CDF a, CDF b) {
 }
 // a - i D b
 template <int D, typename C> __device__ __forceinline__ C sub_rot(C a, C b) { return add_rot<-D>(a, b); }
+
+// a = m + i D h d and b = m - i D h d (real h): fused into the sums, or in double-float with
+// the product taken once.
+template <int D, typename C, typename R> __device__ __forceinline__ void rot_pair(C m, C d, R h, C &a, C &b) {
+    const R p = D > 0 ? h : -h;
+    a = {cfma(C{m.re, m.im}, C{d.im, d.re}, -p).re, cfma(C{m.re, m.im}, C{d.im, d.re}, p).im};
+    b = {cfma(C{m.re, m.im}, C{d.im, d.re}, p).re, cfma(C{m.re, m.im}, C{d.im, d.re}, -p).im};
+}
+template <int D> __device__ __forceinline__ void rot_pair(CDF m, CDF d, DF h, CDF &a, CDF &b) {
+    const CDF t = cscale(d, h);
+    a = add_rot<D>(m, t);
+    b = sub_rot<D>(m, t);
+}
 
 // Product with the constant exp(D 2 pi i m / R), given by its forward value (cr, ci) =
 // exp(-2 pi i m / R): D < 0 multiplies by (cr, ci), D > 0 by (cr, -ci).
@@ -239,12 +279,10 @@ template <int D, typename C> __device__ __forceinline__ void dft4(C &a0, C &a1, 
 template <int D, typename C> __device__ __forceinline__ void dft3(C &a0, C &a1, C &a2) {
     using R = typename CxReal<C>::T;
     const R h = (R)0.86602540378443864676;  // sqrt(3)/2
-    C s = cadd(a1, a2);
-    C d = cscale(csub(a1, a2), h);
-    C m = csub(a0, cscale(s, (R)0.5));
+    const C s = cadd(a1, a2), d = csub(a1, a2);
+    const C m = csub_half(a0, s);
     a0 = cadd(a0, s);
-    a1 = add_rot<D>(m, d);
-    a2 = sub_rot<D>(m, d);
+    rot_pair<D>(m, d, h, a1, a2);
 }
 
 template <int D, typename C> __device__ __forceinline__ void dft5(C &a0, C &a1, C &a2, C &a3, C &a4) {
@@ -254,10 +292,8 @@ template <int D, typename C> __device__ __forceinline__ void dft5(C &a0, C &a1, 
     const R s1 = (R)0.95105651629515357212;   // sin(2 pi / 5)
     const R s2 = (R)0.58778525229247312917;   // sin(4 pi / 5)
     C b1 = cadd(a1, a4), b2 = cadd(a2, a3), d1 = csub(a1, a4), d2 = csub(a2, a3);
-    C p1 = cadd(a0, cadd(cscale(b1, c1), cscale(b2, c2)));
-    C p2 = cadd(a0, cadd(cscale(b1, c2), cscale(b2, c1)));
-    C q1 = cadd(cscale(d1, s1), cscale(d2, s2));
-    C q2 = csub(cscale(d1, s2), cscale(d2, s1));
+    const C p1 = cacc2(a0, b1, c1, b2, c2), p2 = cacc2(a0, b1, c2, b2, c1);
+    const C q1 = cdot2(d1, s1, d2, s2), q2 = cdot2(d1, s2, d2, -s1);
     a0 = cadd(a0, cadd(b1, b2));
     a1 = add_rot<D>(p1, q1);
     a4 = sub_rot<D>(p1, q1);
@@ -297,17 +333,53 @@ template <int R, int D, typename C> __device__ __forceinline__ void dft(C *a) {
         dft4<D>(a[0], a[1], a[2], a[3]);
     } else if constexpr (R == 5) {
         dft5<D>(a[0], a[1], a[2], a[3], a[4]);
-    } else if constexpr (R == 6) {
-        C e[3] = {a[0], a[2], a[4]}, o[3] = {a[1], a[3], a[5]};
-        dft3<D>(e[0], e[1], e[2]);
-        dft3<D>(o[0], o[1], o[2]);
-        const Re cs[3] = {(Re)1, (Re)0.5, (Re)-0.5};
-        const Re sn[3] = {(Re)0, (Re)-0.86602540378443864676, (Re)-0.86602540378443864676};
+    } else if constexpr (R == 6 || R == 10 || R == 12) {
+        // Good-Thomas: R = A B with A, B coprime, input (B i + A j) mod R, output k with
+        // k = p mod A and k = q mod B; no twiddles between the two DFTs.
+        constexpr int B = R == 10 ? 5 : 3, A = R / B;
+        C t[A][B];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const C t = k == 0 ? o[0] : cmulk<D>(o[k], cs[k], sn[k]);
-            a[k] = cadd(e[k], t);
-            a[k + 3] = csub(e[k], t);
+        for (int i = 0; i < A; ++i) {
+#pragma unroll
+            for (int j = 0; j < B; ++j) t[i][j] = a[(B * i + A * j) % R];
+            dft<B, D>(t[i]);
+        }
+#pragma unroll
+        for (int q = 0; q < B; ++q) {
+            C u[A];
+#pragma unroll
+            for (int i = 0; i < A; ++i) u[i] = t[i][q];
+            dft<A, D>(u);
+#pragma unroll
+            for (int p = 0; p < A; ++p) {
+                // the k < R with k = p mod A, k = q mod B
+                constexpr int eA = R == 6 ? 3 : R == 10 ? 5 : 9;  // 1 mod A, 0 mod B
+                constexpr int eB = R == 6 ? 4 : R == 10 ? 6 : 4;  // 0 mod A, 1 mod B
+                a[(eA * p + eB * q) % R] = u[p];
+            }
+        }
+    } else if constexpr (R == 9) {
+        C t[3][3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+#pragma unroll
+            for (int j = 0; j < 3; ++j) t[i][j] = a[i + 3 * j];
+            dft<3, D>(t[i]);
+        }
+        // W_9, W_9^2, W_9^4
+        const Re c1 = (Re)0.76604444311897803520, s1 = (Re)-0.64278760968653932632;
+        const Re c2 = (Re)0.17364817766693034885, s2 = (Re)-0.98480775301220805937;
+        const Re c4 = (Re)-0.93969262078590838405, s4 = (Re)-0.34202014332566873304;
+        t[1][1] = cmulk<D>(t[1][1], c1, s1);
+        t[1][2] = cmulk<D>(t[1][2], c2, s2);
+        t[2][1] = cmulk<D>(t[2][1], c2, s2);
+        t[2][2] = cmulk<D>(t[2][2], c4, s4);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            dft3<D>(t[0][j], t[1][j], t[2][j]);
+            a[j] = t[0][j];
+            a[j + 3] = t[1][j];
+            a[j + 6] = t[2][j];
         }
     } else if constexpr (R == 8) {
         C e[4] = {a[0], a[2], a[4], a[6]}, o[4] = {a[1], a[3], a[5], a[7]};

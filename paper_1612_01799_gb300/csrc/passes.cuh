@@ -195,7 +195,6 @@ template <typename Real> using AnyTw = Cx2<Real>;
 #include "passes_tma.cuh"
 #include "passes_zwarp.cuh"
 #include "passes_xy.cuh"
-#include "passes_any.cuh"
 namespace gsp {
 
 // ---- K1: x forward (real, zero-padded to 2N) -------------------------------------------
@@ -934,83 +933,14 @@ cudaError_t encode_n(DevicePlan &p) {
                                               cudaStream_t, bool);                                         \
     EXT template cudaError_t encode_n<Real, n>(DevicePlan &);
 
-// ---- runtime-length forms: launchers ----------------------------------------------------------
-// Tiles sized so that the ping-pong pair of one CTA stays within about 64 KB of shared memory.
-template <typename Real> int any_tile(int L, int cap, int extra = 0) {
-    const int bytes = 2 * L * (int)sizeof(typename Types<Real>::CS);
-    int t = cap;
-    while (t > 1 && (t + extra) * bytes > 65536) t /= 2;
-    return t;
-}
-inline int ilog2(int t) {
-    int l = 0;
-    while ((1 << (l + 1)) <= t) ++l;
-    return l;
-}
-
+// ---- runtime-length forms: launchers (instantiated in passes_any_*.cu) ---------------------------
 template <typename Real>
 cudaError_t any_x(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int B, cudaStream_t s, bool fwd,
-                  int rows = 0, void *w1 = nullptr) {
-    const int nx = p.n3[0], ny = p.n3[1], nz = p.n3[2];
-    const AnySched sc = any_sched(nx);
-    const int rows_b = ny * nz, nrows = rows ? rows : B * rows_b;
-    const int TR = any_tile<Real>(nx, 16, 1);  // pitch TR + 1
-    const size_t smem = (size_t)2 * nx * (TR + 1) * sizeof(typename Types<Real>::CS);
-    const AnyTw<Real> *tw = static_cast<const AnyTw<Real> *>(p.tw3[0]);
-    Cx2<Real> *ws = static_cast<Cx2<Real> *>(w1 ? w1 : p.w1);
-    const int grid = (nrows + TR - 1) / TR;
-    if (fwd) {
-        GSP_CHECK(set_smem(k_any_x_fwd<Real>, smem));
-        GSP_CHECK(launch_pdl(k_any_x_fwd<Real>, grid, 256, smem, s, rho, ws, tw, sc, rows_b, nrows, p.Px, ilog2(TR)));
-    } else {
-        GSP_CHECK(set_smem(k_any_x_inv<Real>, smem));
-        GSP_CHECK(launch_pdl(k_any_x_inv<Real>, grid, 256, smem, s, static_cast<const Cx2<Real> *>(ws), u, tw, sc,
-                             rows_b, nrows, p.Px, ilog2(TR)));
-    }
-    return cudaGetLastError();
-}
-
+                  int rows = 0, void *w1 = nullptr);
 template <typename Real>
-cudaError_t any_y(const DevicePlan &p, int B, cudaStream_t s, bool fwd, int z0 = 0, int nzs = 0) {
-    const int nx = p.n3[0], ny = p.n3[1], nz = p.n3[2], L = 2 * ny;
-    const AnySched sc = any_sched(L);
-    const int TC = any_tile<Real>(L, 16), ncols = nx + 1, ntx = (ncols + TC - 1) / TC;
-    const int planes = nzs ? nzs : B * nz;
-    const size_t smem = (size_t)2 * L * TC * sizeof(typename Types<Real>::CS);
-    const AnyTw<Real> *tw = static_cast<const AnyTw<Real> *>(p.tw3[1]);
-    const long long Px = p.Px, w1p = (long long)ny * Px, w2p = (long long)L * Px;
-    const Cx2<Real> *w1 = static_cast<const Cx2<Real> *>(p.w1), *w3 = static_cast<const Cx2<Real> *>(p.w3);
-    Cx2<Real> *w1o = static_cast<Cx2<Real> *>(p.w1), *w2 = static_cast<Cx2<Real> *>(p.w2);
-    if (fwd) {
-        GSP_CHECK(set_smem(k_any_col<Real, true>, smem));
-        GSP_CHECK(launch_pdl(k_any_col<Real, true>, ntx * planes, 256, smem, s, w1 + z0 * w1p, w2 + z0 * w2p, tw, sc,
-                             ncols, ntx, ilog2(TC), Px, w1p, Px, w2p));
-    } else {
-        GSP_CHECK(set_smem(k_any_col<Real, false>, smem));
-        GSP_CHECK(launch_pdl(k_any_col<Real, false>, ntx * planes, 256, smem, s, w3 + z0 * w2p, w1o + z0 * w1p, tw, sc,
-                             ncols, ntx, ilog2(TC), Px, w2p, Px, w1p));
-    }
-    return cudaGetLastError();
-}
-
-// The z pass of lines ky0 <= ky < ky0 + nky (nky = 0: all 2 ny lines).  Runs on the tables of
-// any plan: the compiled-length plans' symbol octant has the same layout as the box table
-// and their twiddles W_{2N} are axis z's table.
+cudaError_t any_y(const DevicePlan &p, int B, cudaStream_t s, bool fwd, int z0 = 0, int nzs = 0);
 template <typename Real>
-cudaError_t any_z(const DevicePlan &p, int B, cudaStream_t s, double *tail, int ky0 = 0, int nky = 0) {
-    const int nx = p.n3[0], ny = p.n3[1], nz = p.n3[2], L = 2 * nz;
-    if (nky == 0) nky = 2 * ny;
-    const AnySched sc = any_sched(L);
-    const int TC = any_tile<Real>(L, 16), ncols = nx + 1, ntx = (ncols + TC - 1) / TC;
-    const size_t smem = (size_t)2 * L * TC * sizeof(typename Types<Real>::CS);
-    const AnyTw<Real> *tw = static_cast<const AnyTw<Real> *>(p.any ? p.tw3[2] : p.tw);
-    const int grid = ntx * nky * B;
-    auto k = tail ? k_any_z<Real, true> : k_any_z<Real, false>;
-    GSP_CHECK(set_smem(k, smem));
-    GSP_CHECK(launch_pdl(k, grid, 256, smem, s, static_cast<const Cx2<Real> *>(p.w2), static_cast<Cx2<Real> *>(p.w3),
-                         static_cast<const Real *>(p.sym), tw, sc, nx, ny, ntx, ilog2(TC), p.Px, p.Ps, tail, ky0, nky));
-    return cudaGetLastError();
-}
+cudaError_t any_z(const DevicePlan &p, int B, cudaStream_t s, double *tail, int ky0 = 0, int nky = 0);
 
 template <typename Real>
 cudaError_t solve_any(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int B, cudaStream_t s,

@@ -5,6 +5,8 @@
 
 #include <cstddef>
 
+#include "any_sched.h"
+
 namespace gsp {
 
 // Densities one grouped launch sequence can carry (kernel-parameter arrays of pointers).
@@ -15,20 +17,6 @@ struct PtrArray {
     const void *p[kMaxBatch];
 };
 
-// Radix schedule of a runtime-length transform (the runtime-length pass forms): length L,
-// nst stages of radices r[0..nst) in {2, 3, 4, 5}, first to last; mul[st] the reciprocal
-// floor(2^32 / Ns) + 1 of the product Ns of the earlier radices (0 for the first stage), so
-// that j / Ns = umulhi(j, mul[st]) exactly for j < 4096.
-constexpr int kAnyMaxStages = 16;
-struct AnySched {
-    int L;
-    int nst;
-    int r[kAnyMaxStages];
-    unsigned mul[kAnyMaxStages];
-};
-// The schedule of length L (fives, threes, fours, then a two), or nst = 0 if L has a prime
-// factor above 5.
-AnySched any_sched(int L);
 // N of the runtime-length forms: even, 4 <= N <= 1024, no prime factor above 5.
 bool n_any(int N);
 
@@ -59,6 +47,8 @@ struct DevicePlan {
     int any = 0;
     int n3[3] = {0, 0, 0};
     void *tw3[3] = {nullptr, nullptr, nullptr};
+    // Tiles of the runtime-length passes along x, y and z, per arithmetic (any_plan_tiles).
+    AnyTile any_tile[2][3];
     int Px = 0;
     int Ps = 0;
     void *sym = nullptr;
@@ -101,6 +91,10 @@ inline int pitch_for(int N) { return ((N + 1 + 15) / 16) * 16; }
 inline int sym_pitch_for(int N) { return ((N + 1 + 3) / 4) * 4; }
 
 bool n_supported(int N);
+
+// Fill p.any_tile for p's lengths (any plan: the slab z pass runs on the compiled-length
+// plans too).
+void any_plan_tiles(DevicePlan &p);
 
 // Record a failed CUDA call for poisson_last_cuda_error() (per host thread).
 void note_cuda_error(cudaError_t e);

@@ -1,0 +1,63 @@
+// Test shim: the runtime-length forms' schedules and index arithmetic (csrc/any_sched.h) on the
+// CPU.  Runs the in-place stages of one transform with plain DFTs in place of the radix
+// butterflies.
+#include <cmath>
+#include <complex>
+#include <vector>
+
+#include "any_sched.h"
+
+using cd = std::complex<double>;
+
+// The transform of x (L values) into X in natural order.  Returns 0, or the number of the rule
+// that failed: 1 schedule, 2 slot out of range or taken twice in a stage, 3 frequency of a
+// butterfly's outputs, 4 slot of a frequency, 5 a radix above max_radix, or
+// the last one above max_last.
+extern "C" int shim_any_transform(int L, int max_radix, int max_last, int pad, const double *x, double *X) {
+    const gsp::AnySched s = gsp::any_sched(L, max_radix, max_last, pad != 0);
+    int prod = 1;
+    for (int st = 0; st < s.nst; ++st) {
+        if (s.r[st] > max_radix || (st + 1 == s.nst && s.r[st] > max_last)) return 5;
+        prod *= s.r[st];
+    }
+    if (s.nst < 2 || prod != L || s.r[0] % 2 || s.slots < L) return 1;
+    const double tau = 2.0 * std::acos(-1.0);
+    std::vector<cd> v(s.slots);
+    for (int j = 0; j < s.M[0]; ++j)
+        for (int r = 0; r < s.r[0]; ++r) {
+            const int n = j + r * s.M[0];
+            v[gsp::any_lo_slot(s, 0, j) + r * s.S[0]] = cd(x[2 * n], x[2 * n + 1]);
+        }
+    for (int st = 0; st < s.nst; ++st) {
+        const int R = s.r[st], nb = s.P[st] * s.M[st];
+        std::vector<char> hit(s.slots, 0);
+        for (int b = 0; b < nb; ++b) {
+            const gsp::AnyBfly f = gsp::any_bfly(s, st, b);
+            std::vector<cd> in(R), out(R);
+            for (int r = 0; r < R; ++r) {
+                const int a = f.slot + r * s.S[st];
+                if (a < 0 || a >= s.slots || hit[a]) return 2;
+                hit[a] = 1;
+                in[r] = v[a];
+            }
+            for (int k = 0; k < R; ++k) {
+                cd acc = 0;
+                for (int r = 0; r < R; ++r) acc += in[r] * std::polar(1.0, -tau * (r * k % R) / R);
+                const int e = st + 1 < s.nst ? f.lo * s.P[st] * k : 0;
+                if (e >= L) return 3;
+                out[k] = acc * std::polar(1.0, -tau * e / L);
+            }
+            for (int r = 0; r < R; ++r) {
+                v[f.slot + r * s.S[st]] = out[r];
+                if (st + 1 == s.nst && gsp::any_freq_slot(s, f.freq + r * nb) != f.slot + r * s.S[st]) return 3;
+            }
+        }
+    }
+    for (int k = 0; k < L; ++k) {
+        const int a = gsp::any_freq_slot(s, k);
+        if (a < 0 || a >= s.slots) return 4;
+        X[2 * k] = v[a].real();
+        X[2 * k + 1] = v[a].imag();
+    }
+    return 0;
+}
