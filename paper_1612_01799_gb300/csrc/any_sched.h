@@ -27,21 +27,27 @@ struct AnySched {
 };
 // The schedule of the even 5-smooth length L >= 4 with radices 2, 3, 4, 5, 6, 8, 9, 10 and 12
 // up to max_radix: at least two and otherwise the fewest stages, among those the smallest sum
-// of the radices; the largest even radix first (its stage skips the padding's zeros), the
-// smallest one, at most max_last, last.  nst = 0 if there is none.
+// of the radices.  First (its stage skips the padding's zeros) an 8, whose zero-skipping form
+// has the fewest products to round, or the largest even radix; last the smallest of the
+// others, at most max_last.  nst = 0 if there is none.
 inline AnySched any_sched(int L, int max_radix, int max_last, bool pad) {
     static const int kRadix[] = {12, 10, 9, 8, 6, 5, 4, 3, 2};
+    // Which of the n non-increasing radices goes first, or -1 if none can.
+    auto first_of = [&](const int *f, int n) {
+        const int i8 = (int)(std::find(f, f + n, 8) - f);
+        const int even = (int)(std::find_if(f, f + n, [](int v) { return v % 2 == 0; }) - f);
+        for (int i : {i8, even})
+            if (i < n && f[i == n - 1 ? n - 2 : n - 1] <= max_last) return i;
+        return -1;
+    };
     // Depth-first over non-increasing radices.
     int cur[kAnyMaxStages], best[kAnyMaxStages], nbest = 0, sbest = 0;
     auto search = [&](auto &&self, int m, int n, int from) -> void {
         if (m == 1) {
             if (n < 2 || (nbest && n > nbest)) return;
-            int even = -1, sum = 0;  // the largest even radix goes first
-            for (int i = 0; i < n; ++i) {
-                if (even < 0 && cur[i] % 2 == 0) even = i;
-                sum += cur[i];
-            }
-            if (even >= 0 && cur[even == n - 1 ? n - 2 : n - 1] <= max_last && (n < nbest || !nbest || sum < sbest)) {
+            int sum = 0;
+            for (int i = 0; i < n; ++i) sum += cur[i];
+            if (first_of(cur, n) >= 0 && (n < nbest || !nbest || sum < sbest)) {
                 nbest = n;
                 sbest = sum;
                 std::copy(cur, cur + n, best);
@@ -59,11 +65,10 @@ inline AnySched any_sched(int L, int max_radix, int max_last, bool pad) {
     AnySched s{};
     s.L = L;
     s.nst = nbest;
-    for (int i = 0; i < nbest; ++i)
-        if (best[i] % 2 == 0) {
-            std::rotate(best, best + i, best + i + 1);
-            break;
-        }
+    if (nbest) {
+        const int i = first_of(best, nbest);
+        std::rotate(best, best + i, best + i + 1);
+    }
     for (int st = nbest - 1; st >= 0; --st) {
         const bool last = st == nbest - 1;
         s.r[st] = best[st];

@@ -30,6 +30,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "debug.cuh"
 
@@ -146,13 +147,34 @@ __device__ __forceinline__ CD cadd(CD a, CD b) { return {a.re + b.re, a.im + b.i
 __device__ __forceinline__ CD csub(CD a, CD b) { return {a.re - b.re, a.im - b.im}; }
 __device__ __forceinline__ CV cadd(CV a, CV b) { return {f2add(a.re, b.re), f2add(a.im, b.im)}; }
 __device__ __forceinline__ CV csub(CV a, CV b) { return {f2sub(a.re, b.re), f2sub(a.im, b.im)}; }
-__device__ __forceinline__ CDF cadd(CDF a, CDF b) { return {a.re + b.re, a.im + b.im}; }
-__device__ __forceinline__ CDF csub(CDF a, CDF b) { return {a.re - b.re, a.im - b.im}; }
+// The two double-float sums of a complex sum in one: the real and the imaginary part take the
+// steps of DF's operator+ (the same roundings, the same result) side by side in packed FP32x2
+// instructions, five and six selects and compares in place of ten and six.  The FMA pipe takes
+// a packed instruction in two cycles, so what this saves is issue slots and code size: the
+// compiled-length z pass at N = 128 went from 141 to 136 us, the runtime-length one at
+// N = 162, whose stages compete for the instruction cache, from 480 to 428 us.
+__device__ __forceinline__ CDF cadd(CDF a, CDF b) {
+    const bool p = fabsf(b.re.hi) > fabsf(a.re.hi), q = fabsf(b.im.hi) > fabsf(a.im.hi);
+    const float2 x = f2(p ? b.re.hi : a.re.hi, q ? b.im.hi : a.im.hi);
+    const float2 y = f2(p ? a.re.hi : b.re.hi, q ? a.im.hi : b.im.hi);
+    const float2 s = f2add(x, y), e = f2sub(y, f2sub(s, x));
+    const float2 l = f2add(e, f2add(f2(a.re.lo, a.im.lo), f2(b.re.lo, b.im.lo)));
+    return {DF(s.x, l.x), DF(s.y, l.y)};
+}
+__device__ __forceinline__ CDF csub(CDF a, CDF b) { return cadd(a, CDF{-b.re, -b.im}); }
 
 __device__ __forceinline__ CF cscale(CF a, float s) { return {a.re * s, a.im * s}; }
 __device__ __forceinline__ CD cscale(CD a, double s) { return {a.re * s, a.im * s}; }
 __device__ __forceinline__ CV cscale(CV a, float s) { return {f2mul(a.re, f2(s, s)), f2mul(a.im, f2(s, s))}; }
-__device__ __forceinline__ CDF cscale(CDF a, DF s) { return {a.re * s, a.im * s}; }
+// Both parts of a complex double-float times a real, the steps of DF's operator* packed.
+__device__ __forceinline__ CDF cscale(CDF a, DF s) {
+    const float2 x = f2(a.re.hi, a.im.hi), H = f2(s.hi, s.hi), p = f2mul(x, H);
+    float2 e = f2fma(x, H, f2neg(p));
+    e = f2fma(x, f2(s.lo, s.lo), e);
+    e = f2fma(f2(a.re.lo, a.im.lo), H, e);
+    const float2 h = f2add(p, e), l = f2sub(e, f2sub(h, p));
+    return {DF(h.x, l.x), DF(h.y, l.y)};
+}
 // Lane-wise real scale (CV: one factor per column).
 __device__ __forceinline__ CV cscale2(CV a, float2 s) { return {f2mul(a.re, s), f2mul(a.im, s)}; }
 
@@ -167,14 +189,20 @@ __device__ __forceinline__ CDF cfma(CDF a, CDF x, DF s) { return {a.re + x.re * 
 template <typename C, typename R> __device__ __forceinline__ C cdot2(C x, R sx, C y, R sy) {
     return cfma(cscale(x, sx), y, sy);
 }
-__device__ __forceinline__ CDF cdot2(CDF x, DF sx, CDF y, DF sy) {
-    return {df_sum_prod(x.re, sx, y.re, sy), df_sum_prod(x.im, sx, y.im, sy)};
+__device__ __forceinline__ CDF cdot2(CDF x, DF sx, CDF y, DF sy) {  // df_sum_prod's steps, packed
+    const float2 a = f2(x.re.hi, x.im.hi), c = f2(y.re.hi, y.im.hi), A = f2(sx.hi, sx.hi), B = f2(sy.hi, sy.hi);
+    const float2 p1 = f2mul(a, A), p2 = f2mul(c, B);
+    const float2 e1 = f2fma(a, A, f2neg(p1)), e2 = f2fma(c, B, f2neg(p2));
+    const bool p = fabsf(p2.x) > fabsf(p1.x), q = fabsf(p2.y) > fabsf(p1.y);
+    const float2 u = f2(p ? p2.x : p1.x, q ? p2.y : p1.y), v = f2(p ? p1.x : p2.x, q ? p1.y : p2.y);
+    const float2 s = f2add(u, v);
+    float2 t = f2add(f2sub(v, f2sub(s, u)), f2add(e1, e2));
+    t = f2fma(a, f2(sx.lo, sx.lo), t);
+    t = f2fma(f2(x.re.lo, x.im.lo), A, t);
+    t = f2fma(c, f2(sy.lo, sy.lo), t);
+    t = f2fma(f2(y.re.lo, y.im.lo), B, t);
+    return {DF(s.x, t.x), DF(s.y, t.y)};
 }
-// a + x sx + y sy
-template <typename C, typename R> __device__ __forceinline__ C cacc2(C a, C x, R sx, C y, R sy) {
-    return cfma(cfma(a, y, sy), x, sx);
-}
-__device__ __forceinline__ CDF cacc2(CDF a, CDF x, DF sx, CDF y, DF sy) { return cadd(a, cdot2(x, sx, y, sy)); }
 // a - x / 2 (in double-float the halves are exact, no product)
 template <typename C> __device__ __forceinline__ C csub_half(C a, C x) {
     return cfma(a, x, (typename CxReal<C>::T)-0.5);
@@ -194,10 +222,14 @@ template <int D> __device__ __forceinline__ CV add_rot(CV a, CV b) {
     return D > 0 ? CV{f2sub(a.re, b.im), f2add(a.im, b.re)} : CV{f2add(a.re, b.im), f2sub(a.im, b.re)};
 }
 template <int D> __device__ __forceinline__ CDF add_rot(CDF a, CDF b) {
-    return D > 0 ? CDF{a.re - b.im, a.im + b.re} : CDF{a.re + b.im, a.im - b.re};
+    return D > 0 ? cadd(a, CDF{-b.im, b.re}) : cadd(a, CDF{b.im, -b.re});
 }
 // a - i D b
 template <int D, typename C> __device__ __forceinline__ C sub_rot(C a, C b) { return add_rot<-D>(a, b); }
+
+// -i a
+template <typename C> __device__ __forceinline__ C cmul_mi(C a) { return {a.im, -a.re}; }
+template <> __device__ __forceinline__ CV cmul_mi(CV a) { return {a.im, f2neg(a.re)}; }
 
 // a = m + i D h d and b = m - i D h d (real h): fused into the sums, or in double-float with
 // the product taken once.
@@ -230,6 +262,17 @@ template <int D> __device__ __forceinline__ CV cmulk(CV a, float cr, float ci) {
     const float s = D < 0 ? ci : -ci;
     const float2 R = f2(cr, cr), S = f2(s, s), NS = f2(-s, -s);
     return {f2fma(a.im, NS, f2mul(a.re, R)), f2fma(a.re, S, f2mul(a.im, R))};
+}
+
+// a exp(D 2 pi i m / 8), m = 1 or 3, given h = sqrt(1/2).  Double-float takes the sum and the
+// difference of the parts and scales both by h, packed: 19 instructions where the general
+// product takes 32.
+template <int D, int M, typename C, typename R> __device__ __forceinline__ C cmul_w8(C a, R h) {
+    return cmulk<D>(a, M == 1 ? h : -h, -h);
+}
+template <int D, int M> __device__ __forceinline__ CDF cmul_w8(CDF a, DF h) {
+    // m = 1: h (re - D im, im + D re); m = 3: that times i D: h (-re - D im, D re - im)
+    return cscale(M == 1 ? add_rot<D>(a, a) : add_rot<D>(CDF{-a.re, -a.im}, a), h);
 }
 
 // Twiddle tables hold exp(-2 pi i e / TL): float2 / double2 (re, im) for CF / CD, and the
@@ -292,9 +335,19 @@ template <int D, typename C> __device__ __forceinline__ void dft5(C &a0, C &a1, 
     const R s1 = (R)0.95105651629515357212;   // sin(2 pi / 5)
     const R s2 = (R)0.58778525229247312917;   // sin(4 pi / 5)
     C b1 = cadd(a1, a4), b2 = cadd(a2, a3), d1 = csub(a1, a4), d2 = csub(a2, a3);
-    const C p1 = cacc2(a0, b1, c1, b2, c2), p2 = cacc2(a0, b1, c2, b2, c1);
+    C p1, p2, t = cadd(b1, b2);
+    if constexpr (std::is_same<C, CDF>::value) {
+        // c1 and c2 are -1/4 +- sqrt(5)/4: one product in place of four
+        const C m = cadd(a0, C{R(-0.25f * t.re.hi, -0.25f * t.re.lo), R(-0.25f * t.im.hi, -0.25f * t.im.lo)});
+        const C k = cscale(csub(b1, b2), (R)0.55901699437494742410);
+        p1 = cadd(m, k);
+        p2 = csub(m, k);
+    } else {
+        p1 = cadd(a0, cdot2(b1, c1, b2, c2));
+        p2 = cadd(a0, cdot2(b1, c2, b2, c1));
+    }
     const C q1 = cdot2(d1, s1, d2, s2), q2 = cdot2(d1, s2, d2, -s1);
-    a0 = cadd(a0, cadd(b1, b2));
+    a0 = cadd(a0, t);
     a1 = add_rot<D>(p1, q1);
     a4 = sub_rot<D>(p1, q1);
     a2 = add_rot<D>(p2, q2);
@@ -386,8 +439,15 @@ template <int R, int D, typename C> __device__ __forceinline__ void dft(C *a) {
         dft4<D>(e[0], e[1], e[2], e[3]);
         dft4<D>(o[0], o[1], o[2], o[3]);
         const Re r = (Re)0.70710678118654752440;
-        const Re cs[4] = {(Re)1, r, (Re)0, -r}, sn[4] = {(Re)0, -r, (Re)-1, -r};
-        combine2<D, 4>(e, o, a, cs, sn);
+        const C t1 = cmul_w8<D, 1>(o[1], r), t3 = cmul_w8<D, 3>(o[3], r);
+        a[0] = cadd(e[0], o[0]);
+        a[4] = csub(e[0], o[0]);
+        a[1] = cadd(e[1], t1);
+        a[5] = csub(e[1], t1);
+        a[2] = add_rot<D>(e[2], o[2]);
+        a[6] = sub_rot<D>(e[2], o[2]);
+        a[3] = cadd(e[3], t3);
+        a[7] = csub(e[3], t3);
     } else if constexpr (R == 16) {
         C e[8], o[8];
 #pragma unroll
@@ -404,6 +464,30 @@ template <int R, int D, typename C> __device__ __forceinline__ void dft(C *a) {
         combine2<D, 8>(e, o, a, cs, sn);
     } else {
         static_assert(R == 0, "unsupported radix");
+    }
+}
+
+// The length-R DFT (R = 4 or 8, forward) of a[0 .. R/2 - 1], the rest of a taken as zero: the DFTs
+// of half the length of the values (even outputs) and of the values times W_R^r (odd ones).
+template <int R, typename C> __device__ __forceinline__ void dft_zero_half(C *a) {
+    static_assert(R == 4 || R == 8, "a rotation and W_8 only");
+    constexpr int H = R / 2;
+    C e[H], o[H];
+#pragma unroll
+    for (int r = 0; r < H; ++r) e[r] = a[r];
+    o[0] = a[0];
+    o[H / 2] = cmul_mi(a[H / 2]);
+    if constexpr (R == 8) {
+        const typename CxReal<C>::T h = (typename CxReal<C>::T)0.70710678118654752440;
+        o[1] = cmul_w8<-1, 1>(a[1], h);
+        o[3] = cmul_w8<-1, 3>(a[3], h);
+    }
+    dft<H, -1>(e);
+    dft<H, -1>(o);
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+        a[2 * k] = e[k];
+        a[2 * k + 1] = o[k];
     }
 }
 
@@ -453,7 +537,10 @@ struct Stage {
         }
     }
 
-    // tw: table of exp(-2 pi i e / TL), TL = L * twstride.
+    // tw: table of exp(-2 pi i e / TL), TL = L * twstride.  ZERO: the upper half of a first
+    // stage's inputs is zero (radices 4 and 8 leave it out: a third of the sums of a radix-8
+    // butterfly, half of a radix-4 one).
+    template <bool ZERO>
     static __device__ __forceinline__ void compute(C *v, int q, const Tw *__restrict__ tw, int twstride) {
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
@@ -466,7 +553,8 @@ struct Stage {
                     v[b * R + r] = twmul<D>(v[b * R + r], __ldg(tw + e));
                 }
             }
-            dft<R, D>(&v[b * R]);
+            if constexpr (ZERO && NS == 1 && D < 0 && (R == 4 || R == 8)) dft_zero_half<R>(&v[b * R]);
+            else dft<R, D>(&v[b * R]);
         }
     }
 
@@ -488,7 +576,7 @@ struct Stage {
 // Options of a run of stages.
 struct RunOpt {
     bool from_regs;  // stage 0 starts from v as it is (no gather)
-    bool prune_in;
+    bool prune_in;   // the upper half of stage 0's inputs is zero
     bool to_regs;    // the last stage leaves its outputs in v (no scatter)
     bool prune_out;
     bool sync_last;  // barrier before the final scatter (it writes what the final gather read)
@@ -515,7 +603,7 @@ struct Stages<C, L, E, D, NS, Radices<R, Rs...>> {
     static __device__ __forceinline__ void run_with(C *v, int q, C *sm, const Tw *__restrict__ tw,
                                                     int twstride, Ld &&ld, St &&st, At &&at, Sync &&sync) {
         if constexpr (!O.from_regs) S::template gather<O.prune_in>(v, q, ld);
-        S::compute(v, q, tw, twstride);
+        S::template compute<O.prune_in>(v, q, tw, twstride);
         if constexpr (LAST) {
             if constexpr (!O.to_regs) {
                 if constexpr (O.sync_last) sync();

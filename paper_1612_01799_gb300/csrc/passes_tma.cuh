@@ -186,7 +186,7 @@ k_col_tma(const __grid_constant__ CUtensorMap tin, Cx2<Real> *__restrict__ out,
             issue(t + gridDim.x);
         }
         Cx2<Real> *dst = out + (long long)outer * out_outer + col;
-        constexpr RunOpt opt{true, false, false, !FWD, false};
+        constexpr RunOpt opt{true, FWD, false, !FWD, false};
         Stages<C, L, E, FWD ? -1 : 1, 1, Rs>::template run<opt>(
             v, q, g, xb, NG, tw, 1, [&](int) { return czero<C>(); },
             [&](int row, C x) {
@@ -282,7 +282,7 @@ k_z_symbol_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ 
             fence_proxy_async();
             issue_in(t + gridDim.x);
         }
-        constexpr RunOpt fwd{true, false, true, false, false};
+        constexpr RunOpt fwd{true, true, true, false, false};
         Stages<C, L, E, -1, 1, Rs>::template run<fwd>(
             v, q, g, xb, NG, tw, 1, [&](int) { return czero<C>(); }, [&](int, C) {});
         if constexpr (TAIL) {
