@@ -570,7 +570,7 @@ static int plan_create_impl(poisson_plan *out, const int *n3, double L, const do
     if ((e = cudaMemset(p->dp.w2, 0, w2_bytes)) != cudaSuccess) return fail(e);
     if ((e = cudaMemset(p->dp.w3, 0, w2_bytes)) != cudaSuccess) return fail(e);
     if ((e = cudaMalloc(&p->dp.status, sizeof(int))) != cudaSuccess) return fail(e);
-    if ((e = cudaMalloc(&p->dp.tail, 2 * sizeof(double) * max_batch)) != cudaSuccess) return fail(e);
+    if ((e = cudaMalloc(&p->dp.tail, 2 * sizeof(double) * gsp::kTailSlots * max_batch)) != cudaSuccess) return fail(e);
     if ((e = cudaMemset(p->dp.status, 0, sizeof(int))) != cudaSuccess) return fail(e);
     if (!any && gsp::xy_forms(N, dtype) != 1) {
         const size_t sync_bytes = sizeof(int) * (size_t)gsp::xy_sync_ints();
@@ -983,24 +983,37 @@ extern "C" int poisson_solve_timed(poisson_plan p, const void *rho_d, void *u_d,
     return POISSON_OK;
 }
 
+// The solves of `count` densities with their energy sums; eta[b] from the sums over the pairs.
+static int solve_checked(poisson_plan p, const gsp::PtrArray &in, const gsp::PtrArray &out, int count, double *eta,
+                         cudaStream_t s) {
+    const size_t bytes = 2 * sizeof(double) * gsp::kTailSlots * (size_t)count;
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(p->dp.tail, 0, bytes, s)) != cudaSuccess) return map_cuda(e);
+    if ((e = gsp::launch_solve(p->dp, in, out, count, s, nullptr, p->dp.tail)) != cudaSuccess) return map_cuda(e);
+    double h[2 * gsp::kTailSlots * gsp::kMaxBatch];
+    if ((e = cudaMemcpyAsync(h, p->dp.tail, bytes, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return map_cuda(e);
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return map_cuda(e);
+    for (int b = 0; b < count; ++b) {
+        double shell = 0.0, total = 0.0;
+        for (int i = 0; i < gsp::kTailSlots; ++i) {
+            shell += h[2 * (b * gsp::kTailSlots + i)];
+            total += h[2 * (b * gsp::kTailSlots + i) + 1];
+        }
+        eta[b] = total > 0.0 ? std::sqrt(shell / total) : 0.0;
+    }
+    return POISSON_OK;
+}
+
 extern "C" int poisson_solve_checked(poisson_plan p, const void *rho_d, void *u_d, double *eta,
                                      void *stream) {
     int rc = check_solve_args(p, rho_d, u_d);
     if (rc) return rc;
     if (!eta) return POISSON_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(p->dp.tail, 0, 2 * sizeof(double), s)) != cudaSuccess) return map_cuda(e);
     gsp::PtrArray in, out;
     one(in, rho_d);
     one(out, u_d);
-    if ((e = gsp::launch_solve(p->dp, in, out, 1, s, nullptr, p->dp.tail)) != cudaSuccess) return map_cuda(e);
-    double h[2] = {0.0, 0.0};
-    if ((e = cudaMemcpyAsync(h, p->dp.tail, sizeof(h), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-        return map_cuda(e);
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return map_cuda(e);
-    *eta = h[1] > 0.0 ? std::sqrt(h[0] / h[1]) : 0.0;
-    return POISSON_OK;
+    return solve_checked(p, in, out, 1, eta, s);
 }
 
 extern "C" int poisson_solve_checked_batched(poisson_plan p, int count, const void *const *rho_d, void *const *u_d,
@@ -1008,21 +1021,12 @@ extern "C" int poisson_solve_checked_batched(poisson_plan p, int count, const vo
     if (!p || !rho_d || !u_d || !eta || count < 1 || count > p->dp.max_batch) return POISSON_ERR_ARG;
     for (int i = 0; i < count; ++i)
         if (!rho_d[i] || !u_d[i]) return POISSON_ERR_ARG;
-    cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(p->dp.tail, 0, 2 * sizeof(double) * count, s)) != cudaSuccess) return map_cuda(e);
     gsp::PtrArray in, out;
     for (int i = 0; i < gsp::kMaxBatch; ++i) {
         in.p[i] = i < count ? rho_d[i] : nullptr;
         out.p[i] = i < count ? u_d[i] : nullptr;
     }
-    if ((e = gsp::launch_solve(p->dp, in, out, count, s, nullptr, p->dp.tail)) != cudaSuccess) return map_cuda(e);
-    double h[2 * gsp::kMaxBatch];
-    if ((e = cudaMemcpyAsync(h, p->dp.tail, 2 * sizeof(double) * count, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-        return map_cuda(e);
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return map_cuda(e);
-    for (int i = 0; i < count; ++i) eta[i] = h[2 * i + 1] > 0.0 ? std::sqrt(h[2 * i] / h[2 * i + 1]) : 0.0;
-    return POISSON_OK;
+    return solve_checked(p, in, out, count, eta, (cudaStream_t)stream);
 }
 
 extern "C" int poisson_last_status(poisson_plan p, void *stream) {

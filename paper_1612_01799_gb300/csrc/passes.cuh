@@ -29,6 +29,11 @@
 
 namespace gsp {
 
+// The pair of energy sums this CTA adds to for density b.
+__device__ __forceinline__ double *tail_pair(double *tail, int b) {
+    return tail + 2 * (b * kTailSlots + (int)(blockIdx.x % kTailSlots));
+}
+
 // Per-thread element count E and radix sequence of a length-L transform.  The first and
 // the last radix are even: the pruning rules (inputs r >= R/2 of stage 0 are zero, outputs
 // r >= R/2 of the last stage are dropped) select exactly the rows >= L/2 only then.

@@ -601,8 +601,8 @@ k_any_col(const Cx2<Real> *__restrict__ in, Cx2<Real> *__restrict__ out, const A
 // Tile (tx, ky, b): 2^lg groups of columns kx of line ky of density b.  Forward length Lz = 2 nz
 // (input z < nz), product with the symbol at (|kx|, |ky|, |kz|), inverse, z < nz stored.  With
 // TAIL the forward spectrum's energy in the outer shell (|k_q| >= n_q - n_q / 8 on some axis)
-// and its total energy go to tail[2 b], tail[2 b + 1] (FP32 per thread, FP64 per tile, one
-// atomic pair per tile).  The tiles cover the lines ky0 <= ky < ky0 + nky (all of them:
+// and its total energy go to its pair of tail (FP32 per thread, FP64 per tile, one atomic pair
+// per tile).  The tiles cover the lines ky0 <= ky < ky0 + nky (all of them:
 // ky0 = 0, nky = 2 ny, taken as ky and its mirror in turn, which read the same symbol rows; a
 // rank's slab of lines in the slab decomposition of one solve).
 template <typename Real, bool TAIL>
@@ -688,7 +688,7 @@ k_any_z(const Cx2<Real> *__restrict__ in, Cx2<Real> *__restrict__ out, const Rea
             if (threadIdx.x < 2) {
                 double sum = 0.0;
                 for (unsigned w = 0; w < blockDim.x / 32; ++w) sum += sm_ld(part + 2 * w + threadIdx.x);
-                atomicAdd(tail + 2 * bb + threadIdx.x, sum);
+                atomicAdd(tail_pair(tail, bb) + threadIdx.x, sum);
             }
         }
     }

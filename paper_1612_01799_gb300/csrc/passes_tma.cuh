@@ -324,8 +324,8 @@ k_z_symbol_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ 
                 }
             }
             if (tma_threads<Real, L, 1>() < 32 || (threadIdx.x & 31) == 0) {
-                atomicAdd(tail + 2 * bb, (double)eshell);
-                atomicAdd(tail + 2 * bb + 1, (double)etot);
+                atomicAdd(tail_pair(tail, bb), (double)eshell);
+                atomicAdd(tail_pair(tail, bb) + 1, (double)etot);
             }
         }
         ok = mbar_wait(bar + 1, phase, status);
@@ -503,8 +503,8 @@ k_z_split_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ C
                 }
             }
             if (NT < 32 || (threadIdx.x & 31) == 0) {
-                atomicAdd(tail + 2 * bb, (double)eshell);
-                atomicAdd(tail + 2 * bb + 1, (double)etot);
+                atomicAdd(tail_pair(tail, bb), (double)eshell);
+                atomicAdd(tail_pair(tail, bb) + 1, (double)etot);
             }
         }
         ok = mbar_wait(bar + 1, phase, status);

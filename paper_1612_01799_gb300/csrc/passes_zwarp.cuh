@@ -411,8 +411,8 @@ k_z_warp(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
                 etot += __shfl_xor_sync(0xffffffffu, etot, o);
             }
             if (valid && q == 0) {
-                atomicAdd(tail + 2 * bb, (double)eshell);
-                atomicAdd(tail + 2 * bb + 1, (double)etot);
+                atomicAdd(tail_pair(tail, bb), (double)eshell);
+                atomicAdd(tail_pair(tail, bb) + 1, (double)etot);
             }
         }
         if (!mbar_wait(bar + 1, ph, status)) return;
@@ -1303,8 +1303,8 @@ k_z_w512(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
                 etot += __shfl_xor_sync(0xffffffffu, etot, o);
             }
             if (valid && q == 0) {
-                atomicAdd(tail + 2 * bb, (double)eshell);
-                atomicAdd(tail + 2 * bb + 1, (double)etot);
+                atomicAdd(tail_pair(tail, bb), (double)eshell);
+                atomicAdd(tail_pair(tail, bb) + 1, (double)etot);
             }
         }
         if (!bad) bad = !mbar_wait(bar + 1, ph, status);

@@ -9,11 +9,12 @@
 // MLP: 64 -> 64 -> 64 -> 64 -> K with ReLU on the hidden layers, FP32.  Parameters in one
 // array: W1 (64x64), b1, W2 (64x64), b2, W3 (64x64), b3, W4 (K x 64), b4; W[j][i] multiplies
 // input i into unit j.  Training kernels: forward (keeping the hidden activations), loss
-// gradient of the mean squared error, backward (parameter gradients accumulated with
-// atomics), Adam.
+// gradient of the mean squared error, backward (parameter gradients summed per block, the
+// blocks added with atomics), Adam.
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdint>
 
 #include "../../include/poisson.h"
 #include "solver.h"
@@ -108,87 +109,156 @@ __host__ __device__ inline int off_w(int l) { return l * (kH * kH + kH); }
 __host__ __device__ inline int off_b(int l) { return l * (kH * kH + kH) + kH * kH; }
 __host__ __device__ inline int nparams(int K) { return 3 * (kH * kH + kH) + K * kH + K; }
 
-// One block (64 threads) per sample.  acts: B x 3 x 64 hidden activations (may be null).
-__global__ void __launch_bounds__(kH) k_forward(const float *__restrict__ p, int K, const float *__restrict__ x,
-                                                  float *__restrict__ y, float *__restrict__ acts) {
-    __shared__ float h[2][kH];
-    const int j = threadIdx.x, b = blockIdx.x;
-    h[0][j] = x[(size_t)b * kH + j];
+// Samples per block of the forward and backward passes: a block stages the weights in shared
+// memory once for all its samples, thread (j, sample) makes unit j.
+constexpr int kFwdT = 4, kBwdT = 8, kNT = 256;
+constexpr int kWP = kH + 1;  // pitch of a transposed weight matrix
+
+// acts: B x 3 x 64 hidden activations (may be null).  The weights of all layers come in with
+// coalesced loads, transposed so that the units of a warp read neighbouring words (one block
+// per sample with each thread walking its own row of W took 23 us for 384 samples; TODO us here).
+__global__ void __launch_bounds__(kNT) k_forward(const float *__restrict__ p, int K, const float *__restrict__ x,
+                                                 int count, float *__restrict__ y, float *__restrict__ acts) {
+    extern __shared__ float sw[];  // W1^T, W2^T, W3^T, W4^T
+    __shared__ float h[2][kFwdT][kH];
+    const int j = threadIdx.x % kH, t = threadIdx.x / kH, b = blockIdx.x * kFwdT + t;
+    for (int l = 0; l < 3; ++l)
+#pragma unroll
+        for (int e = threadIdx.x; e < kH * kH; e += kNT) sw[l * kH * kWP + (e % kH) * kWP + e / kH] = p[off_w(l) + e];
+    for (int e = threadIdx.x; e < K * kH; e += kNT) sw[3 * kH * kWP + (e % kH) * kWP + e / kH] = p[off_w(3) + e];
+    h[0][t][j] = b < count ? x[(size_t)b * kH + j] : 0.f;
     __syncthreads();
     int cur = 0;
     for (int l = 0; l < 3; ++l) {
-        const float *W = p + off_w(l);
+        const float *W = sw + l * kH * kWP + j;
         float a = p[off_b(l) + j];
-        for (int i = 0; i < kH; ++i) a += W[j * kH + i] * h[cur][i];
+#pragma unroll 16
+        for (int i = 0; i < kH; ++i) a += W[i * kWP] * h[cur][t][i];
         a = fmaxf(a, 0.f);
-        if (acts) acts[((size_t)b * 3 + l) * kH + j] = a;
-        h[1 - cur][j] = a;
+        if (acts && b < count) acts[((size_t)b * 3 + l) * kH + j] = a;
+        h[1 - cur][t][j] = a;
         __syncthreads();
         cur = 1 - cur;
     }
-    if (j < K) {
-        const float *W = p + off_w(3);
+    if (j < K && b < count) {
+        const float *W = sw + 3 * kH * kWP + j;
         float a = p[off_w(3) + K * kH + j];
-        for (int i = 0; i < kH; ++i) a += W[j * kH + i] * h[cur][i];
+#pragma unroll 16
+        for (int i = 0; i < kH; ++i) a += W[i * kWP] * h[cur][t][i];
         y[(size_t)b * K + j] = a;
     }
 }
+constexpr int kFwdSmem = 4 * kH * kWP * (int)sizeof(float);
 
 // dy = 2 (y - t) / (B K) and the loss sum (y - t)^2 / (B K) (one block).
-__global__ void k_loss(const float *__restrict__ y, const float *__restrict__ t, int n, float *__restrict__ dy,
-                       float *__restrict__ loss) {
-    __shared__ float s[256];
+constexpr int kLossNT = 1024;
+__global__ void __launch_bounds__(kLossNT) k_loss(const float *__restrict__ y, const float *__restrict__ t, int n,
+                                                  float *__restrict__ dy, float *__restrict__ loss) {
+    __shared__ float s[kLossNT / 32];
     float acc = 0.f;
-    for (int i = threadIdx.x; i < n; i += 256) {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += kLossNT) {
         const float d = y[i] - t[i];
         dy[i] = 2.f * d / n;
         acc += d * d;
     }
-    s[threadIdx.x] = acc;
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (threadIdx.x % 32 == 0) s[threadIdx.x / 32] = acc;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
-        __syncthreads();
+    if (threadIdx.x < 32) {
+        acc = s[threadIdx.x];
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (threadIdx.x == 0) *loss = acc / n;
     }
-    if (threadIdx.x == 0) *loss = s[0] / n;
 }
 
-// One block per sample; parameter gradients added into g.
-__global__ void __launch_bounds__(kH) k_backward(const float *__restrict__ p, int K, const float *__restrict__ x,
-                                                   const float *__restrict__ acts, const float *__restrict__ dy,
-                                                   float *__restrict__ g) {
-    __shared__ float a[4][kH];   // layer inputs: x, h1, h2, h3
-    __shared__ float d[2][kH];   // deltas
-    const int j = threadIdx.x, b = blockIdx.x;
-    a[0][j] = x[(size_t)b * kH + j];
-    for (int l = 0; l < 3; ++l) a[l + 1][j] = acts[((size_t)b * 3 + l) * kH + j];
-    __syncthreads();
-    // output layer
-    const float *W4 = p + off_w(3);
-    float *gW4 = g + off_w(3), *gb4 = g + off_w(3) + K * kH;
-    for (int k = 0; k < K; ++k) {
-        const float e = dy[(size_t)b * K + k];
-        atomicAdd(&gW4[k * kH + j], e * a[3][j]);
-        if (j == 0) atomicAdd(&gb4[k], e);
+// g[0..3] += v, in one reduction where g is 16-byte aligned.
+__device__ __forceinline__ void add4(float *g, float4 v, bool vec) {
+    if (vec) {
+        atomicAdd(reinterpret_cast<float4 *>(g), v);
+    } else {
+        atomicAdd(g, v.x);
+        atomicAdd(g + 1, v.y);
+        atomicAdd(g + 2, v.z);
+        atomicAdd(g + 3, v.w);
     }
-    float acc = 0.f;
-    for (int k = 0; k < K; ++k) acc += W4[k * kH + j] * dy[(size_t)b * K + k];
-    d[0][j] = a[3][j] > 0.f ? acc : 0.f;
+}
+
+// A block takes kBwdT samples: their deltas back through the layers, then its part of each
+// weight gradient, sum_b delta_j a_i, as a 4 x 4 tile per thread summed in registers over the
+// samples, added to g with one 16-byte reduction per row (vec: g is 16-byte aligned).  One
+// atomic per sample and parameter, as before, is 5 million at 13 thousand addresses for 384
+// samples: 97 us, TODO us here.
+__global__ void __launch_bounds__(kNT) k_backward(const float *__restrict__ p, int K, const float *__restrict__ x,
+                                                  const float *__restrict__ acts, int count,
+                                                  const float *__restrict__ dy, float *__restrict__ g, bool vec) {
+    __shared__ __align__(16) float a[4][kBwdT][kH];  // layer inputs: x, h1, h2, h3
+    __shared__ __align__(16) float d[3][kBwdT][kH];  // deltas of layers 1, 2, 3
+    __shared__ float e[kBwdT][kMaxK];
+    __shared__ float W[2][kH * kH];                  // W2, W3
+    const int tid = threadIdx.x, j = tid % kH, b0 = blockIdx.x * kBwdT, nb = min(kBwdT, count - b0);
+#pragma unroll
+    for (int l = 1; l < 3; ++l)
+        for (int i = tid; i < kH * kH; i += kNT) W[l - 1][i] = p[off_w(l) + i];
+    for (int t = tid / kH; t < kBwdT; t += kNT / kH) {
+        const bool ok = t < nb;
+        a[0][t][j] = ok ? x[(size_t)(b0 + t) * kH + j] : 0.f;
+        for (int l = 0; l < 3; ++l) a[l + 1][t][j] = ok ? acts[((size_t)(b0 + t) * 3 + l) * kH + j] : 0.f;
+        if (j < K) e[t][j] = ok ? dy[(size_t)(b0 + t) * K + j] : 0.f;
+    }
     __syncthreads();
-    int cur = 0;
-    for (int l = 2; l >= 0; --l) {
-        const float *W = p + off_w(l);
-        float *gW = g + off_w(l), *gb = g + off_b(l);
-        const float dj = d[cur][j];
-        for (int i = 0; i < kH; ++i) atomicAdd(&gW[j * kH + i], dj * a[l][i]);
-        atomicAdd(&gb[j], dj);
-        if (l > 0) {
+    for (int t = tid / kH; t < kBwdT; t += kNT / kH) {
+        float acc = 0.f;
+        for (int k = 0; k < K; ++k) acc += p[off_w(3) + k * kH + j] * e[t][k];
+        d[2][t][j] = a[3][t][j] > 0.f ? acc : 0.f;
+    }
+    __syncthreads();
+    for (int l = 2; l > 0; --l) {
+        for (int t = tid / kH; t < kBwdT; t += kNT / kH) {
             float s = 0.f;
-            for (int k = 0; k < kH; ++k) s += W[k * kH + j] * d[cur][k];
-            d[1 - cur][j] = a[l][j] > 0.f ? s : 0.f;
+#pragma unroll 16
+            for (int k = 0; k < kH; ++k) s += W[l - 1][k * kH + j] * d[l][t][k];
+            d[l - 1][t][j] = a[l][t][j] > 0.f ? s : 0.f;
         }
         __syncthreads();
-        cur = 1 - cur;
+    }
+    const int r0 = 4 * (tid / 16), c0 = 4 * (tid % 16);
+    for (int l = 0; l < 3; ++l) {
+        float4 acc[4] = {};
+#pragma unroll
+        for (int t = 0; t < kBwdT; ++t) {
+            const float4 av = *reinterpret_cast<const float4 *>(&a[l][t][c0]);
+            const float4 dv = *reinterpret_cast<const float4 *>(&d[l][t][r0]);
+            const float dr[4] = {dv.x, dv.y, dv.z, dv.w};
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                acc[r].x += dr[r] * av.x;
+                acc[r].y += dr[r] * av.y;
+                acc[r].z += dr[r] * av.z;
+                acc[r].w += dr[r] * av.w;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) add4(g + off_w(l) + (r0 + r) * kH + c0, acc[r], vec);
+    }
+    if (tid / 16 < K) {  // output layer: row tid / 16
+        const int k = tid / 16;
+        float4 acc = {};
+#pragma unroll
+        for (int t = 0; t < kBwdT; ++t) {
+            const float4 av = *reinterpret_cast<const float4 *>(&a[3][t][c0]);
+            acc.x += e[t][k] * av.x;
+            acc.y += e[t][k] * av.y;
+            acc.z += e[t][k] * av.z;
+            acc.w += e[t][k] * av.w;
+        }
+        add4(g + off_w(3) + k * kH + c0, acc, vec);
+    }
+    for (int i = tid; i < 3 * kH + K; i += kNT) {  // biases
+        float s = 0.f;
+#pragma unroll
+        for (int t = 0; t < kBwdT; ++t) s += i < 3 * kH ? d[i / kH][t][i % kH] : e[t][i - 3 * kH];
+        atomicAdd(i < 3 * kH ? g + off_b(i / kH) + i % kH : g + off_w(3) + K * kH + i - 3 * kH, s);
     }
 }
 
@@ -226,14 +296,16 @@ extern "C" int poisson_mlp_forward(const float *params_d, int K, const float *x_
                                    float *acts_d, void *stream) {
     if (K < 1 || K > kMaxK || count < 0 || (count > 0 && (!params_d || !x_d || !y_d))) return POISSON_ERR_ARG;
     if (count == 0) return POISSON_OK;
-    k_forward<<<count, kH, 0, (cudaStream_t)stream>>>(params_d, K, x_d, y_d, acts_d);
+    const cudaError_t e = cudaFuncSetAttribute(k_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem);
+    if (e != cudaSuccess) return ok(e);
+    k_forward<<<(count + kFwdT - 1) / kFwdT, kNT, kFwdSmem, (cudaStream_t)stream>>>(params_d, K, x_d, count, y_d, acts_d);
     return ok(cudaGetLastError());
 }
 
 extern "C" int poisson_mlp_loss(const float *y_d, const float *target_d, int n, float *dy_d, float *loss_d,
                                 void *stream) {
     if (n < 1 || !y_d || !target_d || !dy_d || !loss_d) return POISSON_ERR_ARG;
-    k_loss<<<1, 256, 0, (cudaStream_t)stream>>>(y_d, target_d, n, dy_d, loss_d);
+    k_loss<<<1, kLossNT, 0, (cudaStream_t)stream>>>(y_d, target_d, n, dy_d, loss_d);
     return ok(cudaGetLastError());
 }
 
@@ -244,7 +316,8 @@ extern "C" int poisson_mlp_backward(const float *params_d, int K, const float *x
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e = cudaMemsetAsync(grad_d, 0, sizeof(float) * nparams(K), s);
     if (e != cudaSuccess || count == 0) return ok(e);
-    k_backward<<<count, kH, 0, s>>>(params_d, K, x_d, acts_d, dy_d, grad_d);
+    const bool vec = reinterpret_cast<uintptr_t>(grad_d) % 16 == 0;
+    k_backward<<<(count + kBwdT - 1) / kBwdT, kNT, 0, s>>>(params_d, K, x_d, acts_d, count, dy_d, grad_d, vec);
     return ok(cudaGetLastError());
 }
 

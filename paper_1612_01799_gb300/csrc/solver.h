@@ -59,7 +59,7 @@ struct DevicePlan {
     void *w2 = nullptr;
     void *w3 = nullptr;
     int *status = nullptr;  // device status word (bit 0: a bounded wait timed out)
-    double *tail = nullptr; // 2 max_batch doubles: spectral-tail sums of a checked solve
+    double *tail = nullptr; // spectral-tail sums of a checked solve: kTailSlots pairs per density
     // z pass form: 0 length-2N transforms, 1 even/odd length-N split, 2 warp form (one
     // warp per column pair, FP32, N = 64 ... 256; one warp per column at N = 512)
     int zform = 0;
@@ -85,6 +85,11 @@ struct DevicePlan {
     CUtensorMap tm_rf;                   // fused forward x-y pass: N-row boxes of its ring in w3
 };
 
+// Pairs (shell, total) that the CTAs of a checked z pass spread a density's energy sums over, added
+// up on the host.  With one pair every warp's FP64 atomics met at two addresses: 12 densities
+// of N = 96 took TODO us a call, TODO us with 32 pairs.
+constexpr int kTailSlots = 32;
+
 constexpr int kStatusTimeoutBit = 1;  // bit of DevicePlan::status set by a timed-out wait
 
 inline int pitch_for(int N) { return ((N + 1 + 15) / 16) * 16; }
@@ -105,8 +110,9 @@ cudaError_t encode_tma_maps(DevicePlan &p);
 
 // The five passes of `count` solves (1 <= count <= p.max_batch) of the plan's geometry on
 // `s`: rho[b] -> u[b].  ev: null, or 6 events recorded before pass 1, between the passes
-// and after pass 5.  tail: null, or 2 count zeroed doubles that receive, per density, the
-// padded spectrum's energy in the outer |k|_inf shell and its total energy.  skip: bit 0
+// and after pass 5.  tail: null, or 2 kTailSlots count zeroed doubles that receive, per density,
+// the padded spectrum's energy in the outer |k|_inf shell and its total energy (in kTailSlots
+// pairs to be added).  skip: bit 0
 // leaves out the forward x and y passes, bit 1 the inverse y and x passes (the caller runs
 // them with launch_xy_slab); not with the fused x-y form.
 cudaError_t launch_solve(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int count,
