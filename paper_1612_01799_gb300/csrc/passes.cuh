@@ -37,6 +37,10 @@ __device__ __forceinline__ double *tail_pair(double *tail, int b) {
 // Per-thread element count E and radix sequence of a length-L transform.  The first and
 // the last radix are even: the pruning rules (inputs r >= R/2 of stage 0 are zero, outputs
 // r >= R/2 of the last stage are dropped) select exactly the rows >= L/2 only then.
+// Fewest stages first, then the fewest values per thread that the radices allow: at 24 values
+// (8, 3, 8) the passes of length 192 kept 10 warps on an SM, at 12 (4, 12, 4) they keep 20 (N = 96:
+// double-float solve 224 -> 126 us, twelve FP32 densities 355 -> 332 us); length 160 as
+// 4, 10, 4 instead of 4, 4, 5, 2 took N = 80 in double-float from 117 to 91 us.
 template <int L> struct FftCfg;
 #define GSP_FFT_CFG(LL, EE, ...)                  \
     template <> struct FftCfg<LL> {              \
@@ -47,19 +51,19 @@ GSP_FFT_CFG(4, 4, 4);
 GSP_FFT_CFG(8, 8, 8);
 GSP_FFT_CFG(16, 16, 16);
 GSP_FFT_CFG(32, 8, 8, 4);
-GSP_FFT_CFG(48, 12, 4, 3, 4);
+GSP_FFT_CFG(48, 12, 4, 12);
 GSP_FFT_CFG(64, 8, 8, 8);
 GSP_FFT_CFG(80, 20, 4, 5, 4);
-GSP_FFT_CFG(96, 24, 8, 3, 4);
+GSP_FFT_CFG(96, 12, 4, 6, 4);
 GSP_FFT_CFG(128, 16, 16, 8);
-GSP_FFT_CFG(160, 20, 4, 4, 5, 2);
-GSP_FFT_CFG(192, 24, 8, 3, 8);
+GSP_FFT_CFG(160, 20, 4, 10, 4);
+GSP_FFT_CFG(192, 12, 4, 12, 4);
 GSP_FFT_CFG(256, 16, 16, 16);
 GSP_FFT_CFG(320, 20, 4, 4, 5, 4);
 GSP_FFT_CFG(384, 24, 8, 8, 6);
 GSP_FFT_CFG(512, 16, 16, 8, 4);
-GSP_FFT_CFG(640, 20, 4, 4, 4, 5, 2);
-GSP_FFT_CFG(768, 24, 8, 8, 6, 2);
+GSP_FFT_CFG(640, 20, 4, 4, 10, 4);
+GSP_FFT_CFG(768, 24, 8, 12, 8);
 GSP_FFT_CFG(1024, 16, 16, 16, 4);
 GSP_FFT_CFG(2048, 16, 16, 16, 8);
 #undef GSP_FFT_CFG
@@ -75,12 +79,12 @@ template <typename Real, int L> struct Cfg : FftCfg<L> {};
         using Rs = Radices<__VA_ARGS__>;         \
     }
 GSP_DF_CFG(16, 4, 4, 4);
-GSP_DF_CFG(96, 12, 4, 6, 4);
+GSP_DF_CFG(48, 12, 4, 3, 4);
 GSP_DF_CFG(128, 8, 8, 4, 4);
 GSP_DF_CFG(256, 8, 8, 8, 4);
 GSP_DF_CFG(384, 12, 4, 4, 6, 4);
 GSP_DF_CFG(512, 8, 8, 8, 8);
-GSP_DF_CFG(768, 12, 4, 4, 4, 6, 2);
+GSP_DF_CFG(768, 12, 4, 12, 4, 4);
 GSP_DF_CFG(1024, 8, 8, 8, 4, 4);
 GSP_DF_CFG(2048, 8, 8, 8, 8, 4);
 #undef GSP_DF_CFG

@@ -119,10 +119,10 @@ __device__ __forceinline__ CD scale_sym_sm(CD x, const double *s) { return cscal
 __device__ __forceinline__ CDF scale_sym_sm(CDF x, const DF *s) { return cscale(x, sm_ld(s)); }
 
 // Blocks per SM requested from the compiler: a register budget of 64 per thread for E <= 8
-// values per thread, 128 otherwise.
+// values per thread, 96 for E <= 12, 128 otherwise.
 template <int T, int E> __host__ __device__ constexpr int min_blocks_for() {
     // Bounded by the SM's 65536 registers, 2048 threads and 32 resident blocks.
-    const int regs = E <= 8 ? 64 : 128;
+    const int regs = E <= 8 ? 64 : E <= 12 ? 96 : 128;
     const int by_regs = 65536 / (T * regs), by_threads = 2048 / T;
     const int b = by_regs < by_threads ? by_regs : by_threads;
     return b > 32 ? 32 : b > 0 ? b : 1;
@@ -363,19 +363,12 @@ k_z_symbol_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ 
 // inputs x_n, n < N, are the nonzero half).  The kept inverse outputs split the same way:
 // u_z = A_z + conj(W_{2N}^z) B_z for z < N, with A and B the length-N inverse DFTs of the
 // even and odd halves of the spectrum.  Half h of the threads of a column group runs the
-// length-N transforms of parity h.  Where the length-N schedule has one stage fewer than
-// the length-2N one, this saves one shared-memory exchange per direction, for the price of
-// reading the staged input twice and one half-size exchange that adds A and B.
-template <class RL> struct NumStages;
-template <int... Rs> struct NumStages<Radices<Rs...>> { static constexpr int v = sizeof...(Rs); };
-
+// length-N transforms of parity h.  At N = 256, 320 and 384 the length-N schedule has one stage
+// fewer than the length-2N one, which saves a shared-memory exchange per direction, for the
+// price of reading the staged input twice and one half-size exchange that adds A and B (the
+// form also exists at N = 16 and 80).
 template <int L> __host__ __device__ constexpr bool zsplit_available() {
-    if constexpr (L < 8) {
-        return false;
-    } else {
-        using Rh = typename FftCfg<L / 2>::Rs;
-        return NumStages<Rh>::v < NumStages<typename FftCfg<L>::Rs>::v && FirstRadix<Rh>::v % 2 == 0;
-    }
+    return L == 32 || L == 160 || L == 512 || L == 640 || L == 768;
 }
 template <typename Real, int L> __host__ __device__ constexpr int zsplit_threads() {
     return TmaLayout<Real, L, 1>::NG * 2 * ((L / 2) / FftCfg<L / 2>::E);
