@@ -112,7 +112,8 @@ int poisson_plan_create_box(poisson_plan *out, int N, double Lx, double Ly, doub
  * nx = ny = nz this is poisson_plan_create_box.  Plans whose counts differ (or whose common
  * count has no compiled transform schedule, poisson_supported_n() == 2) run the
  * runtime-length forms of the five passes: one form per pass (the form knobs have only
- * value 0), the same arithmetics, no TMA staging.  poisson_plan_axis_table returns the x
+ * value 0; small planes take the x and y passes of a direction in one kernel), the same
+ * arithmetics, no TMA staging.  poisson_plan_axis_table returns the x
  * axis's factors (n_terms x (nx + 1)).  Other arguments, errors and use as for
  * poisson_plan_create (one density per solve).
  */
@@ -141,7 +142,8 @@ int poisson_solve(poisson_plan p, const void *rho_d, void *u_d, void *stream);
  * and synchronises the stream before returning.  rho_h, u_h: host pointers to N^3
  * values of the plan's dtype (pinned memory gives full copy bandwidth).  Uses the
  * plan's own device staging buffers.  Where N is a multiple of 8 (N >= 16) and the x and y
- * passes are separate launches, the copies run in 8 z-slabs on a copy stream of the plan,
+ * passes are separate launches (not the fused form, nor a runtime-length plan with small
+ * planes), the copies run in 8 z-slabs on a copy stream of the plan,
  * overlapped with the x and y passes of the neighbouring slabs (those passes transform
  * each z-plane on its own); they start after the work already queued on `stream`.  The result is the
  * same, bit for bit, as poisson_solve's on device copies of the buffers.
@@ -196,7 +198,8 @@ int poisson_compare(const void *a_d, int a_dtype, const void *b_d, int b_dtype, 
  * forward + symbol + z inverse, y inverse, x inverse).  ms[5] receives them.  With the
  * fused x-y form (POISSON_KNOB_XY_FORM = 1) the forward x and y passes are one kernel,
  * timed in ms[0] with ms[1] = 0, and the inverse y and x passes are one kernel, timed in
- * ms[3] with ms[4] = 0.  The call synchronises the stream.  Same arguments and aliasing
+ * ms[3] with ms[4] = 0; so are they in runtime-length plans whose planes are small enough for
+ * one kernel per direction.  The call synchronises the stream.  Same arguments and aliasing
  * rules as poisson_solve.
  */
 int poisson_solve_timed(poisson_plan p, const void *rho_d, void *u_d, void *stream, float *ms);

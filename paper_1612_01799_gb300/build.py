@@ -27,6 +27,7 @@ SOURCES = ["capi.cpp", "setup.cpp", "passes_f32.cu", "passes_f64.cu", "passes_df
            "passes_any_f32_x.cu", "passes_any_f32_y.cu", "passes_any_f32_z.cu",
            "passes_any_f64_x.cu", "passes_any_f64_y.cu", "passes_any_f64_z.cu",
            "passes_any_df_x.cu", "passes_any_df_y.cu", "passes_any_df_z.cu",
+           "passes_plane_f32.cu", "passes_plane_f64.cu", "passes_plane_df.cu",
            "noalloc.cu", "reduce.cu", "sample.cu", "selector.cu", "selftest.cu", "setup_device.cu", "debug.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -133,6 +133,47 @@ inline AnyTile any_tile(int L, int max_radix, int max_warps, bool rows) {
     return t;
 }
 
+// Tile of the plane kernels (passes_plane.cuh): the x and y passes of one nx x ny plane in
+// shared memory, gx row groups (pitch px) by sx.slots and gy column groups (pitch py) by sy.slots;
+// w columns or rows per 16-byte group.  threads as for any_tile, over the stages of both axes.
+struct PlaneTile {
+    AnySched sx, sy;
+    int gx, px, gy, py, threads, smem;
+    bool on;
+};
+constexpr int kPlaneThreads = 384;
+// Largest plane: in FP32 two CTAs fit an SM (solves, separate passes against the plane kernels:
+// 20^3 21.4 and 18.9 us, 60^3 27.2 and 25.5, 64 x 64 x 256 66 and 57, but 72^3 28.6 and 30.2); the
+// wider arithmetics are bound by the longer chain of one CTA soon (20^3 30.6 and 28.7, 36^3 39.6
+// and 41.2).  Cubes whose passes are compiled for their length stay with those (32^3 12.6 and
+// 18.6 us).
+constexpr int plane_smem(bool f32) { return f32 ? 106 * 1024 : 48 * 1024; }
+inline PlaneTile plane_tile(int nx, int ny, int max_radix, int w) {
+    PlaneTile t{};
+    t.sx = any_sched(nx, max_radix, kAnyRowsLast, true);
+    t.sy = any_sched(2 * ny, max_radix, max_radix, false);
+    t.gx = ny / w;
+    t.gy = (nx + w) / w;
+    t.px = t.gx | 1;
+    t.py = t.gy | 1;
+    t.smem = 16 * (t.sx.slots * t.px + t.sy.slots * t.py);
+    // The fewest rounds of butterflies per thread, weighted by their radix; among equals the
+    // fewest threads.
+    int best = 0;
+    for (int n = kPlaneThreads; n >= 128; n -= 32) {
+        int rounds = 0;
+        for (const AnySched *s : {&t.sx, &t.sy})
+            for (int st = 0; st < s->nst; ++st)
+                rounds += (s->L / s->r[st] * (s == &t.sx ? t.gx : t.gy) + n - 1) / n * s->r[st];
+        if (n == kPlaneThreads || rounds <= best) {
+            best = rounds;
+            t.threads = n;
+        }
+    }
+    t.on = t.sx.nst && t.sy.nst && t.smem <= plane_smem(w == 2);
+    return t;
+}
+
 // e / d by its reciprocal mul.
 GSP_HD inline int rdiv(int e, unsigned mul) { return (int)(((unsigned long long)(unsigned)e * mul) >> 32); }
 

@@ -951,19 +951,27 @@ cudaError_t any_y(const DevicePlan &p, int B, cudaStream_t s, bool fwd, int z0 =
 template <typename Real>
 cudaError_t any_z(const DevicePlan &p, int B, cudaStream_t s, double *tail, int ky0 = 0, int nky = 0);
 
+// The x and y passes of small planes, one kernel per direction (passes_plane_*.cu).
+template <typename Real>
+cudaError_t plane_xy(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int B, cudaStream_t s, bool fwd);
+
 template <typename Real>
 cudaError_t solve_any(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int B, cudaStream_t s,
                       cudaEvent_t *ev, double *tail, int skip) {
+    const bool plane = plane_on(p);
+    if (plane && skip) return cudaErrorInvalidValue;
     if (ev) GSP_CHECK(cudaEventRecord(ev[0], s));
-    if (!(skip & 1)) GSP_CHECK(any_x<Real>(p, rho, u, B, s, true));
+    if (plane) GSP_CHECK(plane_xy<Real>(p, rho, u, B, s, true));
+    else if (!(skip & 1)) GSP_CHECK(any_x<Real>(p, rho, u, B, s, true));
     if (ev) GSP_CHECK(cudaEventRecord(ev[1], s));
-    if (!(skip & 1)) GSP_CHECK(any_y<Real>(p, B, s, true));
+    if (!plane && !(skip & 1)) GSP_CHECK(any_y<Real>(p, B, s, true));
     if (ev) GSP_CHECK(cudaEventRecord(ev[2], s));
     GSP_CHECK(any_z<Real>(p, B, s, tail));
     if (ev) GSP_CHECK(cudaEventRecord(ev[3], s));
-    if (!(skip & 2)) GSP_CHECK(any_y<Real>(p, B, s, false));
+    if (plane) GSP_CHECK(plane_xy<Real>(p, rho, u, B, s, false));
+    else if (!(skip & 2)) GSP_CHECK(any_y<Real>(p, B, s, false));
     if (ev) GSP_CHECK(cudaEventRecord(ev[4], s));
-    if (!(skip & 2)) GSP_CHECK(any_x<Real>(p, rho, u, B, s, false));
+    if (!plane && !(skip & 2)) GSP_CHECK(any_x<Real>(p, rho, u, B, s, false));
     if (ev) GSP_CHECK(cudaEventRecord(ev[5], s));
     return cudaSuccess;
 }

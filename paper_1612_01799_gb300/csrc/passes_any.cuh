@@ -229,7 +229,7 @@ template <typename Real> struct AnyTwiddles {
     }
 };
 // Bytes of shared memory of the copy.
-template <typename Real> constexpr int any_tw_bytes(int L) {
+template <typename Real> __host__ __device__ constexpr int any_tw_bytes(int L) {
     return AnyTwiddles<Real>::kCopy ? (L * (int)sizeof(AnyTw<Real>) + 15) / 16 * 16 : 0;
 }
 

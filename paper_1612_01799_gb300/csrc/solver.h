@@ -48,7 +48,10 @@ struct DevicePlan {
     int n3[3] = {0, 0, 0};
     void *tw3[3] = {nullptr, nullptr, nullptr};
     // Tiles of the runtime-length passes along x, y and z, per arithmetic (any_plan_tiles).
-    AnyTile any_tile[2][3];
+    AnyTile any_tile[2][3] = {};
+    // The x and y passes as one kernel per direction (passes_plane.cuh), per arithmetic: on for
+    // runtime-length plans whose planes are small (plane_on).
+    PlaneTile plane[2] = {};
     int Px = 0;
     int Ps = 0;
     void *sym = nullptr;
@@ -98,8 +101,10 @@ inline int sym_pitch_for(int N) { return ((N + 1 + 3) / 4) * 4; }
 bool n_supported(int N);
 
 // Fill p.any_tile for p's lengths (any plan: the slab z pass runs on the compiled-length
-// plans too).
+// plans too) and p.plane.
 void any_plan_tiles(DevicePlan &p);
+// Whether p's solves run the plane kernels in its present arithmetic.
+inline bool plane_on(const DevicePlan &p) { return p.plane[p.arith].on; }
 
 // Record a failed CUDA call for poisson_last_cuda_error() (per host thread).
 void note_cuda_error(cudaError_t e);
