@@ -9,16 +9,25 @@ from . import _lib
 DTYPES = {"f32": _lib.F32, "f64": _lib.F64}
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream_handle(stream):
+    """cudaStream_t of a torch stream (None: the current one) as an integer."""
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def supported_n(N):
@@ -43,6 +52,7 @@ class Plan:
         self.npoints = self.n[0] * self.n[1] * self.n[2]
         self.max_batch = int(max_batch)
         self._lib = _lib.load()
+        self._tdtype = None
         self._h = ctypes.c_void_p()
         if np.ndim(N) and not np.ndim(L):
             L = (float(L),) * 3
@@ -74,10 +84,11 @@ class Plan:
         return np.float32 if self.dtype == "f32" else np.float64
 
     def _check_tensor(self, t, name):
-        torch = _torch()
-        if not isinstance(t, torch.Tensor) or not t.is_cuda:
+        if self._tdtype is None:
+            self._tdtype = self.torch_dtype
+        if not isinstance(t, _torch().Tensor) or not t.is_cuda:
             raise TypeError("%s must be a CUDA tensor" % name)
-        if t.dtype != self.torch_dtype or t.numel() != self.npoints or not t.is_contiguous():
+        if t.dtype != self._tdtype or t.numel() != self.npoints or not t.is_contiguous():
             raise ValueError("%s must be a contiguous %s tensor of nx ny nz = %d values"
                              % (name, self.torch_dtype, self.npoints))
 
@@ -87,8 +98,7 @@ class Plan:
         if out is None:
             out = _torch().empty_like(rho)
         self._check_tensor(out, "out")
-        _lib.check(self._lib.poisson_solve(self._h, ctypes.c_void_p(rho.data_ptr()),
-                                           ctypes.c_void_p(out.data_ptr()), _stream_handle(stream)),
+        _lib.check(self._lib.poisson_solve(self._h, rho.data_ptr(), out.data_ptr(), _stream_handle(stream)),
                    "poisson_solve")
         return out
 

@@ -469,8 +469,6 @@ template <class K> static cudaError_t set_smem(K kernel, size_t bytes) {
         if (e_ != cudaSuccess) return e_;     \
     } while (0)
 
-// Blocks of a persistent kernel: as many as fit on all SMs at once.  The occupancy of
-// each kernel is queried once and cached by the kernel's address.
 // Launch with programmatic dependent launch allowed: the kernel's CTAs may become resident
 // and build their shared tables while the previous kernel on the stream finishes; every
 // pass kernel calls griddep_wait before it touches memory that kernel writes or reads.
@@ -490,12 +488,17 @@ static cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t
     return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
+// Blocks of a persistent kernel: as many as fit on all SMs at once.
+// The count for (kernel, threads, smem) is queried once per device and kept, up to kGridEntries of
+// them (the runtime-length passes come with many shapes; later ones are queried each time).
+constexpr int kGridEntries = 256;
 template <class K> static int persistent_blocks(K kernel, int threads, size_t smem, int ntiles) {
     struct Entry {
         const void *fn;
-        int dev, blocks;
+        size_t smem;
+        int dev, threads, blocks;
     };
-    static Entry cache[64];
+    static Entry cache[kGridEntries];
     static int n = 0;
     static std::mutex mu;  // plans may launch from several host threads
     const void *fn = reinterpret_cast<const void *>(kernel);
@@ -503,8 +506,10 @@ template <class K> static int persistent_blocks(K kernel, int threads, size_t sm
     cudaGetDevice(&dev);
     {
         std::lock_guard<std::mutex> lock(mu);
-        for (int i = 0; i < n; ++i)
-            if (cache[i].fn == fn && cache[i].dev == dev) blocks = cache[i].blocks;
+        for (int i = 0; i < n && !blocks; ++i) {
+            const Entry &e = cache[i];
+            if (e.fn == fn && e.dev == dev && e.threads == threads && e.smem == smem) blocks = e.blocks;
+        }
     }
     if (blocks == 0) {
         int sms = 1, per_sm = 1;
@@ -514,7 +519,7 @@ template <class K> static int persistent_blocks(K kernel, int threads, size_t sm
             per_sm = 1;
         blocks = per_sm * (sms > 0 ? sms : 1);
         std::lock_guard<std::mutex> lock(mu);
-        if (n < 64) cache[n++] = Entry{fn, dev, blocks};
+        if (n < kGridEntries) cache[n++] = Entry{fn, smem, dev, threads, blocks};
     }
     return blocks < ntiles ? blocks : ntiles;
 }

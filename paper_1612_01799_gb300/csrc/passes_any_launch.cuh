@@ -1,7 +1,5 @@
 // Launchers of the runtime-length forms, included by one .cu file per arithmetic.
 #pragma once
-#include <algorithm>
-
 #include "passes.cuh"
 #include "passes_any.cuh"
 
@@ -11,12 +9,7 @@ namespace gsp {
 // the twiddles.  The others hold no copy and take one tile each (double-float, N = 162 and 200:
 // z 479 and 950 us, against 551 and 1106 us when the CTAs walk the tiles).
 template <typename Real, class K> int any_grid(K k, const AnyTile &t, int smem, int ntiles) {
-    if (!AnyTwiddles<Real>::kCopy) return ntiles;
-    int dev = 0, sms = 1, per_sm = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, t.threads, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
-    return std::min(per_sm * sms, ntiles);
+    return AnyTwiddles<Real>::kCopy ? persistent_blocks(k, t.threads, smem, ntiles) : ntiles;
 }
 
 template <typename Real>

@@ -24,6 +24,7 @@ import numpy as np
 
 from . import _lib
 from . import densities as D
+from .api import _stream_handle, _torch
 
 CANDIDATES = (32, 48, 64, 80, 96, 128, 160, 192, 256, 320, 384, 512)
 NPTS = 1024          # grid points per (density, N) where the error is measured
@@ -31,17 +32,12 @@ BOX = 16.0           # selector workload box [-16, 16]^3
 FEATURES = 64
 
 
-def _torch():
-    import torch
-    return torch
-
-
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream():
-    return ctypes.c_void_p(_torch().cuda.current_stream().cuda_stream)
+    return _stream_handle(None)
 
 
 def gaussian_params(g):
@@ -182,15 +178,18 @@ class Network:
     def gradient(self, x, t):
         """Loss and parameter gradient (into self.grad) for inputs x and targets t."""
         torch = _torch()
-        B = x.shape[0]
-        acts = torch.empty(B * 3 * 64, dtype=torch.float32, device="cuda")
-        y = self.forward(x, acts)
-        dy = torch.empty_like(y)
+        B, K, lib, s = x.shape[0], self.K, self.lib, _stream()
+        # activations (B x 3 x 64), outputs and their gradient (B x K) in one buffer
+        work = torch.empty(B * (3 * 64 + 2 * K), dtype=torch.float32, device="cuda")
         loss = torch.empty(1, dtype=torch.float32, device="cuda")
-        _lib.check(self.lib.poisson_mlp_loss(_ptr(y), _ptr(t), y.numel(), _ptr(dy), _ptr(loss), _stream()),
-                   "poisson_mlp_loss")
-        _lib.check(self.lib.poisson_mlp_backward(_ptr(self.params), self.K, _ptr(x), _ptr(acts), B, _ptr(dy),
-                                                 _ptr(self.grad), _stream()), "poisson_mlp_backward")
+        acts, px = work.data_ptr(), x.data_ptr()
+        y = acts + 4 * B * 3 * 64
+        dy = y + 4 * B * K
+        params = self.params.data_ptr()
+        _lib.check(lib.poisson_mlp_forward(params, K, px, B, y, acts, s), "poisson_mlp_forward")
+        _lib.check(lib.poisson_mlp_loss(y, t.data_ptr(), B * K, dy, loss.data_ptr(), s), "poisson_mlp_loss")
+        _lib.check(lib.poisson_mlp_backward(params, K, px, acts, B, dy, self.grad.data_ptr(), s),
+                   "poisson_mlp_backward")
         return loss
 
     def train(self, x, t, epochs=3000, lr=2e-3):
