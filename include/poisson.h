@@ -142,8 +142,7 @@ int poisson_solve(poisson_plan p, const void *rho_d, void *u_d, void *stream);
  * and synchronises the stream before returning.  rho_h, u_h: host pointers to N^3
  * values of the plan's dtype (pinned memory gives full copy bandwidth).  Uses the
  * plan's own device staging buffers.  Where N is a multiple of 8 (N >= 16) and the x and y
- * passes are separate launches (not the fused form, nor a runtime-length plan with small
- * planes), the copies run in 8 z-slabs on a copy stream of the plan,
+ * passes are separate launches (not the fused form, nor a plan with small planes), the copies run in 8 z-slabs on a copy stream of the plan,
  * overlapped with the x and y passes of the neighbouring slabs (those passes transform
  * each z-plane on its own); they start after the work already queued on `stream`.  The result is the
  * same, bit for bit, as poisson_solve's on device copies of the buffers.
@@ -198,8 +197,8 @@ int poisson_compare(const void *a_d, int a_dtype, const void *b_d, int b_dtype, 
  * forward + symbol + z inverse, y inverse, x inverse).  ms[5] receives them.  With the
  * fused x-y form (POISSON_KNOB_XY_FORM = 1) the forward x and y passes are one kernel,
  * timed in ms[0] with ms[1] = 0, and the inverse y and x passes are one kernel, timed in
- * ms[3] with ms[4] = 0; so are they in runtime-length plans whose planes are small enough for
- * one kernel per direction.  The call synchronises the stream.  Same arguments and aliasing
+ * ms[3] with ms[4] = 0; so are they in plans whose planes are small enough for one kernel per
+ * direction.  The call synchronises the stream.  Same arguments and aliasing
  * rules as poisson_solve.
  */
 int poisson_solve_timed(poisson_plan p, const void *rho_d, void *u_d, void *stream, float *ms);

@@ -68,6 +68,7 @@ bool n_any(int N) {
 
 void any_plan_tiles(DevicePlan &p) {
     const bool f32 = p.dtype == POISSON_F32;
+    p.plane_small = !p.any && plane_n_size(p.N, !f32);
     for (int df = 0; df < 2; ++df) {
         for (int q = 0; q < 3; ++q)
             p.any_tile[df][q] = any_tile(q == 0 ? p.n3[0] : 2 * p.n3[q], any_max_radix(df != 0), any_max_warps(f32), q == 0);
@@ -808,7 +809,7 @@ extern "C" int poisson_solve_host(poisson_plan p, const void *rho_h, void *u_h, 
     gsp::PtrArray in, out;
     one(in, p->stage_in);
     one(out, p->stage_out);
-    const bool fused = (p->dp.xyform == 1 && p->dp.sync != nullptr) || gsp::plane_on(p->dp);
+    const bool fused = (p->dp.xyform == 1 && p->dp.sync != nullptr) || gsp::plane_on(p->dp) || gsp::plane_n_plan(p->dp);
     if (fused || nz % kSlabs != 0 || nz < 2 * kSlabs) {
         if ((e = cudaMemcpyAsync(p->stage_in, rho_h, n, cudaMemcpyHostToDevice, s)) != cudaSuccess)
             return map_cuda(e);

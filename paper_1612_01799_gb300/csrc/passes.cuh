@@ -412,6 +412,151 @@ k_x_inverse(const Cx2<Real> *__restrict__ in, const PtrArray u, const Cx2<Real> 
     }
 }
 
+// ---- K1 + K2 and K4 + K5 of small planes -------------------------------------------------------
+// One CTA takes a whole z-plane through the x and the y pass in shared memory, with the steps
+// of k_x_forward, k_col_tma and k_x_inverse (bit for bit their results): the x spectrum never
+// leaves the SM and a solve takes three launches instead of five.  Bound by latency, five block
+// barriers per direction (solves, separate passes and this: FP32 N = 16 13.2 and 7.4 us, 32 12.8
+// and 8.4, 48 17.2 and 12.9; double-float 16 15.6 and 12.0, 32 21.1 and 18.3).  Thread t serves row t mod N (x) and column group t mod GY (y); threads
+// beyond either's count work on a spare row or group so that all meet the barriers.
+template <typename Real, int N> struct PlaneN {
+    static constexpr int W = Types<Real>::W, L = 2 * N;
+    static constexpr int EX = Cfg<Real, N>::E, EY = Cfg<Real, L>::E;
+    static constexpr int GY = (N + W) / W;                            // groups of the N + 1 columns
+    static constexpr int NX = N * (N / EX), NY = GY * (L / EY);       // threads at work in x and y
+    static constexpr int NT = ((NX > NY ? NX : NY) + 31) / 32 * 32;
+    static constexpr int SX = (N + 1) | 1, SY = GY + 1;               // pitches, with the spare row / group
+    static constexpr int X_BYTES = (N + 1) * SX * (int)sizeof(typename Types<Real>::CS);
+    static constexpr int OFF_Y = (X_BYTES + 15) / 16 * 16;
+    static constexpr int SMEM = OFF_Y + L * SY * 16;
+    static constexpr bool ok = plane_n_size(N, !std::is_same<Real, float>::value);
+    static_assert(!ok || (NT <= 1024 && SMEM <= 227 * 1024), "threads and shared memory of one CTA");
+};
+// Element (y, k) of the plane's column layout.
+__device__ __forceinline__ void plane_el_st(CV *yb, int at, int k, CF x) {
+    float *p = reinterpret_cast<float *>(yb + at + (k >> 1)) + (k & 1);
+    sm_st(p, x.re);
+    sm_st(p + 2, x.im);
+}
+__device__ __forceinline__ CF plane_el_ld(const CV *yb, int at, int k) {
+    const float *p = reinterpret_cast<const float *>(yb + at + (k >> 1)) + (k & 1);
+    return {sm_ld(p), sm_ld(p + 2)};
+}
+template <typename C> __device__ __forceinline__ void plane_el_st(C *yb, int at, int k, C x) { sm_st(yb + at + k, x); }
+template <typename C> __device__ __forceinline__ C plane_el_ld(const C *yb, int at, int k) { return sm_ld(yb + at + k); }
+
+template <typename Real, int N>
+__global__ void __launch_bounds__(PlaneN<Real, N>::NT)
+k_plane_n_fwd(const PtrArray rho, Cx2<Real> *__restrict__ w2, const Cx2<Real> *__restrict__ tw,
+              const typename TwOf<typename Types<Real>::CC>::T *__restrict__ twc, int Px) {
+    using C = typename Types<Real>::CS;
+    using CC = typename Types<Real>::CC;
+    using X2 = Ext2<Real>;
+    using P = PlaneN<Real, N>;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    C *sm = reinterpret_cast<C *>(smraw);  // (N + 1) x SX
+    CC *yb = reinterpret_cast<CC *>(smraw + P::OFF_Y);
+    griddep_wait();
+    const int t = threadIdx.x, b = blockIdx.x / N, z = blockIdx.x - b * N;
+    const X2 *src = reinterpret_cast<const X2 *>(rho.p[b]) + (long long)z * N * (N / 2);
+#pragma unroll
+    for (int e = t; e < N * (N / 2); e += P::NT) {
+        const X2 f = __ldg(src + e);
+        sm_st(sm + (e % (N / 2)) * P::SX + e / (N / 2), C{f.x, f.y});
+    }
+    __syncthreads();
+    {
+        const int c = t < P::NX ? t % N : N, q = t < P::NX ? t / N : 0;
+        C v[P::EX];
+        constexpr RunOpt opt{false, true, false, false, true};
+        Stages<C, N, P::EX, -1, 1, typename Cfg<Real, N>::Rs>::template run<opt>(
+            v, q, c, sm, P::SX, tw, 2, [&](int row) { return sm_ld(sm + row * P::SX + c); },
+            [&](int row, C x) { sm_st(sm + row * P::SX + c, x); });
+    }
+    __syncthreads();
+    for (int e = t; e < N * (N / 2 + 1); e += P::NT) {  // the Hermitian split of k_x_forward
+        const int r = e % N, k = e / N;
+        const C ck = sm_ld(sm + k * P::SX + r), cn = sm_ld(sm + ((N - k) % N) * P::SX + r);
+        const C ev = {(Real)0.5 * (ck.re + cn.re), (Real)0.5 * (ck.im - cn.im)};
+        const C od = {(Real)0.5 * (ck.im + cn.im), (Real)0.5 * (cn.re - ck.re)};
+        if (k == 0) {
+            plane_el_st(yb, r * P::SY, 0, C{ev.re + od.re, (Real)0});
+            plane_el_st(yb, r * P::SY, N, C{ev.re - od.re, (Real)0});
+            if (P::W == 2) plane_el_st(yb, r * P::SY, N + 1, C{(Real)0, (Real)0});
+        } else {
+            const C wo = twmul<-1>(od, __ldg(tw + k));
+            plane_el_st(yb, r * P::SY, k, cadd(ev, wo));
+            if (2 * k != N) {
+                const C d = csub(ev, wo);
+                plane_el_st(yb, r * P::SY, N - k, C{d.re, -d.im});
+            }
+        }
+    }
+    __syncthreads();
+    const bool on = t < P::NY;
+    const int g = on ? t % P::GY : P::GY, q = on ? t / P::GY : 0;
+    Cx2<Real> *dst = w2 + (long long)blockIdx.x * P::L * Px + P::W * g;
+    CC v[P::EY];
+    constexpr RunOpt opt{false, true, false, false, false};
+    Stages<CC, P::L, P::EY, -1, 1, typename Cfg<Real, P::L>::Rs>::template run<opt>(
+        v, q, g, yb, P::SY, twc, 1, [&](int row) { return sm_ld(yb + row * P::SY + g); },
+        [&](int row, CC x) {
+            if (on) st_cc(dst + (long long)row * Px, x);
+        });
+}
+
+template <typename Real, int N>
+__global__ void __launch_bounds__(PlaneN<Real, N>::NT)
+k_plane_n_inv(const Cx2<Real> *__restrict__ w3, const PtrArray u, const Cx2<Real> *__restrict__ tw,
+              const typename TwOf<typename Types<Real>::CC>::T *__restrict__ twc, int Px) {
+    using C = typename Types<Real>::CS;
+    using CC = typename Types<Real>::CC;
+    using X2 = Ext2<Real>;
+    using P = PlaneN<Real, N>;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    C *sm = reinterpret_cast<C *>(smraw);
+    CC *yb = reinterpret_cast<CC *>(smraw + P::OFF_Y);
+    griddep_wait();
+    const int t = threadIdx.x, b = blockIdx.x / N, z = blockIdx.x - b * N;
+    {
+        const bool on = t < P::NY;
+        const int g = on ? t % P::GY : P::GY, q = on ? t / P::GY : 0;
+        const Cx2<Real> *src = w3 + (long long)blockIdx.x * P::L * Px + P::W * g;
+        CC v[P::EY];
+        constexpr RunOpt opt{false, false, false, true, true};
+        Stages<CC, P::L, P::EY, 1, 1, typename Cfg<Real, P::L>::Rs>::template run<opt>(
+            v, q, g, yb, P::SY, twc, 1,
+            [&](int row) { return on ? ld_cc(src + (long long)row * Px) : czero<CC>(); },
+            [&](int row, CC x) { sm_st(yb + row * P::SY + g, x); });
+    }
+    __syncthreads();
+    for (int e = t; e < N * (N / 2 + 1); e += P::NT) {  // the combination of k_x_inverse
+        const int r = e % N, k = e / N;
+        const C yk = plane_el_ld(yb, r * P::SY, k), yn = plane_el_ld(yb, r * P::SY, N - k);
+        if (k == 0) {
+            sm_st(sm + r, C{yk.re + yn.re, yk.re - yn.re});
+        } else {
+            const C ev = {yk.re + yn.re, yk.im - yn.im};
+            const C od = twmul<1>(C{yk.re - yn.re, yk.im + yn.im}, __ldg(tw + k));
+            sm_st(sm + k * P::SX + r, add_rot<1>(ev, od));
+            if (2 * k != N) sm_st(sm + (N - k) * P::SX + r, add_rot<1>(C{ev.re, -ev.im}, C{od.re, -od.im}));
+        }
+    }
+    __syncthreads();
+    {
+        const int c = t < P::NX ? t % N : N, q = t < P::NX ? t / N : 0;
+        C v[P::EX];
+        constexpr RunOpt opt{false, false, false, true, true};
+        Stages<C, N, P::EX, 1, 1, typename Cfg<Real, N>::Rs>::template run<opt>(
+            v, q, c, sm, P::SX, tw, 2, [&](int row) { return sm_ld(sm + row * P::SX + c); },
+            [&](int row, C x) { sm_st(sm + row * P::SX + c, x); });
+    }
+    __syncthreads();
+    X2 *dst = reinterpret_cast<X2 *>(const_cast<void *>(u.p[b])) + (long long)z * N * (N / 2);
+#pragma unroll
+    for (int e = t; e < N * (N / 2); e += P::NT) dst[e] = c_ext(sm_ld(sm + (e % (N / 2)) * P::SX + e / (N / 2)));
+}
+
 // ---- symbol octant (setup, FP64 arithmetic) ---------------------------------------------
 // sym[(kz * (N+1) + ky) * Ps + kx] for kx, ky, kz <= N; the pitch Ps (a multiple of 4)
 // keeps the two-column loads of the FP32 z pass aligned.
@@ -757,6 +902,34 @@ cudaError_t xy_pass(const DevicePlan &p, const PtrArray &rho, const PtrArray &u,
     return cudaErrorInvalidValue;
 }
 
+// Whether the x and y passes of B densities run as one kernel per direction (k_plane_n_*).  In
+// the wider arithmetics many planes are better off in the separate passes, whose CTAs are more
+// and smaller (double-float, 16 densities of N = 32: 61 us against 63 us); the bits are the same.
+template <typename Real, int N> bool plane_n_on(const DevicePlan &p, int B) {
+    return PlaneN<Real, N>::ok && plane_n_plan(p) && (std::is_same<Real, float>::value || B * N <= 304);
+}
+template <typename Real, int N>
+cudaError_t plane_n(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int B, cudaStream_t s, bool fwd) {
+    if constexpr (PlaneN<Real, N>::ok) {
+        using P = PlaneN<Real, N>;
+        using T2 = Cx2<Real>;
+        using TwC = typename TwOf<typename Types<Real>::CC>::T;
+        const T2 *tw = static_cast<const T2 *>(p.tw);
+        const TwC *twc = static_cast<const TwC *>(p.twc);
+        if (fwd) {
+            GSP_CHECK(set_smem(k_plane_n_fwd<Real, N>, P::SMEM));
+            GSP_CHECK(launch_pdl(k_plane_n_fwd<Real, N>, B * N, P::NT, P::SMEM, s, rho, static_cast<T2 *>(p.w2), tw, twc,
+                                 p.Px));
+        } else {
+            GSP_CHECK(set_smem(k_plane_n_inv<Real, N>, P::SMEM));
+            GSP_CHECK(launch_pdl(k_plane_n_inv<Real, N>, B * N, P::NT, P::SMEM, s, static_cast<const T2 *>(p.w3), u, tw,
+                                 twc, p.Px));
+        }
+        return cudaGetLastError();
+    }
+    return cudaErrorInvalidValue;
+}
+
 // The x and y passes of planes z0 .. z0 + nz - 1 of one density (rho and u device
 // pointers to the whole density): forward x then y, or inverse y then x, with the kernels
 // of the plan's separate x and y forms on that slab of planes only.
@@ -786,22 +959,25 @@ cudaError_t solve_n(const DevicePlan &p, const PtrArray &rho, const PtrArray &u,
                     cudaEvent_t *ev, double *tail, int skip) {
     const bool fused = xy_fused_on<Real, N>(p);
     if (fused && skip) return cudaErrorInvalidValue;
+    const bool plane = !skip && plane_n_on<Real, N>(p, B);
     if (ev) GSP_CHECK(cudaEventRecord(ev[0], s));
     if (fused) GSP_CHECK((xy_pass<Real, N>(p, rho, u, B, s, true)));
+    else if (plane) GSP_CHECK((plane_n<Real, N>(p, rho, u, B, s, true)));
     else if (!(skip & 1)) GSP_CHECK((x_pass<Real, N>(p, rho, u, B, s, true)));
     if (ev) GSP_CHECK(cudaEventRecord(ev[1], s));
 
-    if (!fused && !(skip & 1)) GSP_CHECK((y_pass<Real, N>(p, B, s, true)));
+    if (!fused && !plane && !(skip & 1)) GSP_CHECK((y_pass<Real, N>(p, B, s, true)));
     if (ev) GSP_CHECK(cudaEventRecord(ev[2], s));
 
     GSP_CHECK((z_pass<Real, N>(p, B, s, tail)));
     if (ev) GSP_CHECK(cudaEventRecord(ev[3], s));
 
     if (fused) GSP_CHECK((xy_pass<Real, N>(p, rho, u, B, s, false)));
+    else if (plane) GSP_CHECK((plane_n<Real, N>(p, rho, u, B, s, false)));
     else if (!(skip & 2)) GSP_CHECK((y_pass<Real, N>(p, B, s, false)));
     if (ev) GSP_CHECK(cudaEventRecord(ev[4], s));
 
-    if (!fused && !(skip & 2)) GSP_CHECK((x_pass<Real, N>(p, rho, u, B, s, false)));
+    if (!fused && !plane && !(skip & 2)) GSP_CHECK((x_pass<Real, N>(p, rho, u, B, s, false)));
     if (ev) GSP_CHECK(cudaEventRecord(ev[5], s));
     return cudaSuccess;
 }

@@ -49,6 +49,9 @@ struct DevicePlan {
     void *tw3[3] = {nullptr, nullptr, nullptr};
     // Tiles of the runtime-length passes along x, y and z, per arithmetic (any_plan_tiles).
     AnyTile any_tile[2][3] = {};
+    // Compiled-length plans with small planes: the x and y passes in one kernel per direction
+    // (the allocation-free solve leaves it false).
+    bool plane_small = false;
     // The x and y passes as one kernel per direction (passes_plane.cuh), per arithmetic: on for
     // runtime-length plans whose planes are small (plane_on).
     PlaneTile plane[2] = {};
@@ -105,6 +108,13 @@ bool n_supported(int N);
 void any_plan_tiles(DevicePlan &p);
 // Whether p's solves run the plane kernels in its present arithmetic.
 inline bool plane_on(const DevicePlan &p) { return p.plane[p.arith].on; }
+// Compiled-length plans: the sizes of the plane kernels (at N = 64 in FP32 they and the separate
+// passes take 20 us, twelve densities 116 and 91 us; double-float N = 48 41.6 and 35.3 us), and
+// whether p's solves run them: with the block forms of both passes.
+__host__ __device__ constexpr bool plane_n_size(int N, bool wide) { return N == 16 || N == 32 || (N == 48 && !wide); }
+inline bool plane_n_plan(const DevicePlan &p) {
+    return p.plane_small && p.xform == 0 && p.yform == 0 && p.xyform == 0;
+}
 
 // Record a failed CUDA call for poisson_last_cuda_error() (per host thread).
 void note_cuda_error(cudaError_t e);

@@ -282,3 +282,31 @@ def test_degenerate_inputs_and_invariants(torch_cuda, N, dtype, forms):
         assert float((uq.double() - 4.0 * u1.double()).norm() / (4.0 * u1.double()).norm()) <= eps_method
         p.last_status()
         q.last_status()
+
+
+@pytest.mark.parametrize("N,dtype,count", [(16, "f32", 3), (32, "f32", 3), (48, "f32", 2), (16, "f64", 20),
+                                           (32, "f64", 10)])
+def test_plane_kernels_equal_separate_passes(torch_cuda, N, dtype, count):
+    """Small compiled sizes take the x and y passes of a plane in one kernel per direction: the
+    bits of the separate passes, which run the slabs of a slab decomposition (its inverse here
+    from the solve's own z output) and, in the wider arithmetics, batches of more than 304
+    planes."""
+    from paper_1612_01799_gb300 import Plan, solve_batched
+    torch = torch_cuda
+    rng = np.random.default_rng(N)
+    with Plan(N, 8.0, 1e-6 if dtype == "f32" else 1e-12, dtype, max_batch=count) as p:
+        for ar in ([None] if dtype == "f32" else ["df", "f64"]):
+            if ar:
+                p.arith = ar
+            rhos = [torch.from_numpy(rng.uniform(-1, 1, (N, N, N)).astype(p.np_dtype)).cuda() for _ in range(count)]
+            outs = solve_batched([p] * count, rhos, [torch.empty_like(r) for r in rhos])
+            for r, o in zip(rhos, outs):
+                assert torch.equal(p.solve(r), o), ar
+            ms = p.solve_timed(rhos[0], outs[0])
+            assert ms[0] > 0 and ms[3] > 0 and ms[1] < 0.02 and ms[4] < 0.02
+            u = torch.empty_like(rhos[0])
+            p.solve(rhos[0], out=outs[0])
+            assert p._lib.poisson_slab_inverse(p.handle, u.data_ptr(), 0, N, None) == 0
+            torch.cuda.synchronize()
+            assert torch.equal(u, outs[0])
+        p.last_status()
