@@ -386,10 +386,10 @@ template <int R, int D, typename C> __device__ __forceinline__ void dft(C *a) {
         dft4<D>(a[0], a[1], a[2], a[3]);
     } else if constexpr (R == 5) {
         dft5<D>(a[0], a[1], a[2], a[3], a[4]);
-    } else if constexpr (R == 6 || R == 10 || R == 12) {
+    } else if constexpr (R == 6 || R == 10 || R == 12 || R == 20) {
         // Good-Thomas: R = A B with A, B coprime, input (B i + A j) mod R, output k with
         // k = p mod A and k = q mod B; no twiddles between the two DFTs.
-        constexpr int B = R == 10 ? 5 : 3, A = R / B;
+        constexpr int B = R % 5 == 0 ? 5 : 3, A = R / B;
         C t[A][B];
 #pragma unroll
         for (int i = 0; i < A; ++i) {
@@ -406,8 +406,8 @@ template <int R, int D, typename C> __device__ __forceinline__ void dft(C *a) {
 #pragma unroll
             for (int p = 0; p < A; ++p) {
                 // the k < R with k = p mod A, k = q mod B
-                constexpr int eA = R == 6 ? 3 : R == 10 ? 5 : 9;  // 1 mod A, 0 mod B
-                constexpr int eB = R == 6 ? 4 : R == 10 ? 6 : 4;  // 0 mod A, 1 mod B
+                constexpr int eA = R == 6 ? 3 : R == 12 ? 9 : 5;  // 1 mod A, 0 mod B
+                constexpr int eB = R == 10 ? 6 : R == 20 ? 16 : 4;  // 0 mod A, 1 mod B
                 a[(eA * p + eB * q) % R] = u[p];
             }
         }

@@ -71,7 +71,9 @@ GSP_FFT_CFG(2048, 16, 16, 16, 8);
 // The schedule a pass uses for its arithmetic: FftCfg, except in double-float, whose
 // butterflies are about ten times longer in instructions: there the lengths that FftCfg
 // does in radix 16 (16 values per thread) run in radices 8 and 4 with 8 values per thread
-// (and 96, 384 and 768 with 12), so that a kernel's code stays within the instruction cache.
+// (and 96, 384 and 768 with 12), so that a kernel's code stays within the instruction cache;
+// 48 keeps three stages, and 320 takes 4, 20, 4, a twiddle less per value (solve at N = 160
+// 716 -> 658 us; in FP32 the warp forms beat either).
 template <typename Real, int L> struct Cfg : FftCfg<L> {};
 #define GSP_DF_CFG(LL, EE, ...)                  \
     template <> struct Cfg<DF, LL> {             \
@@ -82,6 +84,7 @@ GSP_DF_CFG(16, 4, 4, 4);
 GSP_DF_CFG(48, 12, 4, 3, 4);
 GSP_DF_CFG(128, 8, 8, 4, 4);
 GSP_DF_CFG(256, 8, 8, 8, 4);
+GSP_DF_CFG(320, 20, 4, 20, 4);
 GSP_DF_CFG(384, 12, 4, 4, 6, 4);
 GSP_DF_CFG(512, 8, 8, 8, 8);
 GSP_DF_CFG(768, 12, 4, 12, 4, 4);
