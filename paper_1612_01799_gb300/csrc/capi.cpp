@@ -790,8 +790,19 @@ extern "C" int poisson_solve(poisson_plan p, const void *rho_d, void *u_d, void 
     return map_cuda(gsp::launch_solve(p->dp, in, out, 1, (cudaStream_t)stream, nullptr));
 }
 
-// Slabs of the host-buffer solve's copy / x-pass pipeline.
-constexpr int kSlabs = 8;
+// Slabs of the host-buffer solve's copy / x-pass pipeline, in eighths of the volume.  FP32, whose
+// x and y passes take a third of a slab's copy: few copies, graded so that little work follows
+// the last one in and precedes the first one out (N = 256 946 -> 929 us against equal slabs).  The
+// wider arithmetics, whose passes take as long as the copies: equal slabs (N = 160 906 us,
+// graded 925).  Below kHostPipelineBytes the launches cost more than the overlap gains: one
+// copy each way (FP32 N = 64 54 us against 135, N = 128 172 against 182 graded; N = 160, 16 MB, 325
+// against 300).
+constexpr size_t kHostPipelineBytes = (size_t)12 << 20;
+struct HostSlabs {
+    int n, in[8], out[8];
+};
+static const HostSlabs kEqual = {8, {1, 1, 1, 1, 1, 1, 1, 1}, {1, 1, 1, 1, 1, 1, 1, 1}};
+static const HostSlabs kGraded = {4, {4, 2, 1, 1}, {1, 1, 2, 4}};
 
 extern "C" int poisson_solve_host(poisson_plan p, const void *rho_h, void *u_h, void *stream) {
     int rc = check_solve_args(p, rho_h, u_h);
@@ -810,7 +821,7 @@ extern "C" int poisson_solve_host(poisson_plan p, const void *rho_h, void *u_h, 
     one(in, p->stage_in);
     one(out, p->stage_out);
     const bool fused = (p->dp.xyform == 1 && p->dp.sync != nullptr) || gsp::plane_on(p->dp) || gsp::plane_n_plan(p->dp);
-    if (fused || nz % kSlabs != 0 || nz < 2 * kSlabs) {
+    if (fused || n < kHostPipelineBytes || nz % 8 != 0) {
         if ((e = cudaMemcpyAsync(p->stage_in, rho_h, n, cudaMemcpyHostToDevice, s)) != cudaSuccess)
             return map_cuda(e);
         if ((e = gsp::launch_solve(p->dp, in, out, 1, s, nullptr)) != cudaSuccess) return map_cuda(e);
@@ -831,9 +842,10 @@ extern "C" int poisson_solve_host(poisson_plan p, const void *rho_h, void *u_h, 
         p->have_slab_events = true;
     }
     cudaStream_t cs = p->copy_stream;
-    cudaEvent_t *ev_in = p->slab_ev, *ev_out = p->slab_ev + kSlabs, start = p->slab_ev[2 * kSlabs];
-    const int nzs = nz / kSlabs;  // planes per slab
-    const size_t sb = (size_t)nzs * ny * nx * p->elem;
+    const HostSlabs &hs = p->dp.dtype == POISSON_F32 ? kGraded : kEqual;
+    cudaEvent_t *ev_in = p->slab_ev, *ev_out = p->slab_ev + 8, start = p->slab_ev[16];
+    const int unit = nz / 8;  // planes of an eighth
+    const size_t plane = (size_t)ny * nx * p->elem;
     // On an error part of the pipeline may already be queued: wait for both streams so
     // that no copy into or out of the staging buffers outlives the call.
     auto fail = [&](cudaError_t err) {
@@ -845,23 +857,27 @@ extern "C" int poisson_solve_host(poisson_plan p, const void *rho_h, void *u_h, 
     // staging buffers).
     if ((e = cudaEventRecord(start, s)) != cudaSuccess || (e = cudaStreamWaitEvent(cs, start, 0)) != cudaSuccess)
         return map_cuda(e);
-    for (int k = 0; k < kSlabs; ++k) {
-        e = cudaMemcpyAsync(static_cast<char *>(p->stage_in) + k * sb, static_cast<const char *>(rho_h) + k * sb, sb,
-                            cudaMemcpyHostToDevice, cs);
+    for (int k = 0, z0 = 0; k < hs.n; ++k) {
+        const int nzs = hs.in[k] * unit;
+        e = cudaMemcpyAsync(static_cast<char *>(p->stage_in) + z0 * plane, static_cast<const char *>(rho_h) + z0 * plane,
+                            nzs * plane, cudaMemcpyHostToDevice, cs);
         if (e == cudaSuccess) e = cudaEventRecord(ev_in[k], cs);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev_in[k], 0);
-        if (e == cudaSuccess) e = gsp::launch_xy_slab(p->dp, p->stage_in, p->stage_out, k * nzs, nzs, s, true);
+        if (e == cudaSuccess) e = gsp::launch_xy_slab(p->dp, p->stage_in, p->stage_out, z0, nzs, s, true);
         if (e != cudaSuccess) return fail(e);
+        z0 += nzs;
     }
     if ((e = gsp::launch_solve(p->dp, in, out, 1, s, nullptr, nullptr, 3)) != cudaSuccess) return fail(e);
-    for (int k = 0; k < kSlabs; ++k) {
-        e = gsp::launch_xy_slab(p->dp, p->stage_in, p->stage_out, k * nzs, nzs, s, false);
+    for (int k = 0, z0 = 0; k < hs.n; ++k) {
+        const int nzs = hs.out[k] * unit;
+        e = gsp::launch_xy_slab(p->dp, p->stage_in, p->stage_out, z0, nzs, s, false);
         if (e == cudaSuccess) e = cudaEventRecord(ev_out[k], s);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, ev_out[k], 0);
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(static_cast<char *>(u_h) + k * sb, static_cast<char *>(p->stage_out) + k * sb, sb,
-                                cudaMemcpyDeviceToHost, cs);
+            e = cudaMemcpyAsync(static_cast<char *>(u_h) + z0 * plane, static_cast<char *>(p->stage_out) + z0 * plane,
+                                nzs * plane, cudaMemcpyDeviceToHost, cs);
         if (e != cudaSuccess) return fail(e);
+        z0 += nzs;
     }
     // `stream` waits for the last copy, so that work issued after the call is ordered
     // after it, then the call returns once everything has finished.

@@ -183,12 +183,13 @@ def test_batched_host_and_checked(torch_cuda):
     assert eta.value == pytest.approx(ref, rel=2e-3, abs=1e-12)
 
 
-def test_slab_host_solve_box(torch_cuda):
-    """poisson_solve_host's slab pipeline (nz a multiple of 8) on a box with different counts."""
+@pytest.mark.parametrize("n,dtype", [((24, 40, 32), "f32"), ((200, 162, 96), "f32"), ((200, 160, 48), "f64")])
+def test_slab_host_solve_box(torch_cuda, n, dtype):
+    """poisson_solve_host on boxes with different counts: one copy each way, and the slab
+    pipeline (12 MB or more, nz a multiple of 8) with graded and with equal slabs."""
     from paper_1612_01799_gb300 import Plan
-    n = (24, 40, 32)
-    rho = np.random.default_rng(4).uniform(-1, 1, (n[2], n[1], n[0])).astype(np.float32)
-    with Plan(n, (1.0, 2.0, 1.5), 1e-6, "f32") as p:
+    rho = np.random.default_rng(4).uniform(-1, 1, (n[2], n[1], n[0])).astype(np.float32 if dtype == "f32" else np.float64)
+    with Plan(n, (1.0, 2.0, 1.5), 1e-6, dtype) as p:
         dev = run(torch_cuda, p, rho)
         host = p.solve_host(rho)
     assert np.array_equal(host.astype(np.float64).reshape(dev.shape), dev)

@@ -193,9 +193,9 @@ def test_device_errors_are_codes(torch_cuda):
 @pytest.mark.parametrize("N,dtype,xyform", [(256, "f32", 0), (256, "f32", 1), (48, "f32", 0), (80, "f64", 0),
                                             (128, "f64", 0), (8, "f32", 0), (512, "f32", 0)])
 def test_host_solve_slab_pipeline(torch_cuda, N, dtype, xyform):
-    """poisson_solve_host on pinned buffers: the slab pipeline (copies of 8 z-slabs
-    overlapped with the x passes; N a multiple of 8, N >= 16, separate x and y passes) and
-    the plain path (N = 8, or the fused x-y form) give the device solve's bits."""
+    """poisson_solve_host on pinned buffers: the slab pipeline (copies of z-slabs overlapped
+    with the x and y passes; 12 MB or more, N a multiple of 8, separate x and y passes) and
+    the plain path (smaller arrays, or the fused x-y form) give the device solve's bits."""
     from paper_1612_01799_gb300 import Plan
     torch = torch_cuda
     L = 10.0
