@@ -27,16 +27,16 @@ struct AnySched {
 };
 // The schedule of the even 5-smooth length L >= 4 with radices 2, 3, 4, 5, 6, 8, 9, 10 and 12
 // up to max_radix: at least two and otherwise the fewest stages, among those the smallest sum
-// of the radices.  First (its stage skips the padding's zeros) an 8, whose zero-skipping form
-// has the fewest products to round, or the largest even radix; last the smallest of the
+// of the radices.  First (its stage skips the padding's zeros) a 4 or an 8, whose zero-skipping
+// forms have the fewest products to round, or the largest even radix; last the smallest of the
 // others, at most max_last.  nst = 0 if there is none.
 inline AnySched any_sched(int L, int max_radix, int max_last, bool pad) {
     static const int kRadix[] = {12, 10, 9, 8, 6, 5, 4, 3, 2};
     // Which of the n non-increasing radices goes first, or -1 if none can.
     auto first_of = [&](const int *f, int n) {
-        const int i8 = (int)(std::find(f, f + n, 8) - f);
+        const int i4 = (int)(std::find(f, f + n, 4) - f), i8 = (int)(std::find(f, f + n, 8) - f);
         const int even = (int)(std::find_if(f, f + n, [](int v) { return v % 2 == 0; }) - f);
-        for (int i : {i8, even})
+        for (int i : {i4, i8, even})
             if (i < n && f[i == n - 1 ? n - 2 : n - 1] <= max_last) return i;
         return -1;
     };
