@@ -73,8 +73,9 @@ void any_plan_tiles(DevicePlan &p) {
         for (int q = 0; q < 3; ++q)
             p.any_tile[df][q] = any_tile(q == 0 ? p.n3[0] : 2 * p.n3[q], any_max_radix(df != 0), any_max_warps(f32), q == 0);
         p.plane[df] = plane_tile(p.n3[0], p.n3[1], any_max_radix(df != 0), f32 ? 2 : 1);
-        p.plane[df].on = p.plane[df].on && p.any;
+        p.plane[df].on = p.plane[df].on && p.any && !(n_supported(p.n3[0]) && n_supported(p.n3[1]));
     }
+    for (int q = 0; q < 3; ++q) p.axn[q] = p.any && n_supported(p.n3[q]) ? p.n3[q] : 0;
 }
 
 cudaError_t launch_solve(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int count,
@@ -439,10 +440,19 @@ extern "C" int poisson_plan_create_box_n(poisson_plan *out, int nx, int ny, int 
 // Twiddles W_{2N}^e from FP64 (long double arithmetic) into the plan's tables, in its
 // arithmetic's format: FP32 rounded once (and the column passes' (re, re, im, im) copy), FP64,
 // or double-float (re.hi, re.lo, im.hi, im.lo) split from the FP64 value.
-static cudaError_t upload_table(void *dst, int n2, int dtype, int arith) {
+// broadcast: FP32 as the column passes' (re, re, im, im).
+static cudaError_t upload_table(void *dst, int n2, int dtype, int arith, bool broadcast = false) {
     std::vector<double> tw;
     gsp::twiddles(n2, tw);
     const size_t n = (size_t)n2;
+    if (dtype == POISSON_F32 && broadcast) {
+        std::vector<float> tw4(n * 4);
+        for (size_t i = 0; i < n; ++i) {
+            tw4[4 * i] = tw4[4 * i + 1] = (float)tw[2 * i];
+            tw4[4 * i + 2] = tw4[4 * i + 3] = (float)tw[2 * i + 1];
+        }
+        return cudaMemcpy(dst, tw4.data(), n * 4 * sizeof(float), cudaMemcpyHostToDevice);
+    }
     if (dtype == POISSON_F32) {
         std::vector<float> twf(tw.begin(), tw.end());
         return cudaMemcpy(dst, twf.data(), n * 2 * sizeof(float), cudaMemcpyHostToDevice);
@@ -462,6 +472,10 @@ static cudaError_t upload_twiddles(poisson_plan p) {
         // W_{2 n_q}^e of each axis, in the arithmetic's storage.
         for (int q = 0; q < 3; ++q) {
             cudaError_t e = upload_table(p->dp.tw3[q], 2 * p->dp.n3[q], p->dp.dtype, p->dp.arith);
+            if (e != cudaSuccess) return e;
+        }
+        for (int q = 1; q < 3 && p->dp.dtype == POISSON_F32; ++q) {
+            cudaError_t e = upload_table(p->dp.twc3[q - 1], 2 * p->dp.n3[q], p->dp.dtype, 0, true);
             if (e != cudaSuccess) return e;
         }
         return cudaSuccess;
@@ -537,7 +551,7 @@ static int plan_create_impl(poisson_plan *out, const int *n3, double L, const do
     // copy); the runtime-length forms one table W_{2 n_q} per axis (double-float: 16 bytes
     // per entry, as FP64).
     const size_t tw_bytes = any ? (size_t)2 * (nx + ny + nz) * cx : (size_t)2 * N * cx;
-    const size_t twc_bytes = dtype == POISSON_F32 && !any ? (size_t)2 * N * 4 * sizeof(float) : 0;
+    const size_t twc_bytes = dtype == POISSON_F32 ? (size_t)2 * (any ? ny + nz : N) * 4 * sizeof(float) : 0;
     const size_t w1_bytes = (size_t)max_batch * nz * ny * p->dp.Px * cx;
     const size_t w2_bytes = (size_t)max_batch * nz * 2 * ny * p->dp.Px * cx;
     p->ws_bytes = w1_bytes + 2 * w2_bytes;  // for max_batch densities
@@ -568,6 +582,11 @@ static int plan_create_impl(poisson_plan *out, const int *n3, double L, const do
         if ((e = cudaMalloc(&p->dp.twc, twc_bytes)) != cudaSuccess) return fail(e);
     } else {
         p->dp.twc = p->dp.tw;
+    }
+    if (any) {
+        const bool f32 = twc_bytes != 0;
+        p->dp.twc3[0] = f32 ? p->dp.twc : p->dp.tw3[1];
+        p->dp.twc3[1] = f32 ? static_cast<char *>(p->dp.twc) + (size_t)2 * ny * 4 * sizeof(float) : p->dp.tw3[2];
     }
     // Padding columns (kx > N) are carried along by the two-column passes but never used;
     // zeroed once so they hold finite values.

@@ -197,7 +197,8 @@ k_col_tma(const __grid_constant__ CUtensorMap tin, Cx2<Real> *__restrict__ out,
 
 // ---- K3 ----------------------------------------------------------------------------------
 // Tile = (tx, ky, b): input z < N rows of density b in w2, symbol rows kz <= N of the
-// octant at |ky|, output z < N rows of density b in w3.
+// octant at |ky|, output z < N rows of density b in w3; nx and ny points on the other axes (N in
+// a cube).
 // Energy |F|^2 of the padded spectrum in the registers of one element (both lanes of CV),
 // weighted by column (kx = 0 and N once, 0 < kx < N twice for the mirrored -kx, kx > N
 // padding not at all).
@@ -217,7 +218,7 @@ __global__ void __launch_bounds__(tma_threads<Real, L, 1>(), min_blocks_for<tma_
 k_z_symbol_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tsym,
                Cx2<Real> *__restrict__ out,
                const typename TwOf<typename Types<Real>::CC>::T *__restrict__ tw, int ntx, int ntiles,
-               int ncols, int Px, int *__restrict__ status, double *__restrict__ tail) {
+               int nx, int ny, int Px, int *__restrict__ status, double *__restrict__ tail) {
     using C = typename Types<Real>::CC;
     using Lay = TmaLayout<Real, L, 1>;
     using Rs = typename Cfg<Real, L>::Rs;
@@ -234,7 +235,8 @@ k_z_symbol_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ 
     uint64_t *bar = reinterpret_cast<uint64_t *>(base + Lay::OFF_BAR);  // [0] input, [1] symbol
     constexpr int NG = Lay::NG;
     const int g = threadIdx.x % NG, q = threadIdx.x / NG;
-    const long long zs = (long long)L * Px;
+    const int Ly = 2 * ny;
+    const long long zs = (long long)Ly * Px;
 
     if (threadIdx.x == 0) {
         mbar_init(bar, 1);
@@ -242,23 +244,30 @@ k_z_symbol_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ 
         fence_mbar_init();
     }
     __syncthreads();
-    // Consecutive tiles take ky and its mirror 2N - ky, which read the same symbol rows.
-    auto ky_of = [&](int by) { return (by & 1) ? L - ((by + 1) >> 1) : (by >> 1); };
+    // Consecutive tiles take ky and its mirror 2 ny - ky, which read the same symbol rows.  Plans
+    // with several densities are cubes (Ly = L).
+    struct Tile {
+        int tx, ky, b;
+    };
+    auto tile_of = [&](int t) {
+        const int line = t / ntx, b = Ly == L ? line / L : 0, li = line - b * L;
+        return Tile{t - line * ntx, (li & 1) ? Ly - ((li + 1) >> 1) : li >> 1, b};
+    };
     auto issue_in = [&](int t) {
-        const int tx = t % ntx, ky = ky_of((t / ntx) % L), b = t / (ntx * L);
+        const Tile q = tile_of(t);
         mbar_arrive_expect_tx(bar, Lay::IN_BYTES);
 #pragma unroll
         for (int c = 0; c < Lay::NCP; ++c)
-            tma_load_3d(inb + c * Lay::RPC * Lay::ROWB, &tin, bar, tx * TCU, ky, b * N + c * Lay::RPC);
+            tma_load_3d(inb + c * Lay::RPC * Lay::ROWB, &tin, bar, q.tx * TCU, q.ky, q.b * N + c * Lay::RPC);
     };
     auto issue_sym = [&](int t) {
-        const int tx = t % ntx, ky = ky_of((t / ntx) % L);
-        const int kya = ky <= N ? ky : L - ky;
+        const Tile q = tile_of(t);
+        const int kya = q.ky <= ny ? q.ky : Ly - q.ky;
         mbar_arrive_expect_tx(bar + 1, Lay::S_BYTES);
 #pragma unroll
         for (int c = 0; c < Lay::NCS; ++c)
             tma_load_3d(reinterpret_cast<unsigned char *>(sb) + c * Lay::SRC * Lay::SROWB, &tsym, bar + 1,
-                        tx * TC, kya, c * Lay::SRC);
+                        q.tx * TC, kya, c * Lay::SRC);
     };
     int t = blockIdx.x;
     if (threadIdx.x == 0 && t < ntiles) {
@@ -267,9 +276,9 @@ k_z_symbol_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ 
     }
     uint32_t phase = 0;
     for (; t < ntiles; t += gridDim.x) {
-        const int tx = t % ntx, ky = ky_of((t / ntx) % L), bb = t / (ntx * L);
-        const int col = tx * TC + W * g;
-        const bool valid = col < ncols;
+        const Tile tile = tile_of(t);
+        const int ky = tile.ky, bb = tile.b, col = tile.tx * TC + W * g;
+        const bool valid = col <= nx;
         const bool more = t + (int)gridDim.x < ntiles;
         bool ok = mbar_wait(bar, phase, status);
         if (__syncthreads_or(!ok)) return;
@@ -286,13 +295,15 @@ k_z_symbol_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ 
         Stages<C, L, E, -1, 1, Rs>::template run<fwd>(
             v, q, g, xb, NG, tw, 1, [&](int) { return czero<C>(); }, [&](int, C) {});
         if constexpr (TAIL) {
-            const int kya = ky <= N ? ky : L - ky;
+            const int kya = ky <= ny ? ky : Ly - ky;
             constexpr int SHELL = N - N / 8;
+            const int shx = nx - nx / 8;
+            const bool shy = kya >= ny - ny / 8;
             float w[W], eshell = 0.f, etot = 0.f;
 #pragma unroll
             for (int i = 0; i < W; ++i) {
                 const int kx = col + i;
-                w[i] = kx > N || !valid ? 0.f : (kx == 0 || kx == N) ? 1.f : 2.f;
+                w[i] = kx > nx || !valid ? 0.f : (kx == 0 || kx == nx) ? 1.f : 2.f;
             }
 #pragma unroll
             for (int b = 0; b < E / RL; ++b) {
@@ -305,11 +316,11 @@ k_z_symbol_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ 
                     if constexpr (W == 2) {
                         const float2 en = cenergy(v[b * RL + r]);
                         e = w[0] * en.x + w[1] * en.y;
-                        if ((kz >= SHELL || kya >= SHELL) || col >= SHELL) eshell += e;
-                        else if (col + 1 >= SHELL) eshell += w[1] * en.y;
+                        if (kz >= SHELL || shy || col >= shx) eshell += e;
+                        else if (col + 1 >= shx) eshell += w[1] * en.y;
                     } else {
                         e = w[0] * cenergy(v[b * RL + r]);
-                        if (kz >= SHELL || kya >= SHELL || col >= SHELL) eshell += e;
+                        if (kz >= SHELL || shy || col >= shx) eshell += e;
                     }
                     etot += e;
                 }
@@ -347,7 +358,7 @@ k_z_symbol_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ 
             fence_proxy_async();
             issue_sym(t + gridDim.x);
         }
-        Cx2<Real> *dst = out + ((long long)bb * N * L + ky) * Px + col;
+        Cx2<Real> *dst = out + ((long long)bb * N * Ly + ky) * Px + col;
         constexpr RunOpt inv{true, false, false, true, false};
         Stages<C, L, E, 1, 1, Rv>::template run<inv>(
             v, q, g, xb, NG, tw, 1, [&](int) { return czero<C>(); },

@@ -43,10 +43,14 @@ struct DevicePlan {
     // Runtime-length forms (any = 1): the points per axis n3 = (nx, ny, nz), which may
     // differ; N = nx.  Their passes read the twiddles W_{2 n_q}^e of axis q from tw3[q]
     // (the dtype's storage: float2, double2, or double-float float4), the symbol as
-    // [kz <= nz][ky <= ny][kx < Ps], and use no TMA descriptors and no form knobs.
+    // [kz <= nz][ky <= ny][kx < Ps], and have no form knobs.
     int any = 0;
     int n3[3] = {0, 0, 0};
     void *tw3[3] = {nullptr, nullptr, nullptr};
+    // Axes whose count has a compiled schedule run the block forms along it: axn[q] = n_q, else 0,
+    // the y and z axes with the twiddles twc3[0] and twc3[1] in the column passes' form.
+    int axn[3] = {0, 0, 0};
+    void *twc3[2] = {nullptr, nullptr};
     // Tiles of the runtime-length passes along x, y and z, per arithmetic (any_plan_tiles).
     AnyTile any_tile[2][3] = {};
     // Compiled-length plans with small planes: the x and y passes in one kernel per direction

@@ -221,3 +221,34 @@ def test_plane_kernels(torch_cuda, n, dtype, plane):
         host = p.solve_host(rho.astype(p.np_dtype))
         assert torch.equal(p.solve(t, out=t), out)
         assert np.array_equal(host, out.cpu().numpy())
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("n", [(32, 20, 64), (20, 64, 30), (64, 48, 24), (16, 128, 80), (4, 8, 16)])
+def test_box_axes_with_compiled_lengths(torch_cuda, n, dtype):
+    """Boxes with some axes of a compiled length: each pass takes the block form of its own
+    axis, the z pass's energy sums the shell of all three.  Against the oracle, the tail
+    indicator against the padded spectrum of the density."""
+    from paper_1612_01799_gb300 import Plan
+    torch = torch_cuda
+    tol = 1e-12 if dtype == "f64" else 1e-6
+    half = tuple(0.5 * q for q in n)
+    op = obox.make_box_plan(n, tuple(-q for q in half), half, tol)
+    rho = np.random.default_rng(sum(n)).uniform(-1, 1, (n[2], n[1], n[0]))
+    uo = obox.solve_box(rho, op)
+    F = np.abs(np.fft.fftn(rho, s=[2 * q for q in rho.shape], axes=(0, 1, 2))) ** 2
+    k = [np.minimum(np.arange(2 * q), 2 * q - np.arange(2 * q)) >= q - q // 8 for q in rho.shape]
+    shell = k[0][:, None, None] | k[1][None, :, None] | k[2][None, None, :]
+    ref = math.sqrt(F[shell].sum() / F.sum())
+    with Plan(n, half, tol, dtype) as p:
+        for ar in variants(dtype):
+            if ar:
+                p.arith = ar
+            u = run(torch, p, rho)
+            assert rel_l2(u, uo) <= TOL[dtype], ar
+            t = torch.from_numpy(rho.astype(p.np_dtype)).cuda()
+            out, eta = torch.empty_like(t), ctypes.c_double()
+            assert p._lib.poisson_solve_checked(p.handle, t.data_ptr(), out.data_ptr(), ctypes.byref(eta), None) == 0
+            torch.cuda.synchronize()
+            assert eta.value == pytest.approx(ref, rel=1e-5)
+            assert np.array_equal(out.cpu().numpy().astype(np.float64).reshape(u.shape), u)
