@@ -86,16 +86,30 @@ inline AnySched any_sched(int L, int max_radix, int max_last, bool pad) {
 // Largest radix, per arithmetic.  Double-float stops at 10: its butterflies are ten times longer
 // in instructions, and the stages of a kernel should stay within the instruction cache.
 constexpr int any_max_radix(bool df) { return df ? 10 : 12; }
+// The schedule with radices up to 10, or up to max_radix where that takes a stage less; mr: the
+// largest radix (10 or 12) the kernels that run it need.  Kernels without the radix-12 stages
+// are 2 to 10% faster on the same schedule (FP32 solves: N = 400 2.81 and 2.78 ms, N = 162 242 and
+// 234 us, N = 120 107 and 97 us), one more stage costs more (N = 60 25 and 33 us, N = 72 29 and
+// 36 us).
+inline AnySched any_sched_of(int L, int max_radix, int max_last, bool pad, int *mr) {
+    const AnySched a = any_sched(L, 10, std::min(max_last, 10), pad);
+    *mr = std::max(*mr, 10);
+    if (max_radix == 10) return a;
+    const AnySched b = any_sched(L, max_radix, max_last, pad);
+    if (!b.nst || (a.nst && a.nst <= b.nst)) return a;
+    *mr = max_radix;
+    return b;
+}
 // Warps of an SM that their registers admit (80 in FP32, 128 otherwise).
 constexpr int any_max_warps(bool f32) { return f32 ? 24 : 16; }
 // Largest last radix of the x passes, whose last stage holds two butterflies.
 constexpr int kAnyRowsLast = 8;
 
 // Tile of a runtime-length pass: its schedule, 2^lg 16-byte groups, slots pitch groups apart,
-// threads, bytes of shared memory.
+// threads, bytes of shared memory, largest radix of its kernel.
 struct AnyTile {
     AnySched s;
-    int lg, pitch, threads, smem;
+    int lg, pitch, threads, smem, mr;
 };
 constexpr int kAnyThreads = 256;  // threads the kernels are compiled for
 
@@ -110,9 +124,9 @@ constexpr int kAnyThreads = 256;  // threads the kernels are compiled for
 inline AnyTile any_tile(int L, int max_radix, int max_warps, bool rows) {
     AnyTile t{};
     const int max_last = rows ? kAnyRowsLast : max_radix;
-    const AnySched wide = any_sched(L, max_radix, max_last, rows);
+    const AnySched wide = any_sched_of(L, max_radix, max_last, rows, &t.mr);
     t.lg = wide.slots * (rows ? 9 : 8) * 16 <= 70 * 1024 ? 3 : 2;
-    t.s = t.lg == 3 ? wide : any_sched(L, max_radix, max_last, true);
+    t.s = t.lg == 3 ? wide : any_sched_of(L, max_radix, max_last, true, &t.mr);
     t.pitch = (1 << t.lg) + (rows ? 1 : 0);
     t.smem = t.s.slots * t.pitch * 16;
     double best = 0.0;
@@ -138,7 +152,7 @@ inline AnyTile any_tile(int L, int max_radix, int max_warps, bool rows) {
 // w columns or rows per 16-byte group.  threads as for any_tile, over the stages of both axes.
 struct PlaneTile {
     AnySched sx, sy;
-    int gx, px, gy, py, threads, smem;
+    int gx, px, gy, py, threads, smem, mr;
     bool on;
 };
 constexpr int kPlaneThreads = 384;
@@ -150,8 +164,8 @@ constexpr int kPlaneThreads = 384;
 constexpr int plane_smem(bool f32) { return f32 ? 106 * 1024 : 48 * 1024; }
 inline PlaneTile plane_tile(int nx, int ny, int max_radix, int w) {
     PlaneTile t{};
-    t.sx = any_sched(nx, max_radix, kAnyRowsLast, true);
-    t.sy = any_sched(2 * ny, max_radix, max_radix, false);
+    t.sx = any_sched_of(nx, max_radix, kAnyRowsLast, true, &t.mr);
+    t.sy = any_sched_of(2 * ny, max_radix, max_radix, false, &t.mr);
     t.gx = ny / w;
     t.gy = (nx + w) / w;
     t.px = t.gx | 1;

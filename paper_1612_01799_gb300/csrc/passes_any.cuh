@@ -23,7 +23,7 @@
 // three quarters of its slots in z.  Two or three stages of radix 8 to 12 in place of five to
 // seven of radix 2 to 5 with a ping-pong pair, the first stage's zeros left out, took the
 // FP32 solve at N = 400 from 9.45 to 2.77 ms, N = 240 from 2.14 to 0.59 ms, the box 64 x 128 x
-// 192 from 257 to 109 us and the double-float solve at N = 162 from 1.20 to 0.92 ms.
+// 192 from 257 to 109 us and the double-float solve at N = 162 from 1.20 to 0.87 ms.
 //
 // Workspace layout (complex, the arithmetic's storage): w1 [b][z < nz][y < ny][kx < Px],
 // w2 and w3 [b][z < nz][ky < 2 ny][kx < Px], Px = pitch of nx + 1; symbol
@@ -32,9 +32,6 @@
 #pragma once
 
 namespace gsp {
-
-// Largest radix of a stage.
-template <typename Real> constexpr int kAnyMaxRadix = any_max_radix(std::is_same<Real, DF>::value);
 
 // Row r (< TR) of the tile starting at batch row r0: its density and its row in that density.
 // rows_b >= TR, so a tile crosses at most one density boundary.
@@ -164,16 +161,16 @@ template <int R, typename C> __device__ __forceinline__ void any_dft_half_adj(C 
     }
 }
 
-// Runs f.template operator()<R>() for the radix R of a stage: the even ones (first stages) and
-// all of them.
-template <typename Real, typename F> __device__ __forceinline__ void any_radix_even(int R, F &&f) {
+// Runs f.template operator()<R>() for the radix R <= MR (10 or 12) of a stage: the even ones
+// (first stages) and all of them.
+template <int MR, typename F> __device__ __forceinline__ void any_radix_even(int R, F &&f) {
     switch (R) {
         case 2: f.template operator()<2>(); break;
         case 4: f.template operator()<4>(); break;
         case 6: f.template operator()<6>(); break;
         case 8: f.template operator()<8>(); break;
         default:
-            if constexpr (kAnyMaxRadix<Real> > 10) {
+            if constexpr (MR > 10) {
                 if (R == 12) {
                     f.template operator()<12>();
                     break;
@@ -182,17 +179,17 @@ template <typename Real, typename F> __device__ __forceinline__ void any_radix_e
             f.template operator()<10>();
     }
 }
-template <typename Real, typename F> __device__ __forceinline__ void any_radix(int R, F &&f) {
+template <int MR, typename F> __device__ __forceinline__ void any_radix(int R, F &&f) {
     switch (R) {
         case 3: f.template operator()<3>(); break;
         case 5: f.template operator()<5>(); break;
         case 9: f.template operator()<9>(); break;
-        default: any_radix_even<Real>(R, f);
+        default: any_radix_even<MR>(R, f);
     }
 }
 
 // The radices the last stage of the x passes may have (kAnyRowsLast).
-template <typename Real, typename F> __device__ __forceinline__ void any_radix_last(int R, F &&f) {
+template <typename F> __device__ __forceinline__ void any_radix_last(int R, F &&f) {
     switch (R) {
         case 2: f.template operator()<2>(); break;
         case 3: f.template operator()<3>(); break;
@@ -256,7 +253,7 @@ __device__ __forceinline__ void any_stage(float4 *p, int step, const Tw &tw, int
 // The stages st0 <= st < st1 of a tile of 2^lg groups (slot a of group g at buf[a * PG + g]),
 // forward in ascending and inverse in descending order, each behind a block barrier.
 // twstride: the table holds exp(-2 pi i e / (L twstride)).
-template <typename Real, int D>
+template <typename Real, int MR, int D>
 __device__ __forceinline__ void any_stages(float4 *buf, const AnySched &s, int lg, int PG, const AnyTwiddles<Real> &tw,
                                            int st0, int st1) {
     using C = typename Types<Real>::CC;
@@ -266,7 +263,7 @@ __device__ __forceinline__ void any_stages(float4 *buf, const AnySched &s, int l
         __syncthreads();
         const int R = s.r[st], nb = s.P[st] * s.M[st], step = s.S[st] * PG;
         const bool last = st == s.nst - 1;
-        any_radix<Real>(R, [&]<int RR>() {
+        any_radix<MR>(R, [&]<int RR>() {
             for (int b = threadIdx.x >> lg; b < nb; b += blockDim.x >> lg) {
                 const AnyBfly f = any_bfly(s, st, b);
                 float4 *p = buf + f.slot * PG + g;
@@ -279,11 +276,11 @@ __device__ __forceinline__ void any_stages(float4 *buf, const AnySched &s, int l
 
 // The first forward stage of a column transform (time j + r M_0, r < R_0 / 2, loaded by
 // ld(row)) and the last inverse stage (st(row, value) for the kept rows).
-template <typename Real, class Ld>
+template <typename Real, int MR, class Ld>
 __device__ __forceinline__ void any_first(float4 *buf, const AnySched &s, int lg, const AnyTwiddles<Real> &tw, Ld &&ld) {
     using C = typename Types<Real>::CC;
     const int g = threadIdx.x & ((1 << lg) - 1), M = s.M[0], step = s.S[0] << lg;
-    any_radix_even<Real>(s.r[0], [&]<int R>() {
+    any_radix_even<MR>(s.r[0], [&]<int R>() {
         constexpr int H = R / 2;
         for (int j = threadIdx.x >> lg; j < M; j += blockDim.x >> lg) {
             C v[R];
@@ -299,12 +296,12 @@ __device__ __forceinline__ void any_first(float4 *buf, const AnySched &s, int lg
         }
     });
 }
-template <typename Real, class St>
+template <typename Real, int MR, class St>
 __device__ __forceinline__ void any_first_adj(const float4 *buf, const AnySched &s, int lg, const AnyTwiddles<Real> &tw, St &&st) {
     using C = typename Types<Real>::CC;
     const int g = threadIdx.x & ((1 << lg) - 1), M = s.M[0], step = s.S[0] << lg;
     __syncthreads();
-    any_radix_even<Real>(s.r[0], [&]<int R>() {
+    any_radix_even<MR>(s.r[0], [&]<int R>() {
         constexpr int H = R / 2;
         for (int j = threadIdx.x >> lg; j < M; j += blockDim.x >> lg) {
             const float4 *p = buf + (any_lo_slot(s, 0, j) << lg) + g;
@@ -333,7 +330,7 @@ template <typename Real> constexpr int kAnyMinBlocks = sizeof(typename Types<Rea
 // nx-point complex FFT of the (even, odd) sample pairs (pairs >= nx/2 zero) and the Hermitian
 // split into the nx + 1 bins (twiddles W_{2nx}^k; the nx-point FFT reads the same table at
 // stride 2).
-template <typename Real>
+template <typename Real, int MR>
 __global__ void __launch_bounds__(kAnyThreads, kAnyMinBlocks<Real>)
 k_any_x_fwd(const PtrArray rho, Cx2<Real> *__restrict__ out, const AnyTw<Real> *__restrict__ tw,
             const __grid_constant__ AnySched s, int rows_b, int nrows, int Px, unsigned mul_half, int lg, int ntiles) {
@@ -351,7 +348,7 @@ k_any_x_fwd(const PtrArray rho, Cx2<Real> *__restrict__ out, const AnyTw<Real> *
         const int ng = (int)min((long long)NG, (nrows - r0) / W);
         const AnyRows rows(r0, rows_b);
         // Rows as they lie, times j + r M_0 of group g into their slots; missing rows as zeros.
-        any_radix_even<Real>(s.r[0], [&]<int R>() {
+        any_radix_even<MR>(s.r[0], [&]<int R>() {
             for (int e = threadIdx.x; e < NG * M; e += blockDim.x) {
                 const int g = rdiv(e, s.mulM[0]), j = e - g * M;
                 const bool ok = g < ng && dbg_index_ok(rows.row(W * g), rows_b);
@@ -375,7 +372,7 @@ k_any_x_fwd(const PtrArray rho, Cx2<Real> *__restrict__ out, const AnyTw<Real> *
         __syncthreads();
         {
             const int g = threadIdx.x & (NG - 1), step = s.S[0] * PG;
-            any_radix_even<Real>(s.r[0], [&]<int R>() {
+            any_radix_even<MR>(s.r[0], [&]<int R>() {
                 constexpr int H = R / 2;
                 for (int j = threadIdx.x >> lg; j < M; j += blockDim.x >> lg) {
                     float4 *p = buf + any_lo_slot(s, 0, j) * PG + g;
@@ -392,13 +389,13 @@ k_any_x_fwd(const PtrArray rho, Cx2<Real> *__restrict__ out, const AnyTw<Real> *
             });
         }
         const int last = s.nst - 1, P = s.P[last], half = P / 2 + 1;
-        any_stages<Real, -1>(buf, s, lg, PG, ts, 1, last);
+        any_stages<Real, MR, -1>(buf, s, lg, PG, ts, 1, last);
         __syncthreads();
         // The last stage with the split, neighbouring frequencies in a warp: butterfly f makes the
         // bins k = f + r P, its partner P - f the bins n - k.
         // X_k = Ev_k + W_{2n}^k Od_k, X_{n-k} = conj(Ev_k - W_{2n}^k Od_k), with Ev, Od the DFTs
         // of the even and odd samples from C_k and conj C_{n-k}.
-        any_radix_last<Real>(s.r[last], [&]<int R>() {
+        any_radix_last(s.r[last], [&]<int R>() {
             for (int e = threadIdx.x; e < ng * half; e += blockDim.x) {
                 const int g = rdiv(e, mul_half), f = e - g * half;
                 const bool own = f == 0 || 2 * f == P;  // n - k lies in butterfly f itself
@@ -439,7 +436,7 @@ k_any_x_fwd(const PtrArray rho, Cx2<Real> *__restrict__ out, const AnyTw<Real> *
 // The nx + 1 Hermitian bins of each row -> C_k = Ev_k + i Od_k (Ev_k = Y_k + conj Y_{n-k},
 // Od_k = (Y_k - conj Y_{n-k}) W_{2n}^{-k}), the inverse nx-point FFT gives y_{2m} + i y_{2m+1};
 // pairs m < nx/2 are kept (the crop).  Shared layout as in the forward.
-template <typename Real>
+template <typename Real, int MR>
 __global__ void __launch_bounds__(kAnyThreads, kAnyMinBlocks<Real>)
 k_any_x_inv(const Cx2<Real> *__restrict__ in, const PtrArray u, const AnyTw<Real> *__restrict__ tw,
             const __grid_constant__ AnySched s, int rows_b, int nrows, int Px, unsigned mul_half, int lg, int ntiles) {
@@ -457,7 +454,7 @@ k_any_x_inv(const Cx2<Real> *__restrict__ in, const PtrArray u, const AnyTw<Real
         const int ng = (int)min((long long)NG, (nrows - r0) / W);
         // The combination with the first stage of the inverse, as the forward's last one.
         const int last = s.nst - 1, P = s.P[last], half = P / 2 + 1;
-        any_radix_last<Real>(s.r[last], [&]<int R>() {
+        any_radix_last(s.r[last], [&]<int R>() {
             for (int e = threadIdx.x; e < NG * half; e += blockDim.x) {
                 const int g = rdiv(e, mul_half), f = e - g * half;
                 const bool own = f == 0 || 2 * f == P;
@@ -497,11 +494,11 @@ k_any_x_inv(const Cx2<Real> *__restrict__ in, const PtrArray u, const AnyTw<Real
                 for (int r = 0; r < R; ++r) any_st(p + r * PG, x[r]);
             }
         });
-        any_stages<Real, 1>(buf, s, lg, PG, ts, 1, last);
+        any_stages<Real, MR, 1>(buf, s, lg, PG, ts, 1, last);
         __syncthreads();
         {
             const int g = threadIdx.x & (NG - 1), step = s.S[0] * PG;
-            any_radix_even<Real>(s.r[0], [&]<int R>() {
+            any_radix_even<MR>(s.r[0], [&]<int R>() {
                 constexpr int H = R / 2;
                 for (int j = threadIdx.x >> lg; j < M; j += blockDim.x >> lg) {
                     float4 *p = buf + any_lo_slot(s, 0, j) * PG + g;
@@ -520,7 +517,7 @@ k_any_x_inv(const Cx2<Real> *__restrict__ in, const PtrArray u, const AnyTw<Real
         }
         __syncthreads();
         const AnyRows rows(r0, rows_b);
-        any_radix_even<Real>(s.r[0], [&]<int R>() {
+        any_radix_even<MR>(s.r[0], [&]<int R>() {
             for (int e = threadIdx.x; e < ng * M; e += blockDim.x) {
                 const int g = rdiv(e, s.mulM[0]), j = e - g * M;
                 if (!dbg_index_ok(rows.row(W * g), rows_b)) continue;
@@ -540,7 +537,7 @@ k_any_x_inv(const Cx2<Real> *__restrict__ in, const PtrArray u, const AnyTw<Real
 // ---- K2 / K4: y passes --------------------------------------------------------------------------
 // Tile (tx, plane): 2^lg groups of columns of one plane.  FWD: input rows < L/2 (the rest zero),
 // all L rows stored; !FWD: all L input rows, rows < L/2 stored.
-template <typename Real, bool FWD>
+template <typename Real, int MR, bool FWD>
 __global__ void __launch_bounds__(kAnyThreads, kAnyMinBlocks<Real>)
 k_any_col(const Cx2<Real> *__restrict__ in, Cx2<Real> *__restrict__ out, const AnyTw<Real> *__restrict__ tw,
           const __grid_constant__ AnySched s, int ncols, int ntx, int Px, long long in_outer, long long out_outer, int lg, int ntiles) {
@@ -560,11 +557,11 @@ k_any_col(const Cx2<Real> *__restrict__ in, Cx2<Real> *__restrict__ out, const A
         Cx2<Real> *dst = out + plane * out_outer + (valid ? col : 0);
         const int last = s.nst - 1, nb = s.P[last], step = s.S[last];
         if constexpr (FWD) {
-            any_first<Real>(buf, s, lg, ts,
+            any_first<Real, MR>(buf, s, lg, ts,
                                     [&](int row) { return valid ? ld_cc(src + (long long)row * Px) : czero<C>(); });
-            any_stages<Real, -1>(buf, s, lg, 1 << lg, ts, 1, last);
+            any_stages<Real, MR, -1>(buf, s, lg, 1 << lg, ts, 1, last);
             __syncthreads();
-            any_radix<Real>(s.r[last], [&]<int R>() {
+            any_radix<MR>(s.r[last], [&]<int R>() {
                 for (int b = threadIdx.x >> lg; b < nb; b += blockDim.x >> lg) {
                     const AnyBfly f = any_bfly(s, last, b);
                     C v[R];
@@ -577,7 +574,7 @@ k_any_col(const Cx2<Real> *__restrict__ in, Cx2<Real> *__restrict__ out, const A
                 }
             });
         } else {
-            any_radix<Real>(s.r[last], [&]<int R>() {
+            any_radix<MR>(s.r[last], [&]<int R>() {
                 for (int b = threadIdx.x >> lg; b < nb; b += blockDim.x >> lg) {
                     const AnyBfly f = any_bfly(s, last, b);
                     C v[R];
@@ -589,8 +586,8 @@ k_any_col(const Cx2<Real> *__restrict__ in, Cx2<Real> *__restrict__ out, const A
                     for (int r = 0; r < R; ++r) any_st(buf + ((f.slot + r * step) << lg) + g, v[r]);
                 }
             });
-            any_stages<Real, 1>(buf, s, lg, 1 << lg, ts, 1, last);
-            any_first_adj<Real>(buf, s, lg, ts, [&](int row, C x) {
+            any_stages<Real, MR, 1>(buf, s, lg, 1 << lg, ts, 1, last);
+            any_first_adj<Real, MR>(buf, s, lg, ts, [&](int row, C x) {
                 if (valid) st_cc(dst + (long long)row * Px, x);
             });
         }
@@ -605,7 +602,7 @@ k_any_col(const Cx2<Real> *__restrict__ in, Cx2<Real> *__restrict__ out, const A
 // per tile).  The tiles cover the lines ky0 <= ky < ky0 + nky (all of them:
 // ky0 = 0, nky = 2 ny, taken as ky and its mirror in turn, which read the same symbol rows; a
 // rank's slab of lines in the slab decomposition of one solve).
-template <typename Real, bool TAIL>
+template <typename Real, int MR, bool TAIL>
 __global__ void __launch_bounds__(kAnyThreads, kAnyMinBlocks<Real>)
 k_any_z(const Cx2<Real> *__restrict__ in, Cx2<Real> *__restrict__ out, const Real *__restrict__ sym,
         const AnyTw<Real> *__restrict__ tw, const __grid_constant__ AnySched s, int nx, int ny, int ntx, int Px, int Ps,
@@ -629,12 +626,12 @@ k_any_z(const Cx2<Real> *__restrict__ in, Cx2<Real> *__restrict__ out, const Rea
         const long long base = ((long long)bb * nz * Ly + ky) * Px + (valid ? col : 0);
         const Real *srow = sym + (long long)kya * Ps + (valid ? col : 0);
         const long long splane = (long long)(ny + 1) * Ps;
-        any_first<Real>(buf, s, lg, ts, [&](int row) { return valid ? ld_cc(in + base + row * zs) : czero<C>(); });
+        any_first<Real, MR>(buf, s, lg, ts, [&](int row) { return valid ? ld_cc(in + base + row * zs) : czero<C>(); });
         const int last = s.nst - 1, nb = s.P[last], step = s.S[last];
-        any_stages<Real, -1>(buf, s, lg, 1 << lg, ts, 1, last);
+        any_stages<Real, MR, -1>(buf, s, lg, 1 << lg, ts, 1, last);
         __syncthreads();
         float eshell = 0.f, etot = 0.f;
-        any_radix<Real>(s.r[last], [&]<int R>() {
+        any_radix<MR>(s.r[last], [&]<int R>() {
             for (int b = threadIdx.x >> lg; b < nb; b += blockDim.x >> lg) {
                 const AnyBfly f = any_bfly(s, last, b);
                 float4 *p = buf + (f.slot << lg) + g;
@@ -667,8 +664,8 @@ k_any_z(const Cx2<Real> *__restrict__ in, Cx2<Real> *__restrict__ out, const Rea
                 for (int r = 0; r < R; ++r) any_st(p + ((r * step) << lg), v[r]);
             }
         });
-        any_stages<Real, 1>(buf, s, lg, 1 << lg, ts, 1, last);
-        any_first_adj<Real>(buf, s, lg, ts, [&](int row, C x) {
+        any_stages<Real, MR, 1>(buf, s, lg, 1 << lg, ts, 1, last);
+        any_first_adj<Real, MR>(buf, s, lg, ts, [&](int row, C x) {
             if (valid) st_cc(out + base + row * zs, x);
         });
         if constexpr (TAIL) {

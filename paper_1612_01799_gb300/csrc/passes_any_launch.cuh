@@ -12,6 +12,13 @@ template <typename Real, class K> int any_grid(K k, const AnyTile &t, int smem, 
     return AnyTwiddles<Real>::kCopy ? persistent_blocks(k, t.threads, smem, ntiles) : ntiles;
 }
 
+// Runs f.template operator()<MR>() with MR the largest radix the kernels are compiled for.
+template <typename Real, class F> cudaError_t any_with_radix(int mr, F &&f) {
+    if constexpr (any_max_radix(std::is_same<Real, DF>::value) > 10)
+        if (mr > 10) return f.template operator()<12>();
+    return f.template operator()<10>();
+}
+
 template <typename Real>
 cudaError_t any_x(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int B, cudaStream_t s, bool fwd,
                   int rows, void *w1) {
@@ -24,15 +31,17 @@ cudaError_t any_x(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, i
     Cx2<Real> *ws = static_cast<Cx2<Real> *>(w1 ? w1 : p.w1);
     const int TR = Types<Real>::W << t.lg, nt = (nrows + TR - 1) / TR;
     const int smem = t.smem + any_tw_bytes<Real>(nx);
-    if (fwd) {
-        GSP_CHECK(set_smem(k_any_x_fwd<Real>, smem));
-        GSP_CHECK(launch_pdl(k_any_x_fwd<Real>, any_grid<Real>(k_any_x_fwd<Real>, t, smem, nt), t.threads, smem, s, rho, ws, tw, t.s, rows_b, nrows, p.Px, mul_half, t.lg, nt));
-    } else {
-        GSP_CHECK(set_smem(k_any_x_inv<Real>, smem));
-        GSP_CHECK(launch_pdl(k_any_x_inv<Real>, any_grid<Real>(k_any_x_inv<Real>, t, smem, nt), t.threads, smem, s, static_cast<const Cx2<Real> *>(ws), u, tw, t.s, rows_b,
-                             nrows, p.Px, mul_half, t.lg, nt));
-    }
-    return cudaGetLastError();
+    return any_with_radix<Real>(t.mr, [&]<int MR>() {
+        if (fwd) {
+            GSP_CHECK(set_smem(k_any_x_fwd<Real, MR>, smem));
+            GSP_CHECK(launch_pdl(k_any_x_fwd<Real, MR>, any_grid<Real>(k_any_x_fwd<Real, MR>, t, smem, nt), t.threads, smem, s, rho, ws, tw, t.s, rows_b, nrows, p.Px, mul_half, t.lg, nt));
+        } else {
+            GSP_CHECK(set_smem(k_any_x_inv<Real, MR>, smem));
+            GSP_CHECK(launch_pdl(k_any_x_inv<Real, MR>, any_grid<Real>(k_any_x_inv<Real, MR>, t, smem, nt), t.threads, smem, s, static_cast<const Cx2<Real> *>(ws), u, tw, t.s, rows_b,
+                                 nrows, p.Px, mul_half, t.lg, nt));
+        }
+        return cudaGetLastError();
+    });
 }
 
 template <typename Real>
@@ -45,18 +54,20 @@ cudaError_t any_y(const DevicePlan &p, int B, cudaStream_t s, bool fwd, int z0, 
     if (!t.s.nst) return cudaErrorInvalidValue;
     const int TC = Types<Real>::W << t.lg, ntx = (ncols + TC - 1) / TC, nt = ntx * planes;
     const int smem = t.smem + any_tw_bytes<Real>(L);
-    if (fwd) {
-        GSP_CHECK(set_smem(k_any_col<Real, true>, smem));
-        GSP_CHECK(launch_pdl(k_any_col<Real, true>, any_grid<Real>(k_any_col<Real, true>, t, smem, nt), t.threads, smem, s,
-                             static_cast<const Cx2<Real> *>(p.w1) + z0 * w1p, static_cast<Cx2<Real> *>(p.w2) + z0 * w2p,
-                             tw, t.s, ncols, ntx, p.Px, w1p, w2p, t.lg, nt));
-    } else {
-        GSP_CHECK(set_smem(k_any_col<Real, false>, smem));
-        GSP_CHECK(launch_pdl(k_any_col<Real, false>, any_grid<Real>(k_any_col<Real, false>, t, smem, nt), t.threads, smem, s,
-                             static_cast<const Cx2<Real> *>(p.w3) + z0 * w2p, static_cast<Cx2<Real> *>(p.w1) + z0 * w1p,
-                             tw, t.s, ncols, ntx, p.Px, w2p, w1p, t.lg, nt));
-    }
-    return cudaGetLastError();
+    return any_with_radix<Real>(t.mr, [&]<int MR>() {
+        if (fwd) {
+            GSP_CHECK(set_smem(k_any_col<Real, MR, true>, smem));
+            GSP_CHECK(launch_pdl(k_any_col<Real, MR, true>, any_grid<Real>(k_any_col<Real, MR, true>, t, smem, nt), t.threads, smem, s,
+                                 static_cast<const Cx2<Real> *>(p.w1) + z0 * w1p, static_cast<Cx2<Real> *>(p.w2) + z0 * w2p,
+                                 tw, t.s, ncols, ntx, p.Px, w1p, w2p, t.lg, nt));
+        } else {
+            GSP_CHECK(set_smem(k_any_col<Real, MR, false>, smem));
+            GSP_CHECK(launch_pdl(k_any_col<Real, MR, false>, any_grid<Real>(k_any_col<Real, MR, false>, t, smem, nt), t.threads, smem, s,
+                                 static_cast<const Cx2<Real> *>(p.w3) + z0 * w2p, static_cast<Cx2<Real> *>(p.w1) + z0 * w1p,
+                                 tw, t.s, ncols, ntx, p.Px, w2p, w1p, t.lg, nt));
+        }
+        return cudaGetLastError();
+    });
 }
 
 // The z pass of lines ky0 <= ky < ky0 + nky (nky = 0: all 2 ny lines).  Runs on the tables of
@@ -71,12 +82,14 @@ cudaError_t any_z(const DevicePlan &p, int B, cudaStream_t s, double *tail, int 
     if (!t.s.nst) return cudaErrorInvalidValue;
     const int TC = Types<Real>::W << t.lg, ntx = (nx + 1 + TC - 1) / TC, nt = ntx * nky * B;
     const int smem = t.smem + any_tw_bytes<Real>(t.s.L);
-    auto k = tail ? k_any_z<Real, true> : k_any_z<Real, false>;
-    GSP_CHECK(set_smem(k, smem));
-    GSP_CHECK(launch_pdl(k, any_grid<Real>(k, t, smem, nt), t.threads, smem, s, static_cast<const Cx2<Real> *>(p.w2),
-                         static_cast<Cx2<Real> *>(p.w3), static_cast<const Real *>(p.sym), tw, t.s, nx, ny, ntx, p.Px,
-                         p.Ps, tail, ky0, nky, t.lg, nt));
-    return cudaGetLastError();
+    return any_with_radix<Real>(t.mr, [&]<int MR>() {
+        auto k = tail ? k_any_z<Real, MR, true> : k_any_z<Real, MR, false>;
+        GSP_CHECK(set_smem(k, smem));
+        GSP_CHECK(launch_pdl(k, any_grid<Real>(k, t, smem, nt), t.threads, smem, s, static_cast<const Cx2<Real> *>(p.w2),
+                             static_cast<Cx2<Real> *>(p.w3), static_cast<const Real *>(p.sym), tw, t.s, nx, ny, ntx, p.Px,
+                             p.Ps, tail, ky0, nky, t.lg, nt));
+        return cudaGetLastError();
+    });
 }
 
 // One translation unit per pass and arithmetic (the double-float ones compile slowly).

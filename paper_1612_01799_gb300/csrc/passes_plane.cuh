@@ -27,14 +27,14 @@ template <class F> __device__ __forceinline__ void plane_each(int nb, const Plan
 }
 
 // Middle stages st0 <= st < st1, each behind a block barrier.
-template <typename Real, int D>
+template <typename Real, int MR, int D>
 __device__ __forceinline__ void plane_stages(float4 *buf, const AnySched &s, const PlaneGroups &q,
                                              const AnyTwiddles<Real> &tw, int st0, int st1) {
     using C = typename Types<Real>::CC;
     for (int i = st0; i < st1; ++i) {
         const int st = D < 0 ? i : st0 + st1 - 1 - i;
         __syncthreads();
-        any_radix<Real>(s.r[st], [&]<int R>() {
+        any_radix<MR>(s.r[st], [&]<int R>() {
             plane_each(s.P[st] * s.M[st], q, [&](int b, int g) {
                 const AnyBfly f = any_bfly(s, st, b);
                 any_stage<R, D, true, C>(buf + f.slot * q.pitch + g, s.S[st] * q.pitch, tw, f.lo * s.P[st]);
@@ -43,13 +43,13 @@ __device__ __forceinline__ void plane_stages(float4 *buf, const AnySched &s, con
     }
 }
 // First forward stage in place (times j + r M_0, r < R_0 / 2) and its adjoint.
-template <typename Real, int D>
+template <typename Real, int MR, int D>
 __device__ __forceinline__ void plane_first(float4 *buf, const AnySched &s, const PlaneGroups &q,
                                             const AnyTwiddles<Real> &tw) {
     using C = typename Types<Real>::CC;
     const int step = s.S[0] * q.pitch;
     __syncthreads();
-    any_radix_even<Real>(s.r[0], [&]<int R>() {
+    any_radix_even<MR>(s.r[0], [&]<int R>() {
         constexpr int H = R / 2;
         plane_each(s.M[0], q, [&](int j, int g) {
             float4 *p = buf + any_lo_slot(s, 0, j) * q.pitch + g;
@@ -116,7 +116,7 @@ struct PlaneArgs {
 template <typename Real> constexpr int kPlaneMinBlocks = sizeof(typename Types<Real>::CS) == 8 ? 2 : 1;
 
 // ---- K1 + K2 --------------------------------------------------------------------------------------
-template <typename Real>
+template <typename Real, int MR>
 __global__ void __launch_bounds__(kPlaneThreads, kPlaneMinBlocks<Real>)
 k_plane_fwd(const PtrArray rho, Cx2<Real> *__restrict__ w2, const AnyTw<Real> *__restrict__ tw_x,
             const AnyTw<Real> *__restrict__ tw_y, const __grid_constant__ PlaneArgs a) {
@@ -131,7 +131,7 @@ k_plane_fwd(const PtrArray rho, Cx2<Real> *__restrict__ w2, const AnyTw<Real> *_
     griddep_wait();
     const int pl = blockIdx.x, b = pl / a.nz, z = pl - b * a.nz;
     const X2 *plane = reinterpret_cast<const X2 *>(rho.p[b]) + (long long)z * ny * h;
-    any_radix_even<Real>(sx.r[0], [&]<int R>() {
+    any_radix_even<MR>(sx.r[0], [&]<int R>() {
         for (int e = threadIdx.x; e < a.qx.G * M; e += blockDim.x) {
             const int g = rdiv(e, sx.mulM[0]), j = e - g * M;
             const X2 *src = plane + (long long)W * g * h + j;
@@ -146,12 +146,12 @@ k_plane_fwd(const PtrArray rho, Cx2<Real> *__restrict__ w2, const AnyTw<Real> *_
             for (int r = 0; r < R / 2; ++r) any_st(p + r * sx.S[0] * a.qx.pitch, v[r]);
         }
     });
-    plane_first<Real, -1>(xb, sx, a.qx, tx);
+    plane_first<Real, MR, -1>(xb, sx, a.qx, tx);
     const int last = sx.nst - 1, P = sx.P[last], half = P / 2 + 1;
-    plane_stages<Real, -1>(xb, sx, a.qx, tx, 1, last);
+    plane_stages<Real, MR, -1>(xb, sx, a.qx, tx, 1, last);
     __syncthreads();
     // The last x stage with the Hermitian split (as in k_any_x_fwd), into the y buffer.
-    any_radix_last<Real>(sx.r[last], [&]<int R>() {
+    any_radix_last(sx.r[last], [&]<int R>() {
         for (int e = threadIdx.x; e < a.qx.G * half; e += blockDim.x) {
             const int g = rdiv(e, a.mul_half), f = e - g * half;
             const bool own = f == 0 || 2 * f == P;
@@ -183,12 +183,12 @@ k_plane_fwd(const PtrArray rho, Cx2<Real> *__restrict__ w2, const AnyTw<Real> *_
             }
         }
     });
-    plane_first<Real, -1>(yb, sy, a.qy, ty);
+    plane_first<Real, MR, -1>(yb, sy, a.qy, ty);
     const int lasty = sy.nst - 1, nb = sy.P[lasty];
-    plane_stages<Real, -1>(yb, sy, a.qy, ty, 1, lasty);
+    plane_stages<Real, MR, -1>(yb, sy, a.qy, ty, 1, lasty);
     __syncthreads();
     Cx2<Real> *dst = w2 + (long long)pl * sy.L * a.Px;
-    any_radix<Real>(sy.r[lasty], [&]<int R>() {
+    any_radix<MR>(sy.r[lasty], [&]<int R>() {
         plane_each(nb, a.qy, [&](int bf, int g) {
             const AnyBfly f = any_bfly(sy, lasty, bf);
             const float4 *p = yb + f.slot * a.qy.pitch + g;
@@ -203,7 +203,7 @@ k_plane_fwd(const PtrArray rho, Cx2<Real> *__restrict__ w2, const AnyTw<Real> *_
 }
 
 // ---- K4 + K5 --------------------------------------------------------------------------------------
-template <typename Real>
+template <typename Real, int MR>
 __global__ void __launch_bounds__(kPlaneThreads, kPlaneMinBlocks<Real>)
 k_plane_inv(const Cx2<Real> *__restrict__ w3, const PtrArray u, const AnyTw<Real> *__restrict__ tw_x,
             const AnyTw<Real> *__restrict__ tw_y, const __grid_constant__ PlaneArgs a) {
@@ -219,7 +219,7 @@ k_plane_inv(const Cx2<Real> *__restrict__ w3, const PtrArray u, const AnyTw<Real
     const int pl = blockIdx.x, b = pl / a.nz, z = pl - b * a.nz;
     const Cx2<Real> *src = w3 + (long long)pl * sy.L * a.Px;
     const int lasty = sy.nst - 1, nb = sy.P[lasty];
-    any_radix<Real>(sy.r[lasty], [&]<int R>() {
+    any_radix<MR>(sy.r[lasty], [&]<int R>() {
         plane_each(nb, a.qy, [&](int bf, int g) {
             const AnyBfly f = any_bfly(sy, lasty, bf);
             C v[R];
@@ -231,12 +231,12 @@ k_plane_inv(const Cx2<Real> *__restrict__ w3, const PtrArray u, const AnyTw<Real
             for (int r = 0; r < R; ++r) any_st(p + r * a.qy.pitch, v[r]);
         });
     });
-    plane_stages<Real, 1>(yb, sy, a.qy, ty, 1, lasty);
-    plane_first<Real, 1>(yb, sy, a.qy, ty);
+    plane_stages<Real, MR, 1>(yb, sy, a.qy, ty, 1, lasty);
+    plane_first<Real, MR, 1>(yb, sy, a.qy, ty);
     __syncthreads();
     // The combination with the first stage of the x inverse (as in k_any_x_inv).
     const int last = sx.nst - 1, P = sx.P[last], half = P / 2 + 1;
-    any_radix_last<Real>(sx.r[last], [&]<int R>() {
+    any_radix_last(sx.r[last], [&]<int R>() {
         for (int e = threadIdx.x; e < a.qx.G * half; e += blockDim.x) {
             const int g = rdiv(e, a.mul_half), f = e - g * half;
             const bool own = f == 0 || 2 * f == P;
@@ -267,11 +267,11 @@ k_plane_inv(const Cx2<Real> *__restrict__ w3, const PtrArray u, const AnyTw<Real
             for (int r = 0; r < R; ++r) any_st(p + r * a.qx.pitch, w[r]);
         }
     });
-    plane_stages<Real, 1>(xb, sx, a.qx, tx, 1, last);
-    plane_first<Real, 1>(xb, sx, a.qx, tx);
+    plane_stages<Real, MR, 1>(xb, sx, a.qx, tx, 1, last);
+    plane_first<Real, MR, 1>(xb, sx, a.qx, tx);
     __syncthreads();
     X2 *plane = reinterpret_cast<X2 *>(const_cast<void *>(u.p[b])) + (long long)z * ny * h;
-    any_radix_even<Real>(sx.r[0], [&]<int R>() {
+    any_radix_even<MR>(sx.r[0], [&]<int R>() {
         for (int e = threadIdx.x; e < a.qx.G * M; e += blockDim.x) {
             const int g = rdiv(e, sx.mulM[0]), j = e - g * M;
             X2 *dst = plane + (long long)W * g * h + j;
@@ -286,8 +286,8 @@ k_plane_inv(const Cx2<Real> *__restrict__ w3, const PtrArray u, const AnyTw<Real
     });
 }
 
-template <typename Real>
-cudaError_t plane_xy(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int B, cudaStream_t s, bool fwd) {
+template <typename Real, int MR>
+cudaError_t plane_run(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int B, cudaStream_t s, bool fwd) {
     const PlaneTile &t = p.plane[std::is_same<Real, DF>::value];
     auto groups = [](int G, int pitch) { return PlaneGroups{G, (unsigned)((1ull << 32) / (unsigned)G + 1), pitch}; };
     PlaneArgs a{t.sx, t.sy, groups(t.gx, t.px), groups(t.gy, t.py), 0u, p.n3[2], p.Px};
@@ -296,13 +296,19 @@ cudaError_t plane_xy(const DevicePlan &p, const PtrArray &rho, const PtrArray &u
     const AnyTw<Real> *ty = static_cast<const AnyTw<Real> *>(p.tw3[1]);
     const int smem = t.smem + any_tw_bytes<Real>(t.sx.L) + any_tw_bytes<Real>(t.sy.L), planes = B * p.n3[2];
     if (fwd) {
-        GSP_CHECK(set_smem(k_plane_fwd<Real>, smem));
-        GSP_CHECK(launch_pdl(k_plane_fwd<Real>, planes, t.threads, smem, s, rho, static_cast<Cx2<Real> *>(p.w2), tx, ty, a));
+        GSP_CHECK(set_smem(k_plane_fwd<Real, MR>, smem));
+        GSP_CHECK(launch_pdl(k_plane_fwd<Real, MR>, planes, t.threads, smem, s, rho, static_cast<Cx2<Real> *>(p.w2), tx, ty, a));
     } else {
-        GSP_CHECK(set_smem(k_plane_inv<Real>, smem));
-        GSP_CHECK(launch_pdl(k_plane_inv<Real>, planes, t.threads, smem, s, static_cast<const Cx2<Real> *>(p.w3), u, tx, ty, a));
+        GSP_CHECK(set_smem(k_plane_inv<Real, MR>, smem));
+        GSP_CHECK(launch_pdl(k_plane_inv<Real, MR>, planes, t.threads, smem, s, static_cast<const Cx2<Real> *>(p.w3), u, tx, ty, a));
     }
     return cudaGetLastError();
+}
+
+template <typename Real>
+cudaError_t plane_xy(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int B, cudaStream_t s, bool fwd) {
+    const PlaneTile &t = p.plane[std::is_same<Real, DF>::value];
+    return any_with_radix<Real>(t.mr, [&]<int MR>() { return plane_run<Real, MR>(p, rho, u, B, s, fwd); });
 }
 
 }  // namespace gsp

@@ -61,3 +61,16 @@ extern "C" int shim_any_transform(int L, int max_radix, int max_last, int pad, c
     }
     return 0;
 }
+
+// The schedule and the kernel's largest radix that the passes of length L take: 0, or 1 if a
+// radix is above it, 2 if 12 is taken where 10 gives no more stages, 3 if a stage is wasted.
+extern "C" int shim_any_radix_rule(int L, int max_radix, int max_last, int pad) {
+    int mr = 0;
+    const gsp::AnySched s = gsp::any_sched_of(L, max_radix, max_last, pad != 0, &mr);
+    const gsp::AnySched a = gsp::any_sched(L, 10, std::min(max_last, 10), pad != 0);
+    const gsp::AnySched b = gsp::any_sched(L, max_radix, max_last, pad != 0);
+    for (int st = 0; st < s.nst; ++st)
+        if (s.r[st] > mr) return 1;
+    if (mr > 10 && s.nst >= a.nst) return 2;
+    return s.nst == std::min(a.nst, b.nst) ? 0 : 3;
+}

@@ -50,3 +50,13 @@ def test_every_length_is_a_dft(shim, max_radix, rows, pad):
         assert rc == 0, (L, rc)
         ref = np.fft.fft(x.view(complex))
         assert np.abs(X.view(complex) - ref).max() <= 1e-12 * np.abs(ref).max() * np.log2(L), L
+
+
+@pytest.mark.parametrize("max_radix", [10, 12])
+@pytest.mark.parametrize("rows", [0, 1])
+def test_kernel_covers_the_radices(shim, max_radix, rows):
+    """Radix 12 only where it saves a stage, and never in a kernel compiled up to 10."""
+    for n in counts():
+        L = n if rows else 2 * n
+        for pad in (0, 1):
+            assert shim.shim_any_radix_rule(L, max_radix, 8 if rows else max_radix, pad) == 0, L
