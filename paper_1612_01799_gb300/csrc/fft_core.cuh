@@ -147,12 +147,20 @@ __device__ __forceinline__ CD cadd(CD a, CD b) { return {a.re + b.re, a.im + b.i
 __device__ __forceinline__ CD csub(CD a, CD b) { return {a.re - b.re, a.im - b.im}; }
 __device__ __forceinline__ CV cadd(CV a, CV b) { return {f2add(a.re, b.re), f2add(a.im, b.im)}; }
 __device__ __forceinline__ CV csub(CV a, CV b) { return {f2sub(a.re, b.re), f2sub(a.im, b.im)}; }
-// The two double-float sums of a complex sum in one: the real and the imaginary part take the
+// The two double-float sums of a complex sum: plainly, part by part, in the translation units that
+// define GSP_DF_PLAIN_SUMS, else in one: the real and the imaginary part take the
 // steps of DF's operator+ (the same roundings, the same result) side by side in packed FP32x2
 // instructions, five and six selects and compares in place of ten and six.  The FMA pipe takes
 // a packed instruction in two cycles, so what this saves is issue slots and code size: the
 // compiled-length z pass at N = 128 went from 141 to 136 us, the runtime-length one at
-// N = 162, whose stages compete for the instruction cache, from 480 to 428 us.
+// N = 162, whose stages compete for the instruction cache, from 480 to 428 us.  Where the code
+// fits the cache the register pairs it ties together cost more than that: FP64 plans' solves,
+// packed and plain, N = 160 654 and 649 us, 192 957 and 951, 256 2000 and 1991, 384 8086 and
+// 7727, 512 19.48 and 18.47 ms, 1024 201.1 and 196.6 ms; but N = 96 128 and 135 us, N = 128 249.0
+// and 250.6, and N = 320, whose length 640 holds 20 values a thread, 6.97 and 7.98 ms.
+#ifdef GSP_DF_PLAIN_SUMS
+__device__ __forceinline__ CDF cadd(CDF a, CDF b) { return {a.re + b.re, a.im + b.im}; }
+#else
 __device__ __forceinline__ CDF cadd(CDF a, CDF b) {
     const bool p = fabsf(b.re.hi) > fabsf(a.re.hi), q = fabsf(b.im.hi) > fabsf(a.im.hi);
     const float2 x = f2(p ? b.re.hi : a.re.hi, q ? b.im.hi : a.im.hi);
@@ -161,6 +169,7 @@ __device__ __forceinline__ CDF cadd(CDF a, CDF b) {
     const float2 l = f2add(e, f2add(f2(a.re.lo, a.im.lo), f2(b.re.lo, b.im.lo)));
     return {DF(s.x, l.x), DF(s.y, l.y)};
 }
+#endif
 __device__ __forceinline__ CDF csub(CDF a, CDF b) { return cadd(a, CDF{-b.re, -b.im}); }
 
 __device__ __forceinline__ CF cscale(CF a, float s) { return {a.re * s, a.im * s}; }

@@ -1153,9 +1153,9 @@ cudaError_t encode_n(DevicePlan &p) {
 #define GSP_DF_GROUP_4(X) X(96) X(128)
 #define GSP_DF_GROUP_5(X) X(160) X(192)
 #define GSP_DF_GROUP_6(X) X(256)
-#define GSP_DF_GROUP_7(X) X(320) X(384)
+#define GSP_DF_GROUP_7(X) X(320)
 #define GSP_DF_GROUP_8(X) X(512)
-#define GSP_DF_GROUP_9(X) X(1024)
+#define GSP_DF_GROUP_9(X) X(384) X(1024)
 #define GSP_DECLARE_N(EXT, Real, n)                                                                      \
     EXT template cudaError_t solve_n<Real, n>(const DevicePlan &, const PtrArray &, const PtrArray &, int, \
                                               cudaStream_t, cudaEvent_t *, double *, int);                 \

@@ -1,4 +1,4 @@
-// Double-float dispatch of the solve passes (the per-N code is in passes_df_[abc].cu): the
+// Double-float dispatch of the solve passes (the per-N code is in passes_df_1.cu to passes_df_9.cu): the
 // FP64 path's arithmetic on the FP32 pipe (type DF of fft_core.cuh), FP64 at the boundary.
 #include "passes.cuh"
 
