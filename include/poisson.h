@@ -110,10 +110,11 @@ int poisson_plan_create_box(poisson_plan *out, int N, double Lx, double Ly, doub
  * arrays, x fastest (index i + nx (j + ny k)).  Each n_q must be even, 4 <= n_q <= 1024,
  * with no prime factor above 5 (else POISSON_ERR_ARG or POISSON_ERR_UNSUPPORTED).  With
  * nx = ny = nz this is poisson_plan_create_box.  Plans whose counts differ (or whose common
- * count has no compiled transform schedule, poisson_supported_n() == 2) run the
- * runtime-length forms of the five passes: one form per pass (the form knobs have only
- * value 0; small planes take the x and y passes of a direction in one kernel), the same
- * arithmetics, no TMA staging.  poisson_plan_axis_table returns the x
+ * count has no compiled transform schedule, poisson_supported_n() == 2) have one form per pass
+ * (the form knobs have only value 0) and the same arithmetics.  An axis whose count has a
+ * compiled schedule runs its pass in the block form of that length, the others in the
+ * runtime-length forms; small planes take the x and y passes of a direction in one kernel.
+ * poisson_plan_axis_table returns the x
  * axis's factors (n_terms x (nx + 1)).  Other arguments, errors and use as for
  * poisson_plan_create (one density per solve).
  */
