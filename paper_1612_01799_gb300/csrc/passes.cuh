@@ -606,9 +606,14 @@ __global__ void k_symbol_table(Real *__restrict__ sym, const double *__restrict_
     }
 }
 
+// Opens a kernel to a launch with `bytes` of dynamic shared memory.  The limit belongs to the
+// kernel, not to the launch, and plans of several sizes may launch it from several host threads:
+// it always takes the same value, all that a block may have (the pass kernels hold no static
+// shared memory), so that no thread lowers it between another's call here and its launch.  What
+// runs side by side on an SM follows from the launch's own size.
 template <class K> static cudaError_t set_smem(K kernel, size_t bytes) {
     if (bytes <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBlockSmemMax);
 }
 
 #define GSP_CHECK(x)                          \

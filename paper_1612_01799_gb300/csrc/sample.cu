@@ -197,15 +197,17 @@ extern "C" int poisson_sample_gaussians(int N, double L, int ng, const double *p
     if (dtype != POISSON_F32 && dtype != POISSON_F64) return POISSON_ERR_ARG;
     const size_t smem = (size_t)2 * ng * N * sizeof(double);
     cudaStream_t s = (cudaStream_t)stream;
-    // The kernel also has a little static shared memory: opt in above 32 KB of dynamic.
+    // The kernel also has a little static shared memory: opt in above 32 KB of dynamic, always to
+    // the most that any call takes, whatever N another thread samples.
+    const int most = 2 * kMaxG * 1024 * (int)sizeof(double);
     cudaError_t ea = cudaSuccess;
     if (dtype == POISSON_F32) {
         if (smem > 32 * 1024)
-            ea = cudaFuncSetAttribute(k_sample<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            ea = cudaFuncSetAttribute(k_sample<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (ea == cudaSuccess) k_sample<float><<<N, 256, smem, s>>>(G, N, L, static_cast<float *>(out_d));
     } else {
         if (smem > 32 * 1024)
-            ea = cudaFuncSetAttribute(k_sample<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            ea = cudaFuncSetAttribute(k_sample<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (ea == cudaSuccess) k_sample<double><<<N, 256, smem, s>>>(G, N, L, static_cast<double *>(out_d));
     }
     if (ea != cudaSuccess) {

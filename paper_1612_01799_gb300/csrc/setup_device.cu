@@ -131,7 +131,8 @@ cudaError_t launch_axis_table(const double *dtau, const double *dgl, int S, int 
     const int P = axis_table_panels(N);
     const size_t smem = (size_t)16 * P * sizeof(double);
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_axis_table, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // always the same limit, whatever N another thread's plan has
+        cudaError_t e = cudaFuncSetAttribute(k_axis_table, cudaFuncAttributeMaxDynamicSharedMemorySize, kBlockSmemMax);
         if (e != cudaSuccess) return e;
     }
     const dim3 grid((N + 1 + 127) / 128, S);

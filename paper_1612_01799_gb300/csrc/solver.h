@@ -120,6 +120,9 @@ inline bool plane_n_plan(const DevicePlan &p) {
     return p.plane_small && p.xform == 0 && p.yform == 0 && p.xyform == 0;
 }
 
+// Largest shared memory of one block (227 KB).
+constexpr int kBlockSmemMax = 232448;
+
 // Record a failed CUDA call for poisson_last_cuda_error() (per host thread).
 void note_cuda_error(cudaError_t e);
 
