@@ -230,19 +230,19 @@ template <typename Real> __host__ __device__ constexpr int any_tw_bytes(int L) {
     return AnyTwiddles<Real>::kCopy ? (L * (int)sizeof(AnyTw<Real>) + 15) / 16 * 16 : 0;
 }
 
-// Butterfly of a stage in the middle of a transform (also its last one when TW is false),
-// in place over slots p[r * step], with the twiddles W_L^{e r} of the shared table tw.
-template <int R, int D, bool TW, typename C, typename Tw>
-__device__ __forceinline__ void any_stage(float4 *p, int step, const Tw &tw, int e) {
+// Butterfly of a stage in the middle of a transform, in place over slots p[r * step], with the
+// twiddles W_L^{e r} of the shared table tw.
+template <int R, int D, typename C, typename Tw>
+__device__ __forceinline__ void any_stage(float4 *p, int step, const Tw &tw, int e, C) {
     C v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = any_ld(p + r * step, C{});
-    if constexpr (TW && D > 0) {
+    if constexpr (D > 0) {
 #pragma unroll
         for (int r = 1; r < R; ++r) v[r] = any_twmul<1>(v[r], tw[r * e]);
     }
     dft<R, D>(v);
-    if constexpr (TW && D < 0) {
+    if constexpr (D < 0) {
 #pragma unroll
         for (int r = 1; r < R; ++r) v[r] = any_twmul<-1>(v[r], tw[r * e]);
     }
@@ -250,7 +250,7 @@ __device__ __forceinline__ void any_stage(float4 *p, int step, const Tw &tw, int
     for (int r = 0; r < R; ++r) any_st(p + r * step, v[r]);
 }
 
-// The stages st0 <= st < st1 of a tile of 2^lg groups (slot a of group g at buf[a * PG + g]),
+// The middle stages st0 <= st < st1 of a tile of 2^lg groups (slot a of group g at buf[a * PG + g]),
 // forward in ascending and inverse in descending order, each behind a block barrier.
 // twstride: the table holds exp(-2 pi i e / (L twstride)).
 template <typename Real, int MR, int D>
@@ -262,13 +262,11 @@ __device__ __forceinline__ void any_stages(float4 *buf, const AnySched &s, int l
         const int st = D < 0 ? i : st0 + st1 - 1 - i;
         __syncthreads();
         const int R = s.r[st], nb = s.P[st] * s.M[st], step = s.S[st] * PG;
-        const bool last = st == s.nst - 1;
         any_radix<MR>(R, [&]<int RR>() {
             for (int b = threadIdx.x >> lg; b < nb; b += blockDim.x >> lg) {
                 const AnyBfly f = any_bfly(s, st, b);
                 float4 *p = buf + f.slot * PG + g;
-                if (last) any_stage<RR, D, false, C>(p, step, tw, 0);
-                else any_stage<RR, D, true, C>(p, step, tw, f.lo * s.P[st]);
+                any_stage<RR, D>(p, step, tw, f.lo * s.P[st], C{});
             }
         });
     }

@@ -37,7 +37,7 @@ __device__ __forceinline__ void plane_stages(float4 *buf, const AnySched &s, con
         any_radix<MR>(s.r[st], [&]<int R>() {
             plane_each(s.P[st] * s.M[st], q, [&](int b, int g) {
                 const AnyBfly f = any_bfly(s, st, b);
-                any_stage<R, D, true, C>(buf + f.slot * q.pitch + g, s.S[st] * q.pitch, tw, f.lo * s.P[st]);
+                any_stage<R, D>(buf + f.slot * q.pitch + g, s.S[st] * q.pitch, tw, f.lo * s.P[st], C{});
             });
         });
     }
