@@ -106,12 +106,21 @@ constexpr int any_max_warps(bool f32) { return f32 ? 24 : 16; }
 constexpr int kAnyRowsLast = 8;
 
 // Tile of a runtime-length pass: its schedule, 2^lg 16-byte groups, slots pitch groups apart,
-// threads, bytes of shared memory, largest radix of its kernel.
+// threads (few: where all tiles of a launch are resident at once, few_ctas to an SM), bytes of
+// shared memory, largest radix of its kernel.
 struct AnyTile {
     AnySched s;
-    int lg, pitch, threads, smem, mr;
+    int lg, pitch, threads, few, few_ctas, smem, mr;
 };
 constexpr int kAnyThreads = 256;  // threads the kernels are compiled for
+// Whether a launch of ntiles tiles lasts as long as one CTA: all tiles are resident at once, with at
+// most three warps to a scheduler.  Then the threads with the fewest rounds over the butterflies
+// serve it best, not those that fill an SM with CTAs (double-float solves: N = 36 39.4 -> 36.5 us,
+// 40 42.0 -> 39.2, box 12 x 200 x 12 44.5 -> 40.2; with more warps it loses, FP64 N = 50 152.9 ->
+// 154.0, where the rule leaves the threads as they are).
+inline bool any_is_few(const AnyTile &t, int sms, int ntiles) {
+    return ntiles <= sms * t.few_ctas && (long long)ntiles * t.few <= (long long)sms * 384;
+}
 
 // rows: an x pass (one more group of pitch, odd slot strides: conflict-free for neighbouring
 // groups and for neighbouring samples alike); else a column pass (eight groups fill a 128-byte
@@ -120,15 +129,22 @@ constexpr int kAnyThreads = 256;  // threads the kernels are compiled for
 // four; N = 162 243 and 275 us; N = 400, where only two CTAs of eight fit, 2.86 and 2.83 ms).
 // Threads: the multiple of 32 with the most threads of
 // an SM at work, counting the share of thread slots that the rounds over the butterflies of
-// each stage fill and the CTAs that shared memory and max_warps (by registers) admit.
-inline AnyTile any_tile(int L, int max_radix, int max_warps, bool rows) {
+// each stage fill and the CTAs that shared memory and registers admit; few: see any_is_few.
+inline AnyTile any_tile(int L, int max_radix, bool f32, bool rows) {
     AnyTile t{};
-    const int max_last = rows ? kAnyRowsLast : max_radix;
+    const int max_last = rows ? kAnyRowsLast : max_radix, max_warps = any_max_warps(f32);
     const AnySched wide = any_sched_of(L, max_radix, max_last, rows, &t.mr);
     t.lg = wide.slots * (rows ? 9 : 8) * 16 <= 70 * 1024 ? 3 : 2;
     t.s = t.lg == 3 ? wide : any_sched_of(L, max_radix, max_last, true, &t.mr);
     t.pitch = (1 << t.lg) + (rows ? 1 : 0);
     t.smem = t.s.slots * t.pitch * 16;
+    auto rounds_of = [&](int n) {
+        int rounds = 0;
+        for (int st = 0; st < t.s.nst; ++st) rounds += (((L / t.s.r[st]) << t.lg) + n - 1) / n * t.s.r[st];
+        // the Hermitian split on its own, two values an item
+        return rows ? rounds + (((L / 2 + 1) << t.lg) + n - 1) / n * 2 : rounds;
+    };
+    auto ctas_of = [&](int n) { return std::min(232448 / (t.smem + L * 16 + 1024), max_warps * 32 / n); };
     double best = 0.0;
     for (int n = kAnyThreads; n >= 64; n -= 32) {
         double slots = 0.0, used = 0.0;
@@ -137,13 +153,18 @@ inline AnyTile any_tile(int L, int max_radix, int max_warps, bool rows) {
             slots += (double)((items + n - 1) / n) * n * t.s.r[st];
             used += (double)items * t.s.r[st];
         }
-        const int ctas = std::min(232448 / (t.smem + L * 16 + 1024), max_warps * 32 / n);
-        const double score = used / slots * ctas * n;
+        const double score = used / slots * ctas_of(n) * n;
         if (score > best * 1.02 || n == kAnyThreads) {
             best = score;
             t.threads = n;
         }
     }
+    t.few = t.threads;
+    for (int n = kAnyThreads; n >= 64; n -= 32) {
+        const int less = rounds_of(n) - rounds_of(t.few);
+        if (less < 0 || (less == 0 && t.few != t.threads)) t.few = n;
+    }
+    t.few_ctas = ctas_of(t.few);
     return t;
 }
 
@@ -158,10 +179,10 @@ struct PlaneTile {
 constexpr int kPlaneThreads = 384;
 // Largest plane: in FP32 two CTAs fit an SM (solves, separate passes against the plane kernels:
 // 20^3 21.4 and 18.9 us, 60^3 27.2 and 25.5, 64 x 64 x 256 66 and 57, but 72^3 28.6 and 30.2); the
-// wider arithmetics are bound by the longer chain of one CTA soon (20^3 30.6 and 28.7, 36^3 39.6
-// and 41.2).  Cubes whose passes are compiled for their length stay with those (32^3 12.6 and
-// 18.6 us).
-constexpr int plane_smem(bool f32) { return f32 ? 106 * 1024 : 48 * 1024; }
+// wider arithmetics are bound by the longer chain of one CTA soon (double-float 10^3 24.3 and
+// 20.8 us, 18^3 27.4 and 27.4, 20^3 25.9 and 28.5, 30^3 32.0 and 36.6).  Cubes whose passes are
+// compiled for their length have kernels of their own (plane_n_size).
+constexpr int plane_smem(bool f32) { return f32 ? 106 * 1024 : 18 * 1024; }
 inline PlaneTile plane_tile(int nx, int ny, int max_radix, int w) {
     PlaneTile t{};
     t.sx = any_sched_of(nx, max_radix, kAnyRowsLast, true, &t.mr);

@@ -69,11 +69,12 @@ bool n_any(int N) {
 void any_plan_tiles(DevicePlan &p) {
     const bool f32 = p.dtype == POISSON_F32;
     p.plane_small = !p.any && plane_n_size(p.N, !f32);
+    const int W = f32 ? 2 : 1, nx = p.n3[0], ny = p.n3[1];
     for (int df = 0; df < 2; ++df) {
-        for (int q = 0; q < 3; ++q)
-            p.any_tile[df][q] = any_tile(q == 0 ? p.n3[0] : 2 * p.n3[q], any_max_radix(df != 0), any_max_warps(f32), q == 0);
-        p.plane[df] = plane_tile(p.n3[0], p.n3[1], any_max_radix(df != 0), f32 ? 2 : 1);
-        p.plane[df].on = p.plane[df].on && p.any && !(n_supported(p.n3[0]) && n_supported(p.n3[1]));
+        const int R = any_max_radix(df != 0);
+        for (int q = 0; q < 3; ++q) p.any_tile[df][q] = any_tile(q == 0 ? nx : 2 * p.n3[q], R, f32, q == 0);
+        p.plane[df] = plane_tile(nx, ny, R, W);
+        if (!p.any || (n_supported(nx) && n_supported(ny))) p.plane[df].on = false;
     }
     for (int q = 0; q < 3; ++q) p.axn[q] = p.any && n_supported(p.n3[q]) ? p.n3[q] : 0;
 }
@@ -531,6 +532,7 @@ static int plan_create_impl(poisson_plan *out, const int *n3, double L, const do
         return rc;
     }
     cudaError_t e = cudaGetDevice(&p->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->dp.sms, cudaDevAttrMultiProcessorCount, p->device);
     if (e != cudaSuccess) {
         delete p;
         return map_cuda(e);

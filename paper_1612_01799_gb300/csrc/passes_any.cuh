@@ -317,6 +317,27 @@ __device__ __forceinline__ void any_first_adj(const float4 *buf, const AnySched 
     });
 }
 
+// The last radix stage on its own, in place without twiddles, behind a block barrier; another one
+// follows it.
+template <typename Real, int D>
+__device__ __forceinline__ void any_last(float4 *buf, const AnySched &s, int lg, int PG) {
+    using C = typename Types<Real>::CC;
+    const int g = threadIdx.x & ((1 << lg) - 1), last = s.nst - 1;
+    __syncthreads();
+    any_radix_last(s.r[last], [&]<int R>() {
+        for (int b = threadIdx.x >> lg; b < s.P[last]; b += blockDim.x >> lg) {
+            float4 *p = buf + any_bfly(s, last, b).slot * PG + g;
+            C v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = any_ld(p + r * PG, C{});
+            dft<R, D>(v);
+#pragma unroll
+            for (int r = 0; r < R; ++r) any_st(p + r * PG, v[r]);
+        }
+    });
+    __syncthreads();
+}
+
 // Blocks per SM the kernels are compiled for.
 template <typename Real> constexpr int kAnyMinBlocks = sizeof(typename Types<Real>::CS) == 8 ? 3 : 2;
 
@@ -328,7 +349,7 @@ template <typename Real> constexpr int kAnyMinBlocks = sizeof(typename Types<Rea
 // nx-point complex FFT of the (even, odd) sample pairs (pairs >= nx/2 zero) and the Hermitian
 // split into the nx + 1 bins (twiddles W_{2nx}^k; the nx-point FFT reads the same table at
 // stride 2).
-template <typename Real, int MR>
+template <typename Real, int MR, bool SPLIT>
 __global__ void __launch_bounds__(kAnyThreads, kAnyMinBlocks<Real>)
 k_any_x_fwd(const PtrArray rho, Cx2<Real> *__restrict__ out, const AnyTw<Real> *__restrict__ tw,
             const __grid_constant__ AnySched s, int rows_b, int nrows, int Px, unsigned mul_half, int lg, int ntiles) {
@@ -388,45 +409,59 @@ k_any_x_fwd(const PtrArray rho, Cx2<Real> *__restrict__ out, const AnyTw<Real> *
         }
         const int last = s.nst - 1, P = s.P[last], half = P / 2 + 1;
         any_stages<Real, MR, -1>(buf, s, lg, PG, ts, 1, last);
-        __syncthreads();
-        // The last stage with the split, neighbouring frequencies in a warp: butterfly f makes the
-        // bins k = f + r P, its partner P - f the bins n - k.
-        // X_k = Ev_k + W_{2n}^k Od_k, X_{n-k} = conj(Ev_k - W_{2n}^k Od_k), with Ev, Od the DFTs
-        // of the even and odd samples from C_k and conj C_{n-k}.
-        any_radix_last(s.r[last], [&]<int R>() {
-            for (int e = threadIdx.x; e < ng * half; e += blockDim.x) {
-                const int g = rdiv(e, mul_half), f = e - g * half;
-                const bool own = f == 0 || 2 * f == P;  // n - k lies in butterfly f itself
-                C v[R], w[R];
-                const float4 *p = buf + any_freq_slot(s, f) * PG + g;
+        if constexpr (SPLIT) {
+            any_last<Real, -1>(buf, s, lg, PG);
+            for (int e = threadIdx.x; e < ng * (h + 1); e += blockDim.x) {
+                const int g = rdiv(e, mul_half), k = e - g * (h + 1);
+                const C ck = any_ld(buf + any_freq_slot(s, k) * PG + g, C{});
+                const C cn = any_conj(any_ld(buf + any_freq_slot(s, k ? n - k : 0) * PG + g, C{}));
+                const C ev = any_half(cadd(ck, cn)), od = any_half(cmul_mi(csub(ck, cn)));
+                const C wo = any_twmul<-1>(od, __ldg(tw + k));
+                Cx2<Real> *dst = out + (r0 + g) * Px;
+                dst[k] = any_ws(cadd(ev, wo), 0);
+                if (2 * k != n) dst[n - k] = any_ws(any_conj(csub(ev, wo)), 0);
+            }
+        } else {
+            __syncthreads();
+            // The last stage with the split, neighbouring frequencies in a warp: butterfly f makes the
+            // bins k = f + r P, its partner P - f the bins n - k.
+            // X_k = Ev_k + W_{2n}^k Od_k, X_{n-k} = conj(Ev_k - W_{2n}^k Od_k), with Ev, Od the DFTs
+            // of the even and odd samples from C_k and conj C_{n-k}.
+            any_radix_last(s.r[last], [&]<int R>() {
+                for (int e = threadIdx.x; e < ng * half; e += blockDim.x) {
+                    const int g = rdiv(e, mul_half), f = e - g * half;
+                    const bool own = f == 0 || 2 * f == P;  // n - k lies in butterfly f itself
+                    C v[R], w[R];
+                    const float4 *p = buf + any_freq_slot(s, f) * PG + g;
 #pragma unroll
-                for (int r = 0; r < R; ++r) v[r] = any_ld(p + r * PG, C{});
-                dft<R, -1>(v);
-                if (own) {
+                    for (int r = 0; r < R; ++r) v[r] = any_ld(p + r * PG, C{});
+                    dft<R, -1>(v);
+                    if (own) {
 #pragma unroll
-                    for (int r = 0; r < R; ++r) w[r] = f == 0 ? v[(r + 1) % R] : v[r];
-                } else {
-                    p = buf + any_freq_slot(s, P - f) * PG + g;
+                        for (int r = 0; r < R; ++r) w[r] = f == 0 ? v[(r + 1) % R] : v[r];
+                    } else {
+                        p = buf + any_freq_slot(s, P - f) * PG + g;
 #pragma unroll
-                    for (int r = 0; r < R; ++r) w[r] = any_ld(p + r * PG, C{});
-                    dft<R, -1>(w);
-                }
-                Cx2<Real> *dst = out + (r0 + W * g) * Px;
+                        for (int r = 0; r < R; ++r) w[r] = any_ld(p + r * PG, C{});
+                        dft<R, -1>(w);
+                    }
+                    Cx2<Real> *dst = out + (r0 + W * g) * Px;
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int k = f + r * P;
-                    const C ck = v[r], cn = any_conj(w[R - 1 - r]);
-                    const C ev = any_half(cadd(ck, cn)), od = any_half(cmul_mi(csub(ck, cn)));
-                    const C wo = any_twmul<-1>(od, __ldg(tw + k));
-                    const C lo = cadd(ev, wo), hi = any_conj(csub(ev, wo));
+                    for (int r = 0; r < R; ++r) {
+                        const int k = f + r * P;
+                        const C ck = v[r], cn = any_conj(w[R - 1 - r]);
+                        const C ev = any_half(cadd(ck, cn)), od = any_half(cmul_mi(csub(ck, cn)));
+                        const C wo = any_twmul<-1>(od, __ldg(tw + k));
+                        const C lo = cadd(ev, wo), hi = any_conj(csub(ev, wo));
 #pragma unroll
-                    for (int i = 0; i < W; ++i) {
-                        dst[(long long)i * Px + k] = any_ws(lo, i);
-                        if (!own || k == 0) dst[(long long)i * Px + n - k] = any_ws(hi, i);
+                        for (int i = 0; i < W; ++i) {
+                            dst[(long long)i * Px + k] = any_ws(lo, i);
+                            if (!own || k == 0) dst[(long long)i * Px + n - k] = any_ws(hi, i);
+                        }
                     }
                 }
-            }
-        });
+            });
+        }
     }
 }
 
@@ -434,7 +469,7 @@ k_any_x_fwd(const PtrArray rho, Cx2<Real> *__restrict__ out, const AnyTw<Real> *
 // The nx + 1 Hermitian bins of each row -> C_k = Ev_k + i Od_k (Ev_k = Y_k + conj Y_{n-k},
 // Od_k = (Y_k - conj Y_{n-k}) W_{2n}^{-k}), the inverse nx-point FFT gives y_{2m} + i y_{2m+1};
 // pairs m < nx/2 are kept (the crop).  Shared layout as in the forward.
-template <typename Real, int MR>
+template <typename Real, int MR, bool SPLIT>
 __global__ void __launch_bounds__(kAnyThreads, kAnyMinBlocks<Real>)
 k_any_x_inv(const Cx2<Real> *__restrict__ in, const PtrArray u, const AnyTw<Real> *__restrict__ tw,
             const __grid_constant__ AnySched s, int rows_b, int nrows, int Px, unsigned mul_half, int lg, int ntiles) {
@@ -452,46 +487,67 @@ k_any_x_inv(const Cx2<Real> *__restrict__ in, const PtrArray u, const AnyTw<Real
         const int ng = (int)min((long long)NG, (nrows - r0) / W);
         // The combination with the first stage of the inverse, as the forward's last one.
         const int last = s.nst - 1, P = s.P[last], half = P / 2 + 1;
-        any_radix_last(s.r[last], [&]<int R>() {
-            for (int e = threadIdx.x; e < NG * half; e += blockDim.x) {
-                const int g = rdiv(e, mul_half), f = e - g * half;
-                const bool own = f == 0 || 2 * f == P;
-                const Cx2<Real> *src = in + (r0 + W * g) * Px;
-                C v[R], w[R];
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int k = f + r * P;
-                    v[r] = w[r] = czero<C>();
-                    if (g < ng) {
-                        v[r] = any_wpack(__ldg(src + k), __ldg(src + (W - 1) * Px + k), C{});
-                        w[r] = any_wpack(__ldg(src + n - k), __ldg(src + (W - 1) * Px + n - k), C{});
-                    }
+        if constexpr (SPLIT) {
+            for (int e = threadIdx.x; e < NG * (h + 1); e += blockDim.x) {
+                const int g = rdiv(e, mul_half), k = e - g * (h + 1);
+                const Cx2<Real> *src = in + (r0 + g) * Px;
+                C yk = czero<C>(), yn = czero<C>();
+                if (g < ng) {
+                    yk = any_wpack(__ldg(src + k), __ldg(src + k), C{});
+                    yn = any_wpack(__ldg(src + n - k), __ldg(src + n - k), C{});
                 }
-                if (f == 0) {  // Y_0 and Y_n are real: drop what rounding left in their imaginary parts
-                    v[0].im = czero<C>().re;
-                    w[0].im = czero<C>().re;
+                if (k == 0) {  // Y_0 and Y_n are real, as below
+                    yk.im = czero<C>().re;
+                    yn.im = czero<C>().re;
                 }
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const C cn = any_conj(w[r]), ev = cadd(v[r], cn);
-                    const C od = any_twmul<1>(csub(v[r], cn), __ldg(tw + f + r * P));
-                    v[r] = add_rot<1>(ev, od);
-                    w[r] = add_rot<1>(any_conj(ev), any_conj(od));
-                }
-                dft<R, 1>(v);
-                float4 *p = buf + any_freq_slot(s, f) * PG + g;
-#pragma unroll
-                for (int r = 0; r < R; ++r) any_st(p + r * PG, v[r]);
-                if (own) continue;
-                C x[R];
-#pragma unroll
-                for (int r = 0; r < R; ++r) x[r] = w[R - 1 - r];
-                dft<R, 1>(x);
-                p = buf + any_freq_slot(s, P - f) * PG + g;
-#pragma unroll
-                for (int r = 0; r < R; ++r) any_st(p + r * PG, x[r]);
+                const C cn = any_conj(yn), ev = cadd(yk, cn), od = any_twmul<1>(csub(yk, cn), __ldg(tw + k));
+                any_st(buf + any_freq_slot(s, k) * PG + g, add_rot<1>(ev, od));
+                if (k > 0 && 2 * k != n)
+                    any_st(buf + any_freq_slot(s, n - k) * PG + g, add_rot<1>(any_conj(ev), any_conj(od)));
             }
-        });
+            any_last<Real, 1>(buf, s, lg, PG);
+        } else {
+            any_radix_last(s.r[last], [&]<int R>() {
+                for (int e = threadIdx.x; e < NG * half; e += blockDim.x) {
+                    const int g = rdiv(e, mul_half), f = e - g * half;
+                    const bool own = f == 0 || 2 * f == P;
+                    const Cx2<Real> *src = in + (r0 + W * g) * Px;
+                    C v[R], w[R];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const int k = f + r * P;
+                        v[r] = w[r] = czero<C>();
+                        if (g < ng) {
+                            v[r] = any_wpack(__ldg(src + k), __ldg(src + (W - 1) * Px + k), C{});
+                            w[r] = any_wpack(__ldg(src + n - k), __ldg(src + (W - 1) * Px + n - k), C{});
+                        }
+                    }
+                    if (f == 0) {  // Y_0 and Y_n are real: drop what rounding left in their imaginary parts
+                        v[0].im = czero<C>().re;
+                        w[0].im = czero<C>().re;
+                    }
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const C cn = any_conj(w[r]), ev = cadd(v[r], cn);
+                        const C od = any_twmul<1>(csub(v[r], cn), __ldg(tw + f + r * P));
+                        v[r] = add_rot<1>(ev, od);
+                        w[r] = add_rot<1>(any_conj(ev), any_conj(od));
+                    }
+                    dft<R, 1>(v);
+                    float4 *p = buf + any_freq_slot(s, f) * PG + g;
+#pragma unroll
+                    for (int r = 0; r < R; ++r) any_st(p + r * PG, v[r]);
+                    if (own) continue;
+                    C x[R];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) x[r] = w[R - 1 - r];
+                    dft<R, 1>(x);
+                    p = buf + any_freq_slot(s, P - f) * PG + g;
+#pragma unroll
+                    for (int r = 0; r < R; ++r) any_st(p + r * PG, x[r]);
+                }
+            });
+        }
         any_stages<Real, MR, 1>(buf, s, lg, PG, ts, 1, last);
         __syncthreads();
         {

@@ -53,10 +53,11 @@ struct DevicePlan {
     void *twc3[2] = {nullptr, nullptr};
     // Tiles of the runtime-length passes along x, y and z, per arithmetic (any_plan_tiles).
     AnyTile any_tile[2][3] = {};
+    int sms = 1;  // SMs of the plan's device
     // Compiled-length plans with small planes: the x and y passes in one kernel per direction
     // (the allocation-free solve leaves it false).
     bool plane_small = false;
-    // The x and y passes as one kernel per direction (passes_plane.cuh), per arithmetic: on for
+    // The x and y passes as one kernel per direction (passes_plane.cuh), per arithmetic, for
     // runtime-length plans whose planes are small (plane_on).
     PlaneTile plane[2] = {};
     int Px = 0;

@@ -74,3 +74,36 @@ extern "C" int shim_any_radix_rule(int L, int max_radix, int max_last, int pad) 
     if (mr > 10 && s.nst >= a.nst) return 2;
     return s.nst == std::min(a.nst, b.nst) ? 0 : 3;
 }
+
+// The tile of a pass: lg, threads, few, few_ctas, bytes of shared memory with the twiddles, the weighted
+// rounds over the butterflies (and, for rows, over the Hermitian split) with `threads` and with `few`.
+// 0, or 1 if the schedule does not multiply up to L.
+extern "C" int shim_any_tile(int L, int df, int f32, int rows, long long groups, int planes, int sms, int *out) {
+    (void)groups, (void)planes, (void)sms;
+    const gsp::AnyTile t = gsp::any_tile(L, gsp::any_max_radix(df != 0), f32 != 0, rows != 0);
+    int prod = 1;
+    for (int st = 0; st < t.s.nst; ++st) prod *= t.s.r[st];
+    if (t.s.nst < 2 || prod != L || t.smem != t.s.slots * t.pitch * 16) return 1;
+    auto rounds = [&](int n) {
+        int v = rows ? (((L / 2 + 1) << t.lg) + n - 1) / n * 2 : 0;
+        for (int st = 0; st < t.s.nst; ++st) v += (((L / t.s.r[st]) << t.lg) + n - 1) / n * t.s.r[st];
+        return v;
+    };
+    const int v[] = {t.lg, t.threads, t.few, t.few_ctas, t.smem + (f32 ? L * 8 + 8 : 0), rounds(t.threads), rounds(t.few)};
+    std::copy(v, v + 7, out);
+    return 0;
+}
+// Whether a launch of ntiles tiles of that pass takes `few`.
+extern "C" int shim_any_is_few(int threads, int ctas, int sms, int ntiles) {
+    gsp::AnyTile t{};
+    t.few = threads;
+    t.few_ctas = ctas;
+    return gsp::any_is_few(t, sms, ntiles);
+}
+// The plane kernels' tile: on, threads, bytes of shared memory with the twiddles.
+extern "C" int shim_plane_tile(int nx, int ny, int df, int f32, int *out) {
+    const gsp::PlaneTile t = gsp::plane_tile(nx, ny, gsp::any_max_radix(df != 0), f32 ? 2 : 1);
+    const int v[] = {t.on, t.threads, t.smem + (f32 ? (nx + 2 * ny) * 8 + 16 : 0)};
+    std::copy(v, v + 3, out);
+    return 0;
+}

@@ -23,6 +23,22 @@ def counts():
             yield n
 
 
+SMS = 152
+TILE = ("lg", "threads", "few", "ctas", "smem", "rounds", "few_rounds")
+
+
+def tile(shim, L, df, f32, rows, groups=10 ** 6, planes=1):
+    out = (ctypes.c_int * 7)()
+    assert shim.shim_any_tile(L, df, f32, rows, ctypes.c_longlong(groups), planes, SMS, out) == 0, L
+    return dict(zip(TILE, out))
+
+
+def plane(shim, nx, ny, df, f32):
+    out = (ctypes.c_int * 3)()
+    shim.shim_plane_tile(nx, ny, df, f32, out)
+    return tuple(out)
+
+
 @pytest.fixture(scope="module")
 def shim(tmp_path_factory):
     out = str(tmp_path_factory.mktemp("shim") / "any_sched.so")
@@ -60,3 +76,34 @@ def test_kernel_covers_the_radices(shim, max_radix, rows):
         L = n if rows else 2 * n
         for pad in (0, 1):
             assert shim.shim_any_radix_rule(L, max_radix, 8 if rows else max_radix, pad) == 0, L
+
+
+@pytest.mark.parametrize("df,f32", [(0, 1), (0, 0), (1, 0)])
+@pytest.mark.parametrize("rows", [0, 1])
+def test_tiles_fit_and_few_threads_save_rounds(shim, df, f32, rows):
+    """Every tile fits a block's shared memory and the kernels' threads; the threads of a launch
+    of few tiles are those of a full chip or take fewer rounds."""
+    for n in counts():
+        t = tile(shim, n if rows else 2 * n, df, f32, rows)
+        assert t["smem"] <= 232448 - 1024 and t["lg"] in (1, 2, 3), (n, t)
+        assert 64 <= t["threads"] <= 256 and t["threads"] % 32 == 0, (n, t)
+        assert 64 <= t["few"] <= 256 and t["few"] % 32 == 0 and t["ctas"] >= 1, (n, t)
+        assert t["few"] == t["threads"] or t["few_rounds"] < t["rounds"], (n, t)
+
+
+def test_few_tiles(shim):
+    """Double-float N = 30: the z pass's 80 butterflies of radix 6 take one round instead of two.  A
+    launch is of few tiles up to the CTAs that fit the SMs and three warps to a scheduler."""
+    t = tile(shim, 60, 1, 0, 0)
+    assert t["threads"] == 64 and t["few"] == 96 and (t["rounds"], t["few_rounds"]) == (22, 16)
+    assert shim.shim_any_is_few(64, 5, SMS, 5 * SMS) and not shim.shim_any_is_few(64, 5, SMS, 5 * SMS + 1)
+    assert shim.shim_any_is_few(128, 8, SMS, 3 * SMS) and not shim.shim_any_is_few(128, 8, SMS, 3 * SMS + 1)
+
+
+@pytest.mark.parametrize("nx,ny,df,f32,on", [(6, 4, 0, 1, 1), (60, 60, 0, 1, 1), (72, 54, 0, 1, 1), (72, 64, 0, 1, 0),
+                                             (6, 4, 1, 0, 1), (18, 18, 1, 0, 1), (20, 20, 1, 0, 0), (30, 24, 1, 0, 0)])
+def test_plane_kernels_up_to(shim, nx, ny, df, f32, on):
+    """Both sides of the largest plane that takes its x and y passes in one kernel."""
+    got = plane(shim, nx, ny, df, f32)
+    assert got[0] == on and 128 <= got[1] <= 384
+    assert not on or got[2] <= 232448 - 1024

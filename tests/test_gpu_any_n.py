@@ -252,3 +252,35 @@ def test_box_axes_with_compiled_lengths(torch_cuda, n, dtype):
             torch.cuda.synchronize()
             assert eta.value == pytest.approx(ref, rel=1e-5)
             assert np.array_equal(out.cpu().numpy().astype(np.float64).reshape(u.shape), u)
+
+
+@pytest.mark.parametrize("n", [(6, 100, 10), (20, 20, 20), (30, 30, 30), (50, 20, 30), (90, 6, 20), (6, 4, 90)])
+def test_few_tiles(torch_cuda, n):
+    """Small launches of the wider arithmetics, whose x passes take their last stage and the
+    Hermitian split apart: the smallest and longer rows, with tiles that are not full, against the
+    oracle in both arithmetics."""
+    from paper_1612_01799_gb300 import Plan
+    half = (8.0,) * 3
+    op = obox.make_box_plan(n, tuple(-q for q in half), half, 1e-12)
+    rho = np.random.default_rng(sum(n)).uniform(-1, 1, (n[2], n[1], n[0]))
+    uo = obox.solve_box(rho, op)
+    with Plan(n, half, 1e-12, "f64") as p:
+        for ar in variants("f64"):
+            p.arith = ar
+            assert rel_l2(run(torch_cuda, p, rho), uo) <= TOL["f64"], ar
+
+
+@pytest.mark.parametrize("N,count", [(30, 12), (20, 16)])
+def test_batch_of_another_route_gives_the_same_bits(torch_cuda, N, count):
+    """A batch fills the SMs where one density does not, and takes other launches (threads, x stages
+    combined or apart, in FP64 the plane kernels): the bits of the single solves."""
+    from paper_1612_01799_gb300 import Plan, solve_batched
+    torch = torch_cuda
+    rng = np.random.default_rng(N)
+    with Plan(N, 8.0, 1e-12, "f64", max_batch=count) as p:
+        for ar in variants("f64"):
+            p.arith = ar
+            rhos = [torch.from_numpy(rng.uniform(-1, 1, (N, N, N))).cuda() for _ in range(count)]
+            outs = solve_batched([p] * count, rhos, [torch.empty_like(r) for r in rhos])
+            for r, o in zip(rhos, outs):
+                assert torch.equal(p.solve(r), o), ar
