@@ -127,14 +127,20 @@ inline bool any_is_few(const AnyTile &t, int sms, int ntiles) {
 // row, which a quarter-warp reads whole; four groups take odd strides instead).  Eight groups
 // while three CTAs fit an SM, else four (FP32, solves: N = 240 590 us with eight, 605 us with
 // four; N = 162 243 and 275 us; N = 400, where only two CTAs of eight fit, 2.86 and 2.83 ms).
+// groups x planes: the 16-byte groups of one solve's pass (a tile stays within a plane).  Tiles of
+// eight that leave half of the SMs idle are made of four where a stage of eight takes several rounds
+// (box 400 x 12 x 12, double-float 54.4 -> 42.5 us; 400 x 20 x 20, FP32 31.8 -> 27.2 us).
 // Threads: the multiple of 32 with the most threads of
 // an SM at work, counting the share of thread slots that the rounds over the butterflies of
 // each stage fill and the CTAs that shared memory and registers admit; few: see any_is_few.
-inline AnyTile any_tile(int L, int max_radix, bool f32, bool rows) {
+inline AnyTile any_tile(int L, int max_radix, bool f32, bool rows, long long groups, int planes, int sms) {
     AnyTile t{};
     const int max_last = rows ? kAnyRowsLast : max_radix, max_warps = any_max_warps(f32);
     const AnySched wide = any_sched_of(L, max_radix, max_last, rows, &t.mr);
-    t.lg = wide.slots * (rows ? 9 : 8) * 16 <= 70 * 1024 ? 3 : 2;
+    bool eight = wide.slots * (rows ? 9 : 8) * 16 <= 70 * 1024;
+    if (2 * ((groups + 7) / 8) * planes <= sms)
+        for (int st = 0; st < wide.nst; ++st) eight = eight && L / wide.r[st] * 8 <= kAnyThreads;
+    t.lg = eight ? 3 : 2;
     t.s = t.lg == 3 ? wide : any_sched_of(L, max_radix, max_last, true, &t.mr);
     t.pitch = (1 << t.lg) + (rows ? 1 : 0);
     t.smem = t.s.slots * t.pitch * 16;

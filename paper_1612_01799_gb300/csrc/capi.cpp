@@ -69,10 +69,12 @@ bool n_any(int N) {
 void any_plan_tiles(DevicePlan &p) {
     const bool f32 = p.dtype == POISSON_F32;
     p.plane_small = !p.any && plane_n_size(p.N, !f32);
-    const int W = f32 ? 2 : 1, nx = p.n3[0], ny = p.n3[1];
+    const int W = f32 ? 2 : 1, nx = p.n3[0], ny = p.n3[1], nz = p.n3[2], cols = (nx + W) / W;
     for (int df = 0; df < 2; ++df) {
         const int R = any_max_radix(df != 0);
-        for (int q = 0; q < 3; ++q) p.any_tile[df][q] = any_tile(q == 0 ? nx : 2 * p.n3[q], R, f32, q == 0);
+        p.any_tile[df][0] = any_tile(nx, R, f32, true, (long long)ny * nz / W, 1, p.sms);
+        p.any_tile[df][1] = any_tile(2 * ny, R, f32, false, cols, nz, p.sms);
+        p.any_tile[df][2] = any_tile(2 * nz, R, f32, false, cols, 2 * ny, p.sms);
         p.plane[df] = plane_tile(nx, ny, R, W);
         if (!p.any || (n_supported(nx) && n_supported(ny))) p.plane[df].on = false;
     }

@@ -79,8 +79,7 @@ extern "C" int shim_any_radix_rule(int L, int max_radix, int max_last, int pad) 
 // rounds over the butterflies (and, for rows, over the Hermitian split) with `threads` and with `few`.
 // 0, or 1 if the schedule does not multiply up to L.
 extern "C" int shim_any_tile(int L, int df, int f32, int rows, long long groups, int planes, int sms, int *out) {
-    (void)groups, (void)planes, (void)sms;
-    const gsp::AnyTile t = gsp::any_tile(L, gsp::any_max_radix(df != 0), f32 != 0, rows != 0);
+    const gsp::AnyTile t = gsp::any_tile(L, gsp::any_max_radix(df != 0), f32 != 0, rows != 0, groups, planes, sms);
     int prod = 1;
     for (int st = 0; st < t.s.nst; ++st) prod *= t.s.r[st];
     if (t.s.nst < 2 || prod != L || t.smem != t.s.slots * t.pitch * 16) return 1;

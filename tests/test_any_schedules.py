@@ -107,3 +107,11 @@ def test_plane_kernels_up_to(shim, nx, ny, df, f32, on):
     got = plane(shim, nx, ny, df, f32)
     assert got[0] == on and 128 <= got[1] <= 384
     assert not on or got[2] <= 232448 - 1024
+
+
+@pytest.mark.parametrize("L,rows,groups,planes,lg", [(400, 1, 144, 1, 2), (400, 1, 608, 1, 2), (400, 1, 616, 1, 3),
+                                                     (40, 1, 60, 1, 3), (400, 0, 13, 12, 2), (400, 0, 16, 39, 3)])
+def test_tiles_of_four_on_idle_sms(shim, L, rows, groups, planes, lg):
+    """Double-float: eight groups to a tile, four where the eights leave half of 152 SMs idle and
+    a stage of them takes several rounds (not at L = 40)."""
+    assert tile(shim, L, 1, 0, rows, groups, planes)["lg"] == lg

@@ -254,11 +254,12 @@ def test_box_axes_with_compiled_lengths(torch_cuda, n, dtype):
             assert np.array_equal(out.cpu().numpy().astype(np.float64).reshape(u.shape), u)
 
 
-@pytest.mark.parametrize("n", [(6, 100, 10), (20, 20, 20), (30, 30, 30), (50, 20, 30), (90, 6, 20), (6, 4, 90)])
+@pytest.mark.parametrize("n", [(6, 100, 10), (20, 20, 20), (30, 30, 30), (50, 20, 30), (90, 6, 20), (6, 4, 90),
+                               (400, 6, 10), (6, 400, 10)])
 def test_few_tiles(torch_cuda, n):
     """Small launches of the wider arithmetics, whose x passes take their last stage and the
-    Hermitian split apart: the smallest and longer rows, with tiles that are not full, against the
-    oracle in both arithmetics."""
+    Hermitian split apart: the smallest and longer rows, with tiles that are not full, tiles of four
+    groups, against the oracle in both arithmetics."""
     from paper_1612_01799_gb300 import Plan
     half = (8.0,) * 3
     op = obox.make_box_plan(n, tuple(-q for q in half), half, 1e-12)
