@@ -129,7 +129,10 @@ inline bool any_is_few(const AnyTile &t, int sms, int ntiles) {
 // four; N = 162 243 and 275 us; N = 400, where only two CTAs of eight fit, 2.86 and 2.83 ms).
 // groups x planes: the 16-byte groups of one solve's pass (a tile stays within a plane).  Tiles of
 // eight that leave half of the SMs idle are made of four where a stage of eight takes several rounds
-// (box 400 x 12 x 12, double-float 54.4 -> 42.5 us; 400 x 20 x 20, FP32 31.8 -> 27.2 us).
+// (box 400 x 12 x 12, double-float 54.4 -> 42.5 us; 400 x 20 x 20, FP32 31.8 -> 27.2 us).  In the
+// wider arithmetics two groups where four leave room for one CTA of eight warps (the columns of
+// N = 900 to 1000: double-float box 24 x 24 x 1000 213 -> 174 us, cube N = 1000 278 -> 253 ms, in
+// FP64 828 -> 692 us for the box; FP32, whose columns are half as wide, loses at N = 900, 51 -> 61 ms).
 // Threads: the multiple of 32 with the most threads of
 // an SM at work, counting the share of thread slots that the rounds over the butterflies of
 // each stage fill and the CTAs that shared memory and registers admit; few: see any_is_few.
@@ -142,6 +145,7 @@ inline AnyTile any_tile(int L, int max_radix, bool f32, bool rows, long long gro
         for (int st = 0; st < wide.nst; ++st) eight = eight && L / wide.r[st] * 8 <= kAnyThreads;
     t.lg = eight ? 3 : 2;
     t.s = t.lg == 3 ? wide : any_sched_of(L, max_radix, max_last, true, &t.mr);
+    if (!f32 && !rows && t.s.slots * (16 << t.lg) > 112 * 1024) t.lg = 1;
     t.pitch = (1 << t.lg) + (rows ? 1 : 0);
     t.smem = t.s.slots * t.pitch * 16;
     auto rounds_of = [&](int n) {

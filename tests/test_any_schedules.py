@@ -115,3 +115,10 @@ def test_tiles_of_four_on_idle_sms(shim, L, rows, groups, planes, lg):
     """Double-float: eight groups to a tile, four where the eights leave half of 152 SMs idle and
     a stage of them takes several rounds (not at L = 40)."""
     assert tile(shim, L, 1, 0, rows, groups, planes)["lg"] == lg
+
+
+@pytest.mark.parametrize("n,f32,lg", [(810, 0, 2), (900, 0, 1), (1000, 0, 1), (1000, 1, 2)])
+def test_tiles_of_two_for_long_wide_columns(shim, n, f32, lg):
+    """Columns of 2 n points in the wider arithmetics: two groups where four fill an SM."""
+    assert tile(shim, 2 * n, 0, f32, 0)["lg"] == lg
+    assert f32 or tile(shim, 2 * n, 1, f32, 0)["lg"] == lg

@@ -285,3 +285,18 @@ def test_batch_of_another_route_gives_the_same_bits(torch_cuda, N, count):
             outs = solve_batched([p] * count, rhos, [torch.empty_like(r) for r in rhos])
             for r, o in zip(rhos, outs):
                 assert torch.equal(p.solve(r), o), ar
+
+
+@pytest.mark.parametrize("n", [(6, 10, 900), (10, 960, 4)])
+def test_long_columns(torch_cuda, n):
+    """Columns of two groups to a tile (an odd number of columns: the last tile half full) against the
+    oracle in both wide arithmetics."""
+    from paper_1612_01799_gb300 import Plan
+    half = (40.0,) * 3
+    op = obox.make_box_plan(n, tuple(-q for q in half), half, 1e-12)
+    rho = np.random.default_rng(sum(n)).uniform(-1, 1, (n[2], n[1], n[0]))
+    uo = obox.solve_box(rho, op)
+    with Plan(n, half, 1e-12, "f64") as p:
+        for ar in variants("f64"):
+            p.arith = ar
+            assert rel_l2(run(torch_cuda, p, rho), uo) <= TOL["f64"], ar
