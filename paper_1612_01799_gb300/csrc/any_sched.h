@@ -184,16 +184,20 @@ inline AnyTile any_tile(int L, int max_radix, bool f32, bool rows, long long gro
 struct PlaneTile {
     AnySched sx, sy;
     int gx, px, gy, py, threads, smem, mr;
-    bool on;
+    bool on, many;
 };
 constexpr int kPlaneThreads = 384;
 // Largest plane: in FP32 two CTAs fit an SM (solves, separate passes against the plane kernels:
 // 20^3 21.4 and 18.9 us, 60^3 27.2 and 25.5, 64 x 64 x 256 66 and 57, but 72^3 28.6 and 30.2); the
 // wider arithmetics are bound by the longer chain of one CTA soon (double-float 10^3 24.3 and
-// 20.8 us, 18^3 27.4 and 27.4, 20^3 25.9 and 28.5, 30^3 32.0 and 36.6).  Cubes whose passes are
-// compiled for their length have kernels of their own (plane_n_size).
+// 20.8 us, 18^3 27.4 and 27.4, 20^3 25.9 and 28.5, 30^3 32.0 and 36.6).  In FP64 planes
+// up to kPlaneMany are worth a CTA each where they fill the SMs, no wave of them below nine tenths
+// (many; 24 x 24 x 600 413 and 395 us, but 20 x 20 x 240 112 and 122).  Cubes whose passes are compiled for
+// their length have kernels of their own (plane_n_size).
 constexpr int plane_smem(bool f32) { return f32 ? 106 * 1024 : 18 * 1024; }
-inline PlaneTile plane_tile(int nx, int ny, int max_radix, int w) {
+constexpr int kPlaneMany = 48 * 1024;
+// fp64: FP64 arithmetic.
+inline PlaneTile plane_tile(int nx, int ny, int max_radix, int w, bool fp64) {
     PlaneTile t{};
     t.sx = any_sched_of(nx, max_radix, kAnyRowsLast, true, &t.mr);
     t.sy = any_sched_of(2 * ny, max_radix, max_radix, false, &t.mr);
@@ -216,7 +220,14 @@ inline PlaneTile plane_tile(int nx, int ny, int max_radix, int w) {
         }
     }
     t.on = t.sx.nst && t.sy.nst && t.smem <= plane_smem(w == 2);
+    t.many = fp64 && t.sx.nst && t.sy.nst && t.smem <= kPlaneMany;
     return t;
+}
+// Whether a launch of `planes` planes runs the plane kernels.
+inline bool plane_runs(const PlaneTile &t, int sms, int planes) {
+    if (t.on || !t.many) return t.on;
+    const long long resident = (long long)sms * std::max(1, any_max_warps(false) * 32 / t.threads);
+    return 10 * planes >= 9 * ((planes + resident - 1) / resident * resident);
 }
 
 // e / d by its reciprocal mul.

@@ -68,15 +68,15 @@ bool n_any(int N) {
 
 void any_plan_tiles(DevicePlan &p) {
     const bool f32 = p.dtype == POISSON_F32;
-    p.plane_small = !p.any && plane_n_size(p.N, !f32);
+    p.plane_small = !p.any;
     const int W = f32 ? 2 : 1, nx = p.n3[0], ny = p.n3[1], nz = p.n3[2], cols = (nx + W) / W;
     for (int df = 0; df < 2; ++df) {
         const int R = any_max_radix(df != 0);
         p.any_tile[df][0] = any_tile(nx, R, f32, true, (long long)ny * nz / W, 1, p.sms);
         p.any_tile[df][1] = any_tile(2 * ny, R, f32, false, cols, nz, p.sms);
         p.any_tile[df][2] = any_tile(2 * nz, R, f32, false, cols, 2 * ny, p.sms);
-        p.plane[df] = plane_tile(nx, ny, R, W);
-        if (!p.any || (n_supported(nx) && n_supported(ny))) p.plane[df].on = false;
+        p.plane[df] = plane_tile(nx, ny, R, W, !f32 && df == 0);
+        if (!p.any || (n_supported(nx) && n_supported(ny))) p.plane[df].on = p.plane[df].many = false;
     }
     for (int q = 0; q < 3; ++q) p.axn[q] = p.any && n_supported(p.n3[q]) ? p.n3[q] : 0;
 }
@@ -843,7 +843,7 @@ extern "C" int poisson_solve_host(poisson_plan p, const void *rho_h, void *u_h, 
     gsp::PtrArray in, out;
     one(in, p->stage_in);
     one(out, p->stage_out);
-    const bool fused = (p->dp.xyform == 1 && p->dp.sync != nullptr) || gsp::plane_on(p->dp) || gsp::plane_n_plan(p->dp);
+    const bool fused = (p->dp.xyform == 1 && p->dp.sync != nullptr) || gsp::plane_on(p->dp, nz) || gsp::plane_n_plan(p->dp);
     if (fused || n < kHostPipelineBytes || nz % 8 != 0) {
         if ((e = cudaMemcpyAsync(p->stage_in, rho_h, n, cudaMemcpyHostToDevice, s)) != cudaSuccess)
             return map_cuda(e);

@@ -432,7 +432,7 @@ template <typename Real, int N> struct PlaneN {
     static constexpr int X_BYTES = (N + 1) * SX * (int)sizeof(typename Types<Real>::CS);
     static constexpr int OFF_Y = (X_BYTES + 15) / 16 * 16;
     static constexpr int SMEM = OFF_Y + L * SY * 16;
-    static constexpr bool ok = plane_n_size(N, !std::is_same<Real, float>::value);
+    static constexpr bool ok = plane_n_size(N, std::is_same<Real, float>::value, std::is_same<Real, DF>::value);
     static_assert(!ok || (NT <= 1024 && SMEM <= 227 * 1024), "threads and shared memory of one CTA");
 };
 // Element (y, k) of the plane's column layout.
@@ -936,10 +936,10 @@ cudaError_t xy_pass(const DevicePlan &p, const PtrArray &rho, const PtrArray &u,
 }
 
 // Whether the x and y passes of B densities run as one kernel per direction (k_plane_n_*).  In
-// the wider arithmetics many planes are better off in the separate passes, whose CTAs are more
-// and smaller (double-float, 16 densities of N = 32: 61 us against 63 us); the bits are the same.
+// the wider arithmetics more than two planes to an SM are better off in the separate passes, whose CTAs
+// are more and smaller (double-float, 16 densities of N = 32: 61 us against 63 us); the bits are the same.
 template <typename Real, int N> bool plane_n_on(const DevicePlan &p, int B) {
-    return PlaneN<Real, N>::ok && plane_n_plan(p) && (std::is_same<Real, float>::value || B * N <= 304);
+    return PlaneN<Real, N>::ok && plane_n_plan(p) && (std::is_same<Real, float>::value || B * N <= 2 * p.sms);
 }
 template <typename Real, int N>
 cudaError_t plane_n(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int B, cudaStream_t s, bool fwd) {
@@ -1256,7 +1256,7 @@ cudaError_t plane_xy(const DevicePlan &p, const PtrArray &rho, const PtrArray &u
 template <typename Real>
 cudaError_t solve_any(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int B, cudaStream_t s,
                       cudaEvent_t *ev, double *tail, int skip) {
-    const bool plane = plane_on(p);
+    const bool plane = plane_on(p, B * p.n3[2]);
     if (plane && skip) return cudaErrorInvalidValue;
     if (ev) GSP_CHECK(cudaEventRecord(ev[0], s));
     if (plane) GSP_CHECK(plane_xy<Real>(p, rho, u, B, s, true));

@@ -5,6 +5,7 @@
 
 #include <cstddef>
 
+#include "../../include/poisson.h"
 #include "any_sched.h"
 
 namespace gsp {
@@ -54,8 +55,8 @@ struct DevicePlan {
     // Tiles of the runtime-length passes along x, y and z, per arithmetic (any_plan_tiles).
     AnyTile any_tile[2][3] = {};
     int sms = 1;  // SMs of the plan's device
-    // Compiled-length plans with small planes: the x and y passes in one kernel per direction
-    // (the allocation-free solve leaves it false).
+    // Compiled-length plans: small planes may take the x and y passes in one kernel per direction
+    // (plane_n_plan; the allocation-free solve leaves it false).
     bool plane_small = false;
     // The x and y passes as one kernel per direction (passes_plane.cuh), per arithmetic, for
     // runtime-length plans whose planes are small (plane_on).
@@ -111,14 +112,18 @@ bool n_supported(int N);
 // Fill p.any_tile for p's lengths (any plan: the slab z pass runs on the compiled-length
 // plans too) and p.plane.
 void any_plan_tiles(DevicePlan &p);
-// Whether p's solves run the plane kernels in its present arithmetic.
-inline bool plane_on(const DevicePlan &p) { return p.plane[p.arith].on; }
-// Compiled-length plans: the sizes of the plane kernels (at N = 64 in FP32 they and the separate
-// passes take 20 us, twelve densities 116 and 91 us; double-float N = 48 41.6 and 35.3 us), and
-// whether p's solves run them: with the block forms of both passes.
-__host__ __device__ constexpr bool plane_n_size(int N, bool wide) { return N == 16 || N == 32 || (N == 48 && !wide); }
+// Whether p's solves of `planes` z-planes run the plane kernels in its present arithmetic.
+inline bool plane_on(const DevicePlan &p, int planes) { return plane_runs(p.plane[p.arith], p.sms, planes); }
+// Compiled-length plans: the sizes of the plane kernels, per arithmetic (at N = 64 in FP32 they and
+// the separate passes take 20 us, twelve densities 116 and 91 us; double-float N = 48 41.6 and
+// 35.3 us; FP64 N = 16 30.3 and 43.4 us, but N = 32 62 and 45 us: there the FP64 pipe is the bound, of
+// 32 SMs instead of all), and whether p's solves run them: with the block forms of both passes.
+__host__ __device__ constexpr bool plane_n_size(int N, bool f32, bool df) {
+    return N == 16 || (N == 32 && (f32 || df)) || (N == 48 && f32);
+}
 inline bool plane_n_plan(const DevicePlan &p) {
-    return p.plane_small && p.xform == 0 && p.yform == 0 && p.xyform == 0;
+    return p.plane_small && plane_n_size(p.N, p.dtype == POISSON_F32, p.arith == 1) && p.xform == 0 && p.yform == 0 &&
+           p.xyform == 0;
 }
 
 // Largest shared memory of one block (227 KB).

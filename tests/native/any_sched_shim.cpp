@@ -99,10 +99,11 @@ extern "C" int shim_any_is_few(int threads, int ctas, int sms, int ntiles) {
     t.few_ctas = ctas;
     return gsp::any_is_few(t, sms, ntiles);
 }
-// The plane kernels' tile: on, threads, bytes of shared memory with the twiddles.
-extern "C" int shim_plane_tile(int nx, int ny, int df, int f32, int *out) {
-    const gsp::PlaneTile t = gsp::plane_tile(nx, ny, gsp::any_max_radix(df != 0), f32 ? 2 : 1);
-    const int v[] = {t.on, t.threads, t.smem + (f32 ? (nx + 2 * ny) * 8 + 16 : 0)};
+// The plane kernels' tile: whether a launch of `planes` planes on sms SMs runs them, threads, bytes of
+// shared memory with the twiddles.  df: double-float arithmetic, else FP32 or FP64 by f32.
+extern "C" int shim_plane_tile(int nx, int ny, int df, int f32, int sms, int planes, int *out) {
+    const gsp::PlaneTile t = gsp::plane_tile(nx, ny, gsp::any_max_radix(df != 0), f32 ? 2 : 1, !f32 && !df);
+    const int v[] = {gsp::plane_runs(t, sms, planes), t.threads, t.smem + (f32 ? (nx + 2 * ny) * 8 + 16 : 0)};
     std::copy(v, v + 3, out);
     return 0;
 }

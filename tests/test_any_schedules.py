@@ -33,9 +33,9 @@ def tile(shim, L, df, f32, rows, groups=10 ** 6, planes=1):
     return dict(zip(TILE, out))
 
 
-def plane(shim, nx, ny, df, f32):
+def plane(shim, nx, ny, df, f32, planes=1):
     out = (ctypes.c_int * 3)()
-    shim.shim_plane_tile(nx, ny, df, f32, out)
+    shim.shim_plane_tile(nx, ny, df, f32, SMS, planes, out)
     return tuple(out)
 
 
@@ -122,3 +122,10 @@ def test_tiles_of_two_for_long_wide_columns(shim, n, f32, lg):
     """Columns of 2 n points in the wider arithmetics: two groups where four fill an SM."""
     assert tile(shim, 2 * n, 0, f32, 0)["lg"] == lg
     assert f32 or tile(shim, 2 * n, 1, f32, 0)["lg"] == lg
+
+
+@pytest.mark.parametrize("n,df,planes,on", [(18, 0, 1, 1), (30, 0, 152, 1), (30, 0, 160, 0), (30, 0, 304, 1),
+                                                (36, 0, 304, 0), (30, 1, 304, 0)])
+def test_plane_kernels_of_many_planes(shim, n, df, planes, on):
+    """FP64 arithmetic: planes up to 48 KB where their CTAs fill the SMs; not in double-float."""
+    assert plane(shim, n, n, df, 0, planes)[0] == on
