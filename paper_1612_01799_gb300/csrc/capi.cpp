@@ -843,8 +843,7 @@ extern "C" int poisson_solve_host(poisson_plan p, const void *rho_h, void *u_h, 
     gsp::PtrArray in, out;
     one(in, p->stage_in);
     one(out, p->stage_out);
-    const bool fused = (p->dp.xyform == 1 && p->dp.sync != nullptr) || gsp::plane_on(p->dp, nz) || gsp::plane_n_plan(p->dp);
-    if (fused || n < kHostPipelineBytes || nz % 8 != 0) {
+    if (gsp::xy_in_one(p->dp, 1) || n < kHostPipelineBytes || nz % 8 != 0) {
         if ((e = cudaMemcpyAsync(p->stage_in, rho_h, n, cudaMemcpyHostToDevice, s)) != cudaSuccess)
             return map_cuda(e);
         if ((e = gsp::launch_solve(p->dp, in, out, 1, s, nullptr)) != cudaSuccess) return map_cuda(e);
@@ -1024,6 +1023,7 @@ extern "C" int poisson_solve_timed(poisson_plan p, const void *rho_d, void *u_d,
     for (int i = 0; i < 5; ++i)
         if ((e = cudaEventElapsedTime(&ms[i], p->ev[i], p->ev[i + 1])) != cudaSuccess)
             return map_cuda(e);
+    if (gsp::xy_in_one(p->dp, 1)) ms[1] = ms[4] = 0.f;  // no pass between these events
     return POISSON_OK;
 }
 

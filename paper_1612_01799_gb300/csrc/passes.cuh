@@ -935,11 +935,10 @@ cudaError_t xy_pass(const DevicePlan &p, const PtrArray &rho, const PtrArray &u,
     return cudaErrorInvalidValue;
 }
 
-// Whether the x and y passes of B densities run as one kernel per direction (k_plane_n_*).  In
-// the wider arithmetics more than two planes to an SM are better off in the separate passes, whose CTAs
-// are more and smaller (double-float, 16 densities of N = 32: 61 us against 63 us); the bits are the same.
+// Whether the x and y passes of B densities run as one kernel per direction (k_plane_n_*, the bits of
+// the separate passes).
 template <typename Real, int N> bool plane_n_on(const DevicePlan &p, int B) {
-    return PlaneN<Real, N>::ok && plane_n_plan(p) && (std::is_same<Real, float>::value || B * N <= 2 * p.sms);
+    return PlaneN<Real, N>::ok && plane_n_plan(p, B * N);
 }
 template <typename Real, int N>
 cudaError_t plane_n(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int B, cudaStream_t s, bool fwd) {

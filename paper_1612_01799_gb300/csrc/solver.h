@@ -117,13 +117,20 @@ inline bool plane_on(const DevicePlan &p, int planes) { return plane_runs(p.plan
 // Compiled-length plans: the sizes of the plane kernels, per arithmetic (at N = 64 in FP32 they and
 // the separate passes take 20 us, twelve densities 116 and 91 us; double-float N = 48 41.6 and
 // 35.3 us; FP64 N = 16 30.3 and 43.4 us, but N = 32 62 and 45 us: there the FP64 pipe is the bound, of
-// 32 SMs instead of all), and whether p's solves run them: with the block forms of both passes.
+// 32 SMs instead of all), and whether p's solves of `planes` planes run them: with the block forms of both passes.
 __host__ __device__ constexpr bool plane_n_size(int N, bool f32, bool df) {
     return N == 16 || (N == 32 && (f32 || df)) || (N == 48 && f32);
 }
-inline bool plane_n_plan(const DevicePlan &p) {
-    return p.plane_small && plane_n_size(p.N, p.dtype == POISSON_F32, p.arith == 1) && p.xform == 0 && p.yform == 0 &&
-           p.xyform == 0;
+// In the wider arithmetics more than two planes to an SM are better off in the separate passes, whose
+// CTAs are more and smaller (double-float, 16 densities of N = 32: 61 us against 63 us).
+inline bool plane_n_plan(const DevicePlan &p, int planes) {
+    const bool f32 = p.dtype == POISSON_F32;
+    return p.plane_small && plane_n_size(p.N, f32, p.arith == 1) && p.xform == 0 && p.yform == 0 && p.xyform == 0 &&
+           (f32 || planes <= 2 * p.sms);
+}
+// Whether solves of B densities make the x and y passes in one kernel per direction.
+inline bool xy_in_one(const DevicePlan &p, int B) {
+    return (p.xyform == 1 && p.sync != nullptr) || plane_on(p, B * p.n3[2]) || plane_n_plan(p, B * p.N);
 }
 
 // Largest shared memory of one block (227 KB).

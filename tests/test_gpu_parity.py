@@ -288,10 +288,11 @@ def test_degenerate_inputs_and_invariants(torch_cuda, N, dtype, forms):
                                            (32, "f64", 10)])
 def test_plane_kernels_equal_separate_passes(torch_cuda, N, dtype, count):
     """Small compiled sizes take the x and y passes of a plane in one kernel per direction: the
-    bits of the separate passes, which run the slabs of a slab decomposition (its inverse here
-    from the solve's own z output) and, in the wider arithmetics, batches of more than 304
-    planes."""
+    bits of the separate passes, which run the slabs of a slab decomposition (its forward here
+    against the y spectrum that a solve left, its inverse from the solve's own z output) and, in the
+    wider arithmetics, batches of more than two planes to an SM."""
     from paper_1612_01799_gb300 import Plan, solve_batched
+    from paper_1612_01799_gb300.slab import PlanStages
     torch = torch_cuda
     rng = np.random.default_rng(N)
     with Plan(N, 8.0, 1e-6 if dtype == "f32" else 1e-12, dtype, max_batch=count) as p:
@@ -302,8 +303,16 @@ def test_plane_kernels_equal_separate_passes(torch_cuda, N, dtype, count):
             outs = solve_batched([p] * count, rhos, [torch.empty_like(r) for r in rhos])
             for r, o in zip(rhos, outs):
                 assert torch.equal(p.solve(r), o), ar
+            one = ar != "f64" or N == 16          # FP64 arithmetic: N = 16 only
             ms = p.solve_timed(rhos[0], outs[0])
-            assert ms[0] > 0 and ms[3] > 0 and ms[1] < 0.02 and ms[4] < 0.02
+            assert ms[0] > 0 and ms[3] > 0 and (ms[1] == 0, ms[4] == 0) == (one, one), ms
+            # the forward kernel: the y spectrum it left, and the one of the separate passes
+            st = PlanStages(torch, p)
+            cols = (4 if ar == "df" else 2) * (N + 1)
+            got = st.spectrum(0)[:, :, :cols].clone()
+            st.spectrum(0).zero_()
+            st.forward(rhos[0], 0, N)
+            assert torch.equal(st.spectrum(0)[:, :, :cols], got), ar
             u = torch.empty_like(rhos[0])
             p.solve(rhos[0], out=outs[0])
             assert p._lib.poisson_slab_inverse(p.handle, u.data_ptr(), 0, N, None) == 0

@@ -321,7 +321,9 @@ def test_xy_fused_timed_passes(torch_cuda):
         u = torch.empty_like(rho)
         ms = p.solve_timed(rho, u)
         assert ms[0] > 0 and ms[2] > 0 and ms[3] > 0
-        assert ms[1] < 0.02 and ms[4] < 0.02
+        assert ms[1] == 0 and ms[4] == 0
+        p.xy_form = 0
+        assert all(v > 0 for v in p.solve_timed(rho, u))
         assert torch.equal(u, p.solve(rho))
         p.last_status()
 
