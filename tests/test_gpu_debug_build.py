@@ -3,8 +3,8 @@ access of the pass kernels' access helpers and the runtime-length forms' compute
 bounds-checked, a failed check skipping the access and setting a device-wide flag word).
 A child process with POISSON_DEBUG=1 runs solves in every kernel family (compiled warp
 and block forms at several sizes, the N = 512 warp forms, the double-float FP64 plan,
-runtime-length sizes and a box with a different count per axis, a batched and a checked
-solve); no check may fail (flags 0) and each potential must equal the release library's
+runtime-length sizes and boxes with a different count per axis in each of their kernels,
+batched and checked solves); no check may fail (flags 0) and each potential must equal the release library's
 within rounding.  The build's self-test shows the checks firing: its two out-of-range
 predicates (evaluated without an access) set both flag bits."""
 import json
@@ -17,7 +17,8 @@ import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
-# (name, shape, dtype, (z, y, x) forms or None for the plan's own choice)
+# (name, shape, dtype, (z, y, x) forms, the arithmetic of an FP64 plan, or None for the plan's own
+# choice)
 CASES = [
     ("warp64", 64, "f32", (2, 1, 1)),
     ("warp192", 192, "f32", (2, 1, 1)),
@@ -27,6 +28,29 @@ CASES = [
     ("df48", 48, "f64", None),
     ("any24", 24, "f32", None),
     ("anybox", (20, 24, 30), "f64", None),
+    # the separate runtime-length passes: both kernel sizes (radices up to 10 and 12), rows and
+    # columns with the long twiddle copy, tiles of four and of two groups
+    ("any90", (90, 72, 20), "f32", None),
+    ("any72", (72, 72, 10), "f32", None),
+    ("any400", (400, 10, 36), "f32", None),
+    ("long", (10, 400, 24), "f32", None),
+    ("any40df", (40, 50, 36), "f64", "df"),
+    ("any40", (40, 50, 36), "f64", "f64"),
+    ("batched_df", 30, "f64", "df"),
+    ("batched_f64", 30, "f64", "f64"),
+    ("long_df", (20, 6, 960), "f64", "df"),
+    # plane kernels: runtime lengths and compiled ones, in each arithmetic
+    ("plane60", (60, 60, 12), "f32", None),
+    ("plane50", (50, 54, 10), "f32", None),
+    ("plane18df", (18, 12, 10), "f64", "df"),
+    ("plane18", (18, 12, 10), "f64", "f64"),
+    ("plane16df", 16, "f64", "df"),
+    ("plane16", 16, "f64", "f64"),
+    ("plane32df", 32, "f64", "df"),
+    # boxes whose axes differ in kind
+    ("mixed", (32, 20, 64), "f32", None),
+    ("mixed_df", (20, 64, 30), "f64", "df"),
+    ("mixed_f64", (64, 48, 24), "f64", "f64"),
 ]
 
 CHILD = r'''
@@ -55,12 +79,19 @@ for name, shape, dtype, forms in cases:
     n = shape if isinstance(shape, int) else tuple(shape)
     N = n if isinstance(n, int) else n[0]
     rho = np.load(os.path.join(out_dir, name + "_rho.npy"))
-    with Plan(n, 6.0, 1e-6 if dtype == "f32" else 1e-12, dtype) as p:
-        if forms:
+    batch = 16 if name.startswith("batched") else 1
+    with Plan(n, 6.0, 1e-6 if dtype == "f32" else 1e-12, dtype, max_batch=batch) as p:
+        if isinstance(forms, str):
+            p.arith = forms
+        elif forms:
             p.z_form, p.y_form, p.x_form = forms
         t = torch.from_numpy(rho).cuda()
         u = p.solve(t)
-        if name == "warp192":  # the batched driver and the checked (spectral-tail) variant
+        if batch > 1:  # enough CTAs to fill the chip: the launches of many tiles
+            outs = [torch.empty_like(t) for _ in range(batch)]
+            solve_batched([p] * batch, [t] * batch, outs)
+            assert all(torch.equal(u, o) for o in outs)
+        if name in ("warp192", "any90", "any40", "any40df", "mixed", "mixed_df"):  # batched driver, checked variant
             u2 = torch.empty_like(t)
             solve_batched([p, p], [t, t], [u2, torch.empty_like(t)])
             eta, u3 = ctypes.c_double(), torch.empty_like(t)
@@ -92,7 +123,9 @@ def test_debug_build_checks_pass_and_results_match(tmp_path):
         rho = np.ascontiguousarray(rho.astype(np.float32 if dtype == "f32" else np.float64))
         np.save(tmp_path / (name + "_rho.npy"), rho)
         with Plan(n, 6.0, 1e-6 if dtype == "f32" else 1e-12, dtype) as p:
-            if forms:
+            if isinstance(forms, str):
+                p.arith = forms
+            elif forms:
                 p.z_form, p.y_form, p.x_form = forms
             release[name] = p.solve(torch.from_numpy(rho).cuda()).cpu().numpy()
     env = dict(os.environ, POISSON_DEBUG="1", GSP_ROOT=ROOT, GSP_OUT=str(tmp_path), GSP_CASES=json.dumps(CASES))
