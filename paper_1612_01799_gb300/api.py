@@ -25,9 +25,10 @@ def _stream_handle(stream):
     if stream is not None:
         return stream.cuda_stream
     torch = _torch()
-    if not torch.cuda.is_initialized():
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # no Stream object made
+    if raw is None or not torch.cuda.is_initialized():
         return torch.cuda.current_stream().cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return raw(torch.cuda.current_device())
 
 
 def supported_n(N):
