@@ -280,11 +280,12 @@ static cudaError_t pick_form(int forms, int *field, Run &&run, cudaStream_t s, c
 
 // Choose p.arith (FP64 plans), p.zform, p.yform, p.xform and p.xyform: the cached decision
 // for this shape, else the fastest forms that exist, timed on p's zeroed workspace.  An FP64
-// plan first times its passes (block forms) in FP64 and in double-float arithmetic and keeps
-// the faster; timing needs no valid tables, so the caller builds the twiddles and the symbol
-// afterwards, in the chosen arithmetic's format.  The z pass writes only w3, the y passes w2
-// and w1, the x passes (timed with w2 as density and output) w1 and w2, the x-y passes all
-// three, and every solve writes each of them before reading it.  The x-y form is timed last,
+// plan first times a solve (block forms, or the plane kernels where its solves take them) in
+// FP64 and in double-float arithmetic and keeps the faster; timing needs no valid tables, so the
+// caller builds the twiddles and the symbol afterwards, in the chosen arithmetic's format.  The z
+// pass writes only w3, the y passes w2 and w1, the x passes (timed with w2 as density and
+// output) w1 and w2, a solve and the x-y passes all three, and every solve writes each of them
+// before reading it.  The x-y form is timed last,
 // against the separate passes in the y and x forms just chosen.
 static cudaError_t autotune(DevicePlan &p, int dev) {
     p.zform = 0;
@@ -311,9 +312,9 @@ static cudaError_t autotune(DevicePlan &p, int dev) {
     if (e == cudaSuccess) e = cudaEventCreate(&b);
     if (e == cudaSuccess && af != 1)
         e = pick_form(af, &p.arith, [&] {
-            cudaError_t r = launch_x_passes(p, s);
-            if (r == cudaSuccess) r = launch_y_passes(p, s);
-            return r == cudaSuccess ? launch_z_pass(p, s) : r;
+            PtrArray io{};  // a buffer that the solve's first kernel reads and its last one writes
+            io.p[0] = xy_in_one(p, 1) ? p.w1 : p.w2;
+            return launch_solve(p, io, io, 1, s, nullptr);
         }, s, a, b);
     if (e == cudaSuccess)
         e = pick_form(any ? 1 : z_forms(p.N, p.dtype, p.arith), &p.zform, [&] { return launch_z_pass(p, s); }, s, a,
