@@ -484,30 +484,10 @@ static cudaError_t upload_twiddles(poisson_plan p) {
         }
         return cudaSuccess;
     }
-    const int N = p->dp.N;
-    std::vector<double> tw;
-    gsp::twiddles(2 * N, tw);
-    const size_t n = (size_t)2 * N;
-    cudaError_t e;
-    if (p->dp.dtype == POISSON_F32) {
-        std::vector<float> twf(tw.begin(), tw.end());
-        e = cudaMemcpy(p->dp.tw, twf.data(), n * 2 * sizeof(float), cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) return e;
-        std::vector<float> tw4(n * 4);
-        for (size_t i = 0; i < n; ++i) {
-            tw4[4 * i] = tw4[4 * i + 1] = (float)tw[2 * i];
-            tw4[4 * i + 2] = tw4[4 * i + 3] = (float)tw[2 * i + 1];
-        }
-        return cudaMemcpy(p->dp.twc, tw4.data(), n * 4 * sizeof(float), cudaMemcpyHostToDevice);
-    }
-    if (!p->dp.arith) return cudaMemcpy(p->dp.tw, tw.data(), n * 2 * sizeof(double), cudaMemcpyHostToDevice);
-    std::vector<float> twd(n * 4);
-    for (size_t i = 0; i < 2 * n; ++i) {
-        const float hi = (float)tw[i];
-        twd[2 * i] = hi;
-        twd[2 * i + 1] = (float)(tw[i] - (double)hi);
-    }
-    return cudaMemcpy(p->dp.tw, twd.data(), n * 4 * sizeof(float), cudaMemcpyHostToDevice);
+    const int n2 = 2 * p->dp.N;
+    cudaError_t e = upload_table(p->dp.tw, n2, p->dp.dtype, p->dp.arith);
+    if (e != cudaSuccess || p->dp.dtype != POISSON_F32) return e;
+    return upload_table(p->dp.twc, n2, p->dp.dtype, 0, true);
 }
 
 static int plan_create_impl(poisson_plan *out, const int *n3, double L, const double *L3, double tol, int dtype,

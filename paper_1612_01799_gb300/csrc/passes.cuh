@@ -112,18 +112,6 @@ template <> struct Types<DF> {
     static constexpr int W = 1;
 };
 
-// Columns per CTA of a column pass: 128-byte row segments (16 FP32 or 8 FP64 complex),
-// halved until the block has <= 1024 threads and <= 128 KB of shared memory.
-template <typename Real, int L> __host__ __device__ constexpr int col_tc() {
-    const int W = Types<Real>::W;
-    int tc = sizeof(Real) == 4 ? 16 : 8;
-    const int P = L / Cfg<Real, L>::E;
-    while (tc > W && ((tc / W) * P > 1024 || tc * L * 2 * (int)sizeof(Real) > 131072)) tc /= 2;
-    return tc;
-}
-template <typename Real, int L> __host__ __device__ constexpr int col_threads() {
-    return (col_tc<Real, L>() / Types<Real>::W) * (L / Cfg<Real, L>::E);
-}
 // Rows per CTA of an x pass (shared tile (N+1) x (TR+1) complex).
 template <typename Real, int L> __host__ __device__ constexpr int row_tr() {
     int tr = sizeof(Real) == 4 ? 16 : 8;
@@ -271,82 +259,6 @@ k_x_forward(const PtrArray rho, Cx2<Real> *__restrict__ out, const Cx2<Real> *__
         const int r = e / (N + 1), k = e - r * (N + 1);
         st_ws(dst + (long long)r * Px + k, sm[k * SP + r]);
     }
-}
-
-// ---- K2 / K4: y transform over columns kx --------------------------------------------
-// FWD: rows < L/2 of the input are nonzero, all L outputs stored.
-// !FWD: all L inputs, outputs < L/2 stored.
-template <typename Real, int L, bool FWD>
-__global__ void __launch_bounds__(col_threads<Real, L>())
-k_col(const Cx2<Real> *__restrict__ in, Cx2<Real> *__restrict__ out,
-      const typename TwOf<typename Types<Real>::CC>::T *__restrict__ tw, int ncols, long long in_row,
-      long long in_outer, long long out_row, long long out_outer) {
-    using C = typename Types<Real>::CC;
-    constexpr int W = Types<Real>::W, E = Cfg<Real, L>::E, TC = col_tc<Real, L>(), NG = TC / W;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    C *sm = reinterpret_cast<C *>(smraw);  // L x NG
-    const int g = threadIdx.x % NG, q = threadIdx.x / NG;
-    const int col = blockIdx.x * TC + W * g;
-    const bool valid = col < ncols;
-    const Cx2<Real> *src = in + (long long)blockIdx.y * in_outer + col;
-    Cx2<Real> *dst = out + (long long)blockIdx.y * out_outer + col;
-    C v[E];
-    constexpr RunOpt opt{false, FWD, false, !FWD, false};
-    Stages<C, L, E, FWD ? -1 : 1, 1, typename Cfg<Real, L>::Rs>::template run<opt>(
-        v, q, g, sm, NG, tw, 1,
-        [&](int row) { return valid ? ld_cc(src + row * in_row) : czero<C>(); },
-        [&](int row, C x) {
-            if (valid) st_cc(dst + row * out_row, x);
-        });
-}
-
-// ---- K3: z forward, symbol, z inverse --------------------------------------------------
-template <typename Real, int L>
-__global__ void __launch_bounds__(col_threads<Real, L>())
-k_z_symbol(const Cx2<Real> *__restrict__ in, Cx2<Real> *__restrict__ out, const Real *__restrict__ sym,
-           const typename TwOf<typename Types<Real>::CC>::T *__restrict__ tw, int ncols, int Px,
-           int Ps) {
-    using C = typename Types<Real>::CC;
-    using Rs = typename Cfg<Real, L>::Rs;
-    constexpr int N = L / 2, W = Types<Real>::W, E = Cfg<Real, L>::E, TC = col_tc<Real, L>(), NG = TC / W;
-    constexpr int P = L / E;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    C *sm = reinterpret_cast<C *>(smraw);  // L x NG
-    const int g = threadIdx.x % NG, q = threadIdx.x / NG;
-    const int col = blockIdx.x * TC + W * g;
-    const bool valid = col < ncols;
-    // Consecutive blocks take ky and its mirror 2N - ky, which read the same symbol rows.
-    const int by = blockIdx.y;
-    const int ky = (by & 1) ? L - ((by + 1) >> 1) : (by >> 1);
-    const int kya = ky <= N ? ky : L - ky;
-    const long long zs = (long long)L * Px;  // z stride of w2 / w3
-    const Cx2<Real> *src = in + (long long)ky * Px + col;
-    Cx2<Real> *dst = out + (long long)ky * Px + col;
-    const long long plane = (long long)(N + 1) * Ps;
-    const Real *srow = sym + (long long)kya * Ps + (valid ? col : 0);
-    C v[E];
-    constexpr RunOpt fwd{false, true, true, false, false};
-    Stages<C, L, E, -1, 1, Rs>::template run<fwd>(
-        v, q, g, sm, NG, tw, 1, [&](int row) { return valid ? ld_cc(src + row * zs) : czero<C>(); },
-        [&](int, C) {});
-    // The forward's last stage (radix RL) left row j + r L/RL of butterfly b in v[b RL + r].
-    constexpr int RL = LastRadix<Rs>::v;
-#pragma unroll
-    for (int b = 0; b < E / RL; ++b) {
-        const int j = q + P * b;
-#pragma unroll
-        for (int r = 0; r < RL; ++r) {
-            const int row = j + r * (L / RL);
-            const int kz = row <= N ? row : L - row;
-            v[b * RL + r] = scale_sym(v[b * RL + r], srow + kz * plane);
-        }
-    }
-    constexpr RunOpt inv{true, false, false, true, false};
-    Stages<C, L, E, 1, 1, Reverse<Rs>>::template run<inv>(
-        v, q, g, sm, NG, tw, 1, [&](int) { return czero<C>(); },
-        [&](int row, C x) {
-            if (valid) st_cc(dst + row * zs, x);
-        });
 }
 
 // ---- K5: x inverse (Hermitian N+1 bins -> N real samples) -------------------------------

@@ -211,8 +211,8 @@ __device__ __forceinline__ float cenergy(CDF x) {
 }
 
 // With TAIL, the forward spectrum's energy in the outer shell max(|kx|,|ky|,|kz|) >= 7N/8
-// and its total energy are added (FP32 per thread, FP64 per tile) to tail[2 b], tail[2 b + 1]
-// for density b: the a-posteriori indicator of the density's resolution.
+// and its total energy are added (FP32 per thread, FP64 per tile) to the CTA's pair of density b
+// (tail_pair): the a-posteriori indicator of the density's resolution.
 template <typename Real, int L, bool TAIL>
 __global__ void __launch_bounds__(tma_threads<Real, L, 1>(), min_blocks_for<tma_threads<Real, L, 1>(), Cfg<Real, L>::E>())
 k_z_symbol_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tsym,
@@ -374,10 +374,13 @@ k_z_symbol_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ 
 // inputs x_n, n < N, are the nonzero half).  The kept inverse outputs split the same way:
 // u_z = A_z + conj(W_{2N}^z) B_z for z < N, with A and B the length-N inverse DFTs of the
 // even and odd halves of the spectrum.  Half h of the threads of a column group runs the
-// length-N transforms of parity h.  At N = 256, 320 and 384 the length-N schedule has one stage
-// fewer than the length-2N one, which saves a shared-memory exchange per direction, for the
-// price of reading the staged input twice and one half-size exchange that adds A and B (the
-// form also exists at N = 16 and 80).
+// length-N transforms of parity h.  Where the length-N schedule has one stage fewer than the
+// length-2N one (N = 256: 16, 16 and 16, 8, 4) this saves a shared-memory exchange per direction, for
+// the price of reading the staged input twice and one half-size exchange that adds A and B.  z pass,
+// direct and split form: N = 256 FP64 7255 and 7208 us, FP32 258 and 262; at the other sizes, kept
+// for callers that ask for the form by its knob, it loses (FP32 N = 16 5.6 and 11.7 us, 80 15.8
+// and 22.0, 320 737 and 1024, 384 1180 and 1822; FP64 N = 16 11.9 and 24.1, 80 217 and 231, 320 15.8 and
+// 16.6 ms, 384 24.7 and 26.2 ms).
 template <int L> __host__ __device__ constexpr bool zsplit_available() {
     return L == 32 || L == 160 || L == 512 || L == 640 || L == 768;
 }

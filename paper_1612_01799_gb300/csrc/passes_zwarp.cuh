@@ -295,7 +295,7 @@ template <int E1> __device__ __forceinline__ void zw_back(CV *v, const ZwLane &z
 
 // Tile t = (tx, ky, b): tx the 8-column block, consecutive tiles take ky and its mirror
 // 2N - ky (same symbol rows), b the density.  With TAIL the forward spectrum's shell and
-// total energies are added to tail[2 b], tail[2 b + 1] (as in k_z_symbol_tma).
+// total energies are added to the CTA's pair of density b (as in k_z_symbol_tma).
 template <int E1, bool TAIL>
 __global__ void __launch_bounds__(ZWarp<E1>::NT, ZWarp<E1>::MINB)
 k_z_warp(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tsym,
@@ -1150,7 +1150,7 @@ template <int D> __device__ __forceinline__ CF w32mul(CF x, int r) {
 
 // Tile t = (tx, ky, b): tx the 8-column block, consecutive tiles take ky and its mirror
 // 2N - ky (same symbol lines), b the density.  With TAIL the forward spectrum's shell and
-// total energies are added to tail[2 b], tail[2 b + 1] (as in k_z_warp).
+// total energies are added to the CTA's pair of density b (as in k_z_warp).
 //
 // Each step runs on packed pairs of the lane's 32 values (CV u[16]), two DFT lanes of one
 // column per packed instruction:

@@ -158,8 +158,7 @@ cudaError_t launch_solve(const DevicePlan &p, const PtrArray &rho, const PtrArra
 cudaError_t launch_xy_slab(const DevicePlan &p, const void *rho, void *u, int z0, int nz, cudaStream_t s, bool fwd);
 
 // Forms of the z pass that exist for (N, dtype, arith), as a bit mask over DevicePlan::zform:
-// bit 0 always; bit 1 where the length-N schedule has fewer stages than the length-2N one
-// (not in double-float arithmetic); bit 2 for FP32 at N = 64, 96, 128, 160, 192, 256 and 512.
+// bit 0 always; bit 1 at N = 16, 80, 256, 320 and 384 (not in double-float arithmetic); bit 2 for FP32 at N = 64, 96, 128, 160, 192, 256 and 512.
 int z_forms(int N, int dtype, int arith = 0);
 
 // Forms of the x passes that exist for (N, dtype), as a bit mask over DevicePlan::xform:
