@@ -246,8 +246,7 @@ int poisson_plan_info(poisson_plan p, double *delta, double *eps, int *n_terms, 
  *       G-tensor along the last axis):
  *       0 = length-2N transforms, a column pair spread over the threads of a block;
  *       1 = the pruned length-2N transforms split into even- and odd-frequency length-N
- *           transforms, where the length-N schedule has fewer stages
- *           (N = 16, 80, 256, 320, 384);
+ *           transforms (N = 16, 80, 256, 320, 384; not in double-float arithmetic);
  *       2 = one warp per column pair: an E1-point DFT (N = 16 E1) and a 16-point DFT in
  *           registers, a radix-2 step between lane pairs and one warp-local
  *           shared-memory exchange per direction (POISSON_F32, N = 64, 96, 128, 160,

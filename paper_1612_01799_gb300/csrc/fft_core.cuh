@@ -117,15 +117,21 @@ __device__ __forceinline__ DF df_sum_prod(DF a, DF b, DF c, DF d) {
     return DF(s, t);  // left unnormalised, as a sum's result
 }
 
-struct CDF {
+// A complex double-float.  PACK: its complex sums take both parts in packed instructions, else part by
+// part (cadd below; the bits are the same).
+template <bool PACK> struct CDFx {
     DF re, im;
+    template <bool P> __host__ __device__ operator CDFx<P>() const { return {re, im}; }
 };
+using CDF = CDFx<true>;
+template <typename C> constexpr bool is_cdf = false;
+template <bool P> constexpr bool is_cdf<CDFx<P>> = true;
 
 template <typename C> struct CxReal;
 template <> struct CxReal<CF> { using T = float; };
 template <> struct CxReal<CD> { using T = double; };
 template <> struct CxReal<CV> { using T = float; };
-template <> struct CxReal<CDF> { using T = DF; };
+template <bool P> struct CxReal<CDFx<P>> { using T = DF; };
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float2 f2add(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -139,7 +145,8 @@ template <typename C> __device__ __forceinline__ C czero();
 template <> __device__ __forceinline__ CF czero<CF>() { return {0.f, 0.f}; }
 template <> __device__ __forceinline__ CD czero<CD>() { return {0.0, 0.0}; }
 template <> __device__ __forceinline__ CV czero<CV>() { return {f2(0.f, 0.f), f2(0.f, 0.f)}; }
-template <> __device__ __forceinline__ CDF czero<CDF>() { return {DF(0.f, 0.f), DF(0.f, 0.f)}; }
+template <> __device__ __forceinline__ CDFx<true> czero<CDFx<true>>() { return {DF(0.f, 0.f), DF(0.f, 0.f)}; }
+template <> __device__ __forceinline__ CDFx<false> czero<CDFx<false>>() { return {DF(0.f, 0.f), DF(0.f, 0.f)}; }
 
 __device__ __forceinline__ CF cadd(CF a, CF b) { return {a.re + b.re, a.im + b.im}; }
 __device__ __forceinline__ CF csub(CF a, CF b) { return {a.re - b.re, a.im - b.im}; }
@@ -147,36 +154,36 @@ __device__ __forceinline__ CD cadd(CD a, CD b) { return {a.re + b.re, a.im + b.i
 __device__ __forceinline__ CD csub(CD a, CD b) { return {a.re - b.re, a.im - b.im}; }
 __device__ __forceinline__ CV cadd(CV a, CV b) { return {f2add(a.re, b.re), f2add(a.im, b.im)}; }
 __device__ __forceinline__ CV csub(CV a, CV b) { return {f2sub(a.re, b.re), f2sub(a.im, b.im)}; }
-// The two double-float sums of a complex sum: plainly, part by part, in the translation units that
-// define GSP_DF_PLAIN_SUMS, else in one: the real and the imaginary part take the
+// The two double-float sums of a complex sum: plainly, part by part, or (PACK) in one: the real and
+// the imaginary part take the
 // steps of DF's operator+ (the same roundings, the same result) side by side in packed FP32x2
 // instructions, five and six selects and compares in place of ten and six.  The FMA pipe takes
 // a packed instruction in two cycles, so what this saves is issue slots and code size: the
 // compiled-length z pass at N = 128 went from 141 to 136 us, the runtime-length one at
-// N = 162, whose stages compete for the instruction cache, from 480 to 428 us.  Where the code
-// fits the cache the register pairs it ties together cost more than that: FP64 plans' solves,
-// packed and plain, N = 160 654 and 649 us, 192 957 and 951, 256 2000 and 1991, 384 8086 and
-// 7727, 512 19.48 and 18.47 ms, 1024 201.1 and 196.6 ms; but N = 96 128 and 135 us, N = 128 249.0
-// and 250.6, and N = 320, whose length 640 holds 20 values a thread, 6.97 and 7.98 ms.
-#ifdef GSP_DF_PLAIN_SUMS
-__device__ __forceinline__ CDF cadd(CDF a, CDF b) { return {a.re + b.re, a.im + b.im}; }
-#else
-__device__ __forceinline__ CDF cadd(CDF a, CDF b) {
-    const bool p = fabsf(b.re.hi) > fabsf(a.re.hi), q = fabsf(b.im.hi) > fabsf(a.im.hi);
-    const float2 x = f2(p ? b.re.hi : a.re.hi, q ? b.im.hi : a.im.hi);
-    const float2 y = f2(p ? a.re.hi : b.re.hi, q ? a.im.hi : b.im.hi);
-    const float2 s = f2add(x, y), e = f2sub(y, f2sub(s, x));
-    const float2 l = f2add(e, f2add(f2(a.re.lo, a.im.lo), f2(b.re.lo, b.im.lo)));
-    return {DF(s.x, l.x), DF(s.y, l.y)};
+// N = 162, whose stages compete for the instruction cache, from 480 to 428 us.  Elsewhere the
+// register pairs it ties together cost more than that: no size or stage count tells the two apart
+// beforehand, so the lengths that take plain sums (df_plain_sums) are those measured faster with them.
+template <bool P> __device__ __forceinline__ CDFx<P> cadd(CDFx<P> a, CDFx<P> b) {
+    if constexpr (P) {
+        const bool p = fabsf(b.re.hi) > fabsf(a.re.hi), q = fabsf(b.im.hi) > fabsf(a.im.hi);
+        const float2 x = f2(p ? b.re.hi : a.re.hi, q ? b.im.hi : a.im.hi);
+        const float2 y = f2(p ? a.re.hi : b.re.hi, q ? a.im.hi : b.im.hi);
+        const float2 s = f2add(x, y), e = f2sub(y, f2sub(s, x));
+        const float2 l = f2add(e, f2add(f2(a.re.lo, a.im.lo), f2(b.re.lo, b.im.lo)));
+        return {DF(s.x, l.x), DF(s.y, l.y)};
+    } else {
+        return {a.re + b.re, a.im + b.im};
+    }
 }
-#endif
-__device__ __forceinline__ CDF csub(CDF a, CDF b) { return cadd(a, CDF{-b.re, -b.im}); }
+template <bool P> __device__ __forceinline__ CDFx<P> csub(CDFx<P> a, CDFx<P> b) {
+    return cadd(a, CDFx<P>{-b.re, -b.im});
+}
 
 __device__ __forceinline__ CF cscale(CF a, float s) { return {a.re * s, a.im * s}; }
 __device__ __forceinline__ CD cscale(CD a, double s) { return {a.re * s, a.im * s}; }
 __device__ __forceinline__ CV cscale(CV a, float s) { return {f2mul(a.re, f2(s, s)), f2mul(a.im, f2(s, s))}; }
 // Both parts of a complex double-float times a real, the steps of DF's operator* packed.
-__device__ __forceinline__ CDF cscale(CDF a, DF s) {
+template <bool P> __device__ __forceinline__ CDFx<P> cscale(CDFx<P> a, DF s) {
     const float2 x = f2(a.re.hi, a.im.hi), H = f2(s.hi, s.hi), p = f2mul(x, H);
     float2 e = f2fma(x, H, f2neg(p));
     e = f2fma(x, f2(s.lo, s.lo), e);
@@ -194,11 +201,11 @@ __device__ __forceinline__ CD cfma(CD a, CD x, double s) { return {fma(x.re, s, 
 __device__ __forceinline__ CV cfma(CV a, CV x, float s) {
     return {f2fma(x.re, f2(s, s), a.re), f2fma(x.im, f2(s, s), a.im)};
 }
-__device__ __forceinline__ CDF cfma(CDF a, CDF x, DF s) { return {a.re + x.re * s, a.im + x.im * s}; }
+template <bool P> __device__ __forceinline__ CDFx<P> cfma(CDFx<P> a, CDFx<P> x, DF s) { return {a.re + x.re * s, a.im + x.im * s}; }
 template <typename C, typename R> __device__ __forceinline__ C cdot2(C x, R sx, C y, R sy) {
     return cfma(cscale(x, sx), y, sy);
 }
-__device__ __forceinline__ CDF cdot2(CDF x, DF sx, CDF y, DF sy) {  // df_sum_prod's steps, packed
+template <bool P> __device__ __forceinline__ CDFx<P> cdot2(CDFx<P> x, DF sx, CDFx<P> y, DF sy) {  // df_sum_prod's steps, packed
     const float2 a = f2(x.re.hi, x.im.hi), c = f2(y.re.hi, y.im.hi), A = f2(sx.hi, sx.hi), B = f2(sy.hi, sy.hi);
     const float2 p1 = f2mul(a, A), p2 = f2mul(c, B);
     const float2 e1 = f2fma(a, A, f2neg(p1)), e2 = f2fma(c, B, f2neg(p2));
@@ -216,7 +223,7 @@ __device__ __forceinline__ CDF cdot2(CDF x, DF sx, CDF y, DF sy) {  // df_sum_pr
 template <typename C> __device__ __forceinline__ C csub_half(C a, C x) {
     return cfma(a, x, (typename CxReal<C>::T)-0.5);
 }
-__device__ __forceinline__ CDF csub_half(CDF a, CDF x) {
+template <bool P> __device__ __forceinline__ CDFx<P> csub_half(CDFx<P> a, CDFx<P> x) {
     return {a.re + DF(-0.5f * x.re.hi, -0.5f * x.re.lo), a.im + DF(-0.5f * x.im.hi, -0.5f * x.im.lo)};
 }
 
@@ -230,8 +237,8 @@ template <int D> __device__ __forceinline__ CD add_rot(CD a, CD b) {
 template <int D> __device__ __forceinline__ CV add_rot(CV a, CV b) {
     return D > 0 ? CV{f2sub(a.re, b.im), f2add(a.im, b.re)} : CV{f2add(a.re, b.im), f2sub(a.im, b.re)};
 }
-template <int D> __device__ __forceinline__ CDF add_rot(CDF a, CDF b) {
-    return D > 0 ? cadd(a, CDF{-b.im, b.re}) : cadd(a, CDF{b.im, -b.re});
+template <int D, bool P> __device__ __forceinline__ CDFx<P> add_rot(CDFx<P> a, CDFx<P> b) {
+    return D > 0 ? cadd(a, CDFx<P>{-b.im, b.re}) : cadd(a, CDFx<P>{b.im, -b.re});
 }
 // a - i D b
 template <int D, typename C> __device__ __forceinline__ C sub_rot(C a, C b) { return add_rot<-D>(a, b); }
@@ -247,8 +254,8 @@ template <int D, typename C, typename R> __device__ __forceinline__ void rot_pai
     a = {cfma(C{m.re, m.im}, C{d.im, d.re}, -p).re, cfma(C{m.re, m.im}, C{d.im, d.re}, p).im};
     b = {cfma(C{m.re, m.im}, C{d.im, d.re}, p).re, cfma(C{m.re, m.im}, C{d.im, d.re}, -p).im};
 }
-template <int D> __device__ __forceinline__ void rot_pair(CDF m, CDF d, DF h, CDF &a, CDF &b) {
-    const CDF t = cscale(d, h);
+template <int D, bool P> __device__ __forceinline__ void rot_pair(CDFx<P> m, CDFx<P> d, DF h, CDFx<P> &a, CDFx<P> &b) {
+    const CDFx<P> t = cscale(d, h);
     a = add_rot<D>(m, t);
     b = sub_rot<D>(m, t);
 }
@@ -263,7 +270,7 @@ template <int D> __device__ __forceinline__ CD cmulk(CD a, double cr, double ci)
     const double s = D < 0 ? ci : -ci;
     return {a.re * cr - a.im * s, a.re * s + a.im * cr};
 }
-template <int D> __device__ __forceinline__ CDF cmulk(CDF a, DF cr, DF ci) {
+template <int D, bool P> __device__ __forceinline__ CDFx<P> cmulk(CDFx<P> a, DF cr, DF ci) {
     const DF s = D < 0 ? ci : -ci;
     return {df_sum_prod(a.re, cr, a.im, -s), df_sum_prod(a.re, s, a.im, cr)};
 }
@@ -279,9 +286,9 @@ template <int D> __device__ __forceinline__ CV cmulk(CV a, float cr, float ci) {
 template <int D, int M, typename C, typename R> __device__ __forceinline__ C cmul_w8(C a, R h) {
     return cmulk<D>(a, M == 1 ? h : -h, -h);
 }
-template <int D, int M> __device__ __forceinline__ CDF cmul_w8(CDF a, DF h) {
+template <int D, int M, bool P> __device__ __forceinline__ CDFx<P> cmul_w8(CDFx<P> a, DF h) {
     // m = 1: h (re - D im, im + D re); m = 3: that times i D: h (-re - D im, D re - im)
-    return cscale(M == 1 ? add_rot<D>(a, a) : add_rot<D>(CDF{-a.re, -a.im}, a), h);
+    return cscale(M == 1 ? add_rot<D>(a, a) : add_rot<D>(CDFx<P>{-a.re, -a.im}, a), h);
 }
 
 // Twiddle tables hold exp(-2 pi i e / TL): float2 / double2 (re, im) for CF / CD, and the
@@ -290,7 +297,7 @@ template <typename C> struct TwOf;
 template <> struct TwOf<CF> { using T = float2; };
 template <> struct TwOf<CD> { using T = double2; };
 template <> struct TwOf<CV> { using T = float4; };
-template <> struct TwOf<CDF> { using T = float4; };  // (re.hi, re.lo, im.hi, im.lo)
+template <bool P> struct TwOf<CDFx<P>> { using T = float4; };  // (re.hi, re.lo, im.hi, im.lo)
 
 // a times w (D < 0) or conj(w) (D > 0).
 template <int D> __device__ __forceinline__ CF twmul(CF a, float2 w) {
@@ -301,7 +308,7 @@ template <int D> __device__ __forceinline__ CD twmul(CD a, double2 w) {
     const double s = D < 0 ? w.y : -w.y;
     return {a.re * w.x - a.im * s, a.re * s + a.im * w.x};
 }
-template <int D> __device__ __forceinline__ CDF twmul(CDF a, float4 w) {
+template <int D, bool P> __device__ __forceinline__ CDFx<P> twmul(CDFx<P> a, float4 w) {
     const DF wr(w.x, w.y), wi(w.z, w.w);
     const DF s = D < 0 ? wi : -wi;
     return {df_sum_prod(a.re, wr, a.im, -s), df_sum_prod(a.re, s, a.im, wr)};
@@ -345,7 +352,7 @@ template <int D, typename C> __device__ __forceinline__ void dft5(C &a0, C &a1, 
     const R s2 = (R)0.58778525229247312917;   // sin(4 pi / 5)
     C b1 = cadd(a1, a4), b2 = cadd(a2, a3), d1 = csub(a1, a4), d2 = csub(a2, a3);
     C p1, p2, t = cadd(b1, b2);
-    if constexpr (std::is_same<C, CDF>::value) {
+    if constexpr (is_cdf<C>) {
         // c1 and c2 are -1/4 +- sqrt(5)/4: one product in place of four
         const C m = cadd(a0, C{R(-0.25f * t.re.hi, -0.25f * t.re.lo), R(-0.25f * t.im.hi, -0.25f * t.im.lo)});
         const C k = cscale(csub(b1, b2), (R)0.55901699437494742410);

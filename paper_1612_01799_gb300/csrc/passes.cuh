@@ -112,6 +112,18 @@ template <> struct Types<DF> {
     static constexpr int W = 1;
 };
 
+// The complex types of a block-form kernel for N points on its axis: those of Types, in
+// double-float with plain sums where these are faster.  FP64 plans' solves, packed and plain sums:
+// N = 160 654 and 649 us, 192 957 and 951, 256 2000 and 1991, 384 8086 and 7727, 512 19.48 and
+// 18.47 ms, 1024 201.1 and 196.6 ms; but N = 96 128 and 135 us, N = 128 249.0 and 250.6, and N = 320,
+// whose length 640 holds 20 values a thread, 6.97 and 7.98 ms.
+constexpr bool df_plain_sums(int N) { return (N >= 160 && N <= 256) || N >= 384; }
+template <typename Real, int N> struct CxOf : Types<Real> {};
+template <int N> struct CxOf<DF, N> {
+    using CS = CDFx<!df_plain_sums(N)>;
+    using CC = CS;
+};
+
 // Rows per CTA of an x pass (shared tile (N+1) x (TR+1) complex).
 template <typename Real, int L> __host__ __device__ constexpr int row_tr() {
     int tr = sizeof(Real) == 4 ? 16 : 8;
@@ -204,7 +216,7 @@ template <typename Real, int N>
 __global__ void __launch_bounds__(row_tr<Real, N>() * (N / Cfg<Real, N>::E))
 k_x_forward(const PtrArray rho, Cx2<Real> *__restrict__ out, const Cx2<Real> *__restrict__ tw, int rows_b,
             int nrows, int Px) {
-    using C = typename Types<Real>::CS;
+    using C = typename CxOf<Real, N>::CS;
     using T2 = Cx2<Real>;
     using X2 = Ext2<Real>;
     constexpr int E = Cfg<Real, N>::E, P = N / E, TR = row_tr<Real, N>(), SP = TR + 1, NT = TR * P;
@@ -266,7 +278,7 @@ template <typename Real, int N>
 __global__ void __launch_bounds__(row_tr<Real, N>() * (N / Cfg<Real, N>::E))
 k_x_inverse(const Cx2<Real> *__restrict__ in, const PtrArray u, const Cx2<Real> *__restrict__ tw, int rows_b,
             int nrows, int Px) {
-    using C = typename Types<Real>::CS;
+    using C = typename CxOf<Real, N>::CS;
     using T2 = Cx2<Real>;
     using X2 = Ext2<Real>;
     constexpr int E = Cfg<Real, N>::E, P = N / E, TR = row_tr<Real, N>(), SP = TR + 1, NT = TR * P;

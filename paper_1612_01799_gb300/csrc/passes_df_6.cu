@@ -1,5 +1,4 @@
 // Double-float passes for the sizes of group 6 (see passes.cuh).
-#define GSP_DF_PLAIN_SUMS  // measured beside cadd in fft_core.cuh
 #include "passes.cuh"
 
 namespace gsp {

@@ -112,6 +112,9 @@ template <> __device__ __forceinline__ CDF ld_sm_cc<CDF>(const unsigned char *p)
     const float4 f = sm_ld(reinterpret_cast<const float4 *>(p));
     return {DF(f.x, f.y), DF(f.z, f.w)};
 }
+template <> __device__ __forceinline__ CDFx<false> ld_sm_cc<CDFx<false>>(const unsigned char *p) {
+    return ld_sm_cc<CDF>(p);
+}
 __device__ __forceinline__ CV scale_sym_sm(CV x, const float *s) {
     return cscale2(x, sm_ld(reinterpret_cast<const float2 *>(s)));
 }
@@ -139,7 +142,7 @@ __global__ void __launch_bounds__(tma_threads<Real, L, KIND>(), min_blocks_for<t
 k_col_tma(const __grid_constant__ CUtensorMap tin, Cx2<Real> *__restrict__ out,
           const typename TwOf<typename Types<Real>::CC>::T *__restrict__ tw, int ntx, int ntiles,
           int ncols, long long out_row, long long out_outer, int *__restrict__ status, int z0) {
-    using C = typename Types<Real>::CC;
+    using C = typename CxOf<Real, L / 2>::CC;
     using Lay = TmaLayout<Real, L, KIND>;
     using Rs = typename Cfg<Real, L>::Rs;
     constexpr bool FWD = KIND == 0;
@@ -219,7 +222,7 @@ k_z_symbol_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ 
                Cx2<Real> *__restrict__ out,
                const typename TwOf<typename Types<Real>::CC>::T *__restrict__ tw, int ntx, int ntiles,
                int nx, int ny, int Px, int *__restrict__ status, double *__restrict__ tail) {
-    using C = typename Types<Real>::CC;
+    using C = typename CxOf<Real, L / 2>::CC;
     using Lay = TmaLayout<Real, L, 1>;
     using Rs = typename Cfg<Real, L>::Rs;
     using Rv = Reverse<Rs>;
