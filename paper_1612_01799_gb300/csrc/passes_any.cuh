@@ -81,9 +81,7 @@ template <int D> __device__ __forceinline__ CD any_twmul(CD a, double2 w) { retu
 template <int D> __device__ __forceinline__ CDF any_twmul(CDF a, float4 w) {
     // Renormalised: the stages of larger radix collect more in lo (rel-L2 error of a solve at
     // N = 100 and 162 over eight densities: 8.2e-15 and 8.2e-15 without, 6.0e-15 and 7.4e-15 with).
-    const CDF p = twmul<D>(a, w);
-    const float2 h = f2(p.re.hi, p.im.hi), l = f2(p.re.lo, p.im.lo), s = f2add(h, l), e = f2sub(l, f2sub(s, h));
-    return {DF(s.x, e.x), DF(s.y, e.y)};
+    return cnorm(twmul<D>(a, w));
 }
 
 // One row pair's worth of consecutive real sample pairs (x_2m, x_2m+1) as a group and back:

@@ -146,3 +146,22 @@ def test_checked_solve_tail(torch_cuda):
     ref = selection.spectral_tail(rho)
     assert abs(eta.value - ref) <= 1e-3 * ref + 1e-12
     assert rel_l2(u.cpu().numpy(), osolver.solve(rho, L, 1e-12)) <= TOL
+
+
+@pytest.mark.parametrize("N,bound", [(80, 7.3e-15), (160, 7.55e-15)])
+def test_error_of_lengths_with_a_factor_5(torch_cuda, N, bound):
+    """Mean difference of double-float and FP64 arithmetic over eight densities: 7.0e-15 and
+    7.3e-15 (7.6e-15 and 7.8e-15 where the radix-5 sums' lo parts reach the last stage as they
+    are; the difference of two densities is 1e-15, the bits do not vary from run to run)."""
+    from paper_1612_01799_gb300 import Plan
+    torch = torch_cuda
+    errors = []
+    with Plan(N, 10.0, 1e-12, "f64") as p:
+        for seed in range(8):
+            rho = torch.from_numpy(D.config_aniso4(N=N, seed=seed).gaussians.sample(N, 10.0)).cuda()
+            p.arith = "df"
+            u = p.solve(rho)
+            p.arith = "f64"
+            w = p.solve(rho)
+            errors.append(float((u - w).norm() / w.norm()))
+    assert np.mean(errors) <= bound, errors
