@@ -190,12 +190,13 @@ constexpr int kPlaneThreads = 384;
 // Largest plane: in FP32 two CTAs fit an SM (solves, separate passes against the plane kernels:
 // 20^3 21.4 and 18.9 us, 60^3 27.2 and 25.5, 64 x 64 x 256 66 and 57, but 72^3 28.6 and 30.2); the
 // wider arithmetics are bound by the longer chain of one CTA soon (double-float 10^3 24.3 and
-// 20.8 us, 18^3 27.4 and 27.4, 20^3 25.9 and 28.5, 30^3 32.0 and 36.6).  In FP64 planes
-// up to kPlaneMany are worth a CTA each where they fill the SMs, no wave of them below nine tenths
-// (many; 24 x 24 x 600 413 and 395 us, but 20 x 20 x 240 112 and 122).  Cubes whose passes are compiled for
+// 20.8 us, 18^3 27.4 and 27.4, 20^3 25.9 and 28.5, 30^3 32.0 and 36.6).  Larger planes, up
+// to plane_many, are worth a CTA each where they fill the SMs, no wave of them below nine tenths
+// (many; FP64 24 x 24 x 600 413 and 395 us, but 20 x 20 x 240 112 and 122; double-float 20 x 20 x 300 45.8
+// and 43.3, but 20 x 20 x 400 53.8 and 62.4 and 24 x 24 x 300 56.6 and 61.5).  Cubes whose passes are compiled for
 // their length have kernels of their own (plane_n_size).
 constexpr int plane_smem(bool f32) { return f32 ? 106 * 1024 : 18 * 1024; }
-constexpr int kPlaneMany = 48 * 1024;
+constexpr int plane_many(bool fp64) { return fp64 ? 48 * 1024 : 20 * 1024; }
 // fp64: FP64 arithmetic.
 inline PlaneTile plane_tile(int nx, int ny, int max_radix, int w, bool fp64) {
     PlaneTile t{};
@@ -220,7 +221,7 @@ inline PlaneTile plane_tile(int nx, int ny, int max_radix, int w, bool fp64) {
         }
     }
     t.on = t.sx.nst && t.sy.nst && t.smem <= plane_smem(w == 2);
-    t.many = fp64 && t.sx.nst && t.sy.nst && t.smem <= kPlaneMany;
+    t.many = w == 1 && t.sx.nst && t.sy.nst && t.smem <= plane_many(fp64);
     return t;
 }
 // Whether a launch of `planes` planes runs the plane kernels.

@@ -796,11 +796,13 @@ extern "C" int poisson_solve(poisson_plan p, const void *rho_d, void *u_d, void 
 
 // Slabs of the host-buffer solve's copy / x-pass pipeline, in eighths of the volume.  FP32, whose
 // x and y passes take a third of a slab's copy: few copies, graded so that little work follows
-// the last one in and precedes the first one out (N = 256 946 -> 929 us against equal slabs).  The
-// wider arithmetics, whose passes take as long as the copies: equal slabs (N = 160 906 us,
-// graded 925).  Below kHostPipelineBytes the launches cost more than the overlap gains: one
-// copy each way (FP32 N = 64 54 us against 135, N = 128 172 against 182 graded; N = 160, 16 MB, 325
-// against 300).
+// the last one in and precedes the first one out (pinned buffers, graded and equal slabs: N = 256 930
+// and 946 us, N = 160 296 and 312; pageable N = 256 1173 and 1311).  The wider arithmetics, whose
+// passes take as long as the copies: equal slabs (double-float N = 160 907 us graded and 889 equal, N = 192
+// 1339 and 1245).  Below kHostPipelineBytes the launches cost more than the overlap gains: one
+// copy each way (FP32 N = 64 54 us against 135, N = 128 171 against 180 graded; N = 160, 16 MB, 325
+// against 300; double-float against equal slabs N = 64 88 and 202 us, N = 96, 7 MB, 220 and 332, and
+// above it N = 128, 17 MB, 440 and 435, N = 160 994 and 889).
 constexpr size_t kHostPipelineBytes = (size_t)12 << 20;
 struct HostSlabs {
     int n, in[8], out[8];

@@ -1114,7 +1114,9 @@ cudaError_t any_z(const DevicePlan &p, int B, cudaStream_t s, double *tail, int 
 
 // The passes of a runtime-length plan: along an axis whose count has a compiled schedule
 // (p.axn) the block forms, else the runtime-length forms: a pass touches one axis only, and the
-// layouts agree.  (FP32 box 64 x 128 x 192: 102.5 us with the runtime-length forms, 67.3 with these.)
+// layouts agree.  (FP32 box 64 x 128 x 192: 102.5 us with the runtime-length forms, 67.3 with these.
+// The rounding error of a box in FP32 is then that of the cubes: 1.15e-7 here against 1.09e-7, 1.22e-7
+// against 1.07e-7 at 128 x 128 x 64; double-float 4% less.)
 template <typename Real>
 cudaError_t box_x(const DevicePlan &p, const PtrArray &rho, const PtrArray &u, int B, cudaStream_t s, bool fwd,
                   int rows = 0, void *w1 = nullptr) {

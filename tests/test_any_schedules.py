@@ -125,7 +125,8 @@ def test_tiles_of_two_for_long_wide_columns(shim, n, f32, lg):
 
 
 @pytest.mark.parametrize("n,df,planes,on", [(18, 0, 1, 1), (30, 0, 152, 1), (30, 0, 160, 0), (30, 0, 304, 1),
-                                                (36, 0, 304, 0), (30, 1, 304, 0)])
+                                                (36, 0, 304, 0), (20, 1, 304, 1), (20, 1, 320, 0), (24, 1, 304, 0)])
 def test_plane_kernels_of_many_planes(shim, n, df, planes, on):
-    """FP64 arithmetic: planes up to 48 KB where their CTAs fill the SMs; not in double-float."""
+    """Wider arithmetics: planes up to 48 KB (FP64) and 20 KB (double-float) where their CTAs fill the
+    SMs."""
     assert plane(shim, n, n, df, 0, planes)[0] == on

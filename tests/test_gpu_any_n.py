@@ -272,7 +272,7 @@ def test_few_tiles(torch_cuda, n):
             assert rel_l2(run(torch_cuda, p, rho), uo) <= TOL["f64"], ar
 
 
-@pytest.mark.parametrize("N,count", [(30, 12), (20, 16)])
+@pytest.mark.parametrize("N,count", [(30, 12), (20, 15), (20, 16)])
 def test_batch_of_another_route_gives_the_same_bits(torch_cuda, N, count):
     """A batch fills the SMs where one density does not, and takes other launches (threads, x stages
     combined or apart, in FP64 the plane kernels): the bits of the single solves."""
