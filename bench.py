@@ -45,8 +45,8 @@ KERNEL_NAMES = ["k_x_forward", "k_col<fwd>", "k_z_symbol", "k_col<inv>", "k_x_in
 # DRAM bytes per launch of the dominant kernel from one ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum), keyed by the hash of the kernel sources it was taken on; a
 # source change makes the figure stale and it is reported as null.
-NCU_TRAFFIC = {("3080996c4f1255ff", "k_z_warp", 256): 358018816 + 237190656,
-               ("3080996c4f1255ff", "k_z_w512", 512): 3144715264 + 2140066304}
+NCU_TRAFFIC = {("4cc36ad94c67403a", "k_z_warp", 256): 357841408 + 236752128,
+               ("4cc36ad94c67403a", "k_z_w512", 512): 3152322816 + 2140549376}
 
 
 def kernel_source_hash():

@@ -227,7 +227,7 @@ k_x_forward(const PtrArray rho, Cx2<Real> *__restrict__ out, const Cx2<Real> *__
     const int t = threadIdx.x;
     const long long r0 = (long long)blockIdx.x * TR;
     const int nr = (int)min((long long)TR, (long long)nrows - r0);
-    const int b = (int)(r0 / rows_b);
+    const int b = rows_b == N * N ? (int)(r0 / (N * N)) : 0;  // a box has one density
     // The tile is nr consecutive rows of N reals: contiguous N/2-pair chunks.
     const X2 *src = reinterpret_cast<const X2 *>(rho.p[b]) + (r0 - (long long)b * rows_b) * (N / 2);
     for (int e = t; e < nr * (N / 2); e += NT) {
@@ -331,7 +331,7 @@ k_x_inverse(const Cx2<Real> *__restrict__ in, const PtrArray u, const Cx2<Real> 
         v, q, c, sm, SP, tw, 2, [&](int row) { return sm[row * SP + c]; },
         [&](int row, C x) { sm[row * SP + c] = x; });
     __syncthreads();
-    const int b = (int)(r0 / rows_b);
+    const int b = rows_b == N * N ? (int)(r0 / (N * N)) : 0;  // a box has one density
     X2 *dst = reinterpret_cast<X2 *>(const_cast<void *>(u.p[b])) + (r0 - (long long)b * rows_b) * (N / 2);
     for (int e = t; e < nr * (N / 2); e += NT) {
         const int r = e / (N / 2), m = e - r * (N / 2);

@@ -40,7 +40,7 @@ struct AnyRows {
     long long first;  // row of r0 within density b0
     long long left;   // rows of density b0 from r0 on
     __device__ AnyRows(long long r0, int rows_b) {
-        b0 = (int)(r0 / rows_b);
+        b0 = (int)((unsigned)r0 / (unsigned)rows_b);  // r0 lies below the number of rows, an int
         first = r0 - (long long)b0 * rows_b;
         left = rows_b - first;
     }
